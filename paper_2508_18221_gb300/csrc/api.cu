@@ -59,7 +59,7 @@ struct grmhd_ctx {
     double* scratch;         // nv * P
     double* divB;            // d_i (sqrt(gamma) B^i) (GLM only)
     double* ham;             // Hamiltonian constraint per node (diagnostics)
-    double* met;             // 9 * P: the metric of the last k_prep (e^{4phi}, e^{-4phi}, sqrt(gamma), gammatilde^ij)
+    double* met;             // N_MET * P: the metric of the last k_prep
     double* ham_out;         // non-null while a diagnostic stage is enqueued: k_rhs writes H there
     int nv;                  // evolved variables: GRMHD_NV, + 1 (psi) with GLM
     double* Dr;              // Nr x Nr reference CGL matrix on [-1, 1]
@@ -472,7 +472,7 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
     AL(c->d2, N_D2 * 6 * P);
     AL(c->divF, 8 * P);
     AL(c->ham, P);
-    AL(c->met, 9 * P);
+    AL(c->met, N_MET * P);
     AL(c->scratch, nv * P);
     AL(c->Dr, Nr * Nr); AL(c->Dt, Nt * Nt); AL(c->Dp, Np);
     AL(c->Fr, Nr * Nr); AL(c->Ft, Nt * Nt); AL(c->Fp, Np);

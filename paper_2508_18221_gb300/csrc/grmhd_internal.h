@@ -22,7 +22,10 @@ enum {
     N_D2 = 11,
     N_PRIM = 7,     // rho, v^r, v^th, v^ph, eps, p, W
     N_FLUX = 24,    // sqrt(gamma) scriptF^i_v  [dir][var]
-    N_TMN = 10,     // T^{00},T^{01},T^{02},T^{03},T^{11},T^{12},T^{13},T^{22},T^{23},T^{33}
+    // matter terms.  FP64: sqrt(gamma) times E, S_i, E + S, S^ij, Z v_i v_j - b_i b_j (17);
+    // mixed modes: T^{00},T^{01},T^{02},T^{03},T^{11},T^{12},T^{13},T^{22},T^{23},T^{33} (10)
+    N_TMN = 17,
+    N_MET = 10,     // e^{4phi}, e^{-4phi}, sqrt(gamma), gammatilde^ij (6), 1/sqrt(gamma) (FP64)
 };
 
 // d1 field f (0..20) direction d: index (f*3 + d); d2 field slot s (0..10) pair q:
@@ -84,8 +87,9 @@ struct FoldJob {
 cudaError_t kernels_init();
 cudaError_t eo_init();
 cudaError_t tc_init();
-// met: 9 P doubles written per node (e^{4phi}, e^{-4phi}, sqrt(gamma), gammatilde^ij in the
-// packed order rr r-theta r-phi theta-theta theta-phi phi-phi), read by launch_rhs
+// met: N_MET doubles written per node (e^{4phi}, e^{-4phi}, sqrt(gamma), gammatilde^ij in the
+// packed order rr r-theta r-phi theta-theta theta-phi phi-phi; 1/sqrt(gamma) in FP64), read
+// by launch_rhs
 cudaError_t launch_prep(const Dims& d, const PhysParams& pp, const double* U, double* prim,
                         double* flux, double* tmn, double* lam, unsigned long long* nfail, double* met,
                         cudaStream_t s, int fp32_algebra = 0);

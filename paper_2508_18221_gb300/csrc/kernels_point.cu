@@ -290,6 +290,79 @@ __device__ int con2prim_damped_point(double D, const double S_d[3], double tau, 
 }
 
 // --------------------------------------------------------------------------- k_prep
+// Densitized fluxes and matter terms of one node in FP64 from the primitives: W b^i and
+// the Eulerian projections of T^{mu nu},
+//   Z = rho h* W^2, b^i = B^i / W + W (v.B) v^i, E = Z - p* - W^2 (v.B)^2,
+//   S_i = Z v_i - W (v.B) b_i, S^ij = Z v^i v^j + p* gamma^ij - b^i b^j,
+// with h* = 1 + eps + (p + b^2)/rho, p* = p + b^2/2 (alpha b^0 = W (v.B); the spatial part of
+// b_mu is b_i).  The factor sqrt(gamma) goes into the scalars once instead of into every
+// flux, F^i_{B^k} is formed from the densitized field and antisymmetric, and no T^{mu nu}
+// is built: ~140 FP64 instructions against ~240 for the four-vector form, on a kernel
+// that the FP64 pipe bounds.  mat (densitized): E, S_i, E + S, S^ij, Z v_i v_j - b_i b_j (the
+// right-hand side needs S_ij only up to multiples of gamma_ij; S = E - rho (1 + eps) + 3 p).
+__device__ __forceinline__ void fluxes64(long long p, long long P, double alpha, const double beta[3],
+                                         const double g[3][3], const double gi[3][3], double e4, double sqg,
+                                         double rho, const double v[3], double eps, double pr, double W,
+                                         const double B[3], const double* __restrict__ U, double* __restrict__ flux,
+                                         double* __restrict__ mat) {
+    double v_d[3], B_d[3], b_u[3], b_d[3], vt[3];
+    for (int i = 0; i < 3; i++) {
+        v_d[i] = g[i][0] * v[0] + g[i][1] * v[1] + g[i][2] * v[2];
+        B_d[i] = g[i][0] * B[0] + g[i][1] * B[1] + g[i][2] * B[2];
+    }
+    const double iW = 1.0 / W;
+    const double vB = v_d[0] * B[0] + v_d[1] * B[1] + v_d[2] * B[2], WvB = W * vB;
+    const double b2 = (B_d[0] * B[0] + B_d[1] * B[1] + B_d[2] * B[2]) * (iW * iW) + vB * vB;
+    for (int i = 0; i < 3; i++) {
+        b_u[i] = B[i] * iW + WvB * v[i];
+        b_d[i] = B_d[i] * iW + WvB * v_d[i];
+        vt[i] = alpha * v[i] - beta[i];
+    }
+    const double r1 = rho + rho * eps, ps = pr + 0.5 * b2;
+    const double Z = (r1 + pr + b2) * (W * W);
+    const double D = sqg * (rho * W), E = sqg * (Z - ps - WvB * WvB), tau = E - D;
+    const double sZ = sqg * Z, aps = alpha * (sqg * ps), sW = sqg * WvB;
+    double S[3], Bw[3], Bs[3];
+    const double aw = alpha * iW;
+    for (int i = 0; i < 3; i++) {
+        S[i] = sZ * v_d[i] - sW * b_d[i];
+        Bs[i] = U[(V_B + i) * P + p];
+        Bw[i] = aw * Bs[i];
+    }
+    for (int i = 0; i < 3; i++) {
+        double* F = flux + (long long)(i * 8) * P + p;
+        F[0 * P] = D * vt[i];
+        for (int j = 0; j < 3; j++) {
+            const double f = S[j] * vt[i] - b_d[j] * Bw[i];
+            F[(1 + j) * P] = i == j ? f + aps : f;
+        }
+        F[4 * P] = tau * vt[i] + (aps * v[i] - WvB * Bw[i]);
+        F[(5 + i) * P] = 0.0;
+    }
+    for (int i = 0; i < 3; i++)
+        for (int k = i + 1; k < 3; k++) {
+            const double f = vt[i] * Bs[k] - vt[k] * Bs[i];
+            flux[(long long)(i * 8 + 5 + k) * P + p] = f;
+            flux[(long long)(k * 8 + 5 + i) * P + p] = -f;
+        }
+    mat[0 * P + p] = E;
+    for (int i = 0; i < 3; i++) mat[(1 + i) * P + p] = S[i];
+    mat[4 * P + p] = 2.0 * E - sqg * (r1 - 3.0 * pr);
+    const double sp = sqg * ps;
+    double zv[3], zd[3], sb[3], sd[3];
+    for (int i = 0; i < 3; i++) {
+        zv[i] = sZ * v[i];
+        zd[i] = sZ * v_d[i];
+        sb[i] = sqg * b_u[i];
+        sd[i] = sqg * b_d[i];
+    }
+    for (int i = 0; i < 3; i++)
+        for (int j = i; j < 3; j++) {
+            mat[(5 + SI(i, j)) * P + p] = zv[i] * v[j] + (sp * gi[i][j] - sb[i] * b_u[j]);
+            mat[(11 + SI(i, j)) * P + p] = zd[i] * v_d[j] - sd[i] * b_d[j];
+        }
+}
+
 template <typename R>
 __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const double* __restrict__ U,
                                               double* __restrict__ prim, double* __restrict__ flux,
@@ -373,9 +446,13 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
         prim[5 * P + p] = pr;
         prim[6 * P + p] = W;
 
-        // ---- four-vectors, fluxes and T^{mu nu} in R: FP64, or FP32 in the mixed modes
-        // (their consumers, the tensor-core contractions and the FP32 right-hand side, keep
-        // about 24 bits); the primitive recovery above stays FP64
+        if constexpr (sizeof(R) == 8) {
+            fluxes64(p, P, alpha, beta, g, gi, e4, sqg, rho, v, eps, pr, W, B_u, U, flux, tmn);
+            met[9 * P + p] = isq;
+        } else {
+        // ---- four-vectors, fluxes and T^{mu nu} of the mixed modes in FP32 (their consumers,
+        // the tensor-core contractions and the FP32 right-hand side, keep about 24 bits); the
+        // primitive recovery above stays FP64
         const R alphaR = narrow<R>(alpha), sqgR = narrow<R>(sqg), WR = narrow<R>(W);
         R gR[3][3], betaR[3], vR[3], BR[3];
         for (int i = 0; i < 3; i++) {
@@ -415,15 +492,9 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
         // W^2 - 1 = W^2 v^2 and W - 1 = W^2 v^2 / (W + 1),
         // tau = rho W (eps W + W^2 v^2 / (W + 1)) + p W^2 v^2 + b^2 (W^2 - 1/2) - alpha^2 b0^2
         // (tau ~ 1e-3 D for a cold gas: the direct form loses 3 digits, all of FP32's margin)
-        // (FP32 only; FP64 keeps the direct form, which the oracle also uses)
-        R taup;
-        if constexpr (sizeof(R) == 4) {
-            const R Wv2 = WR * WR * (v_d[0] * vR[0] + v_d[1] * vR[1] + v_d[2] * vR[2]);
-            taup = rhoR * WR * (epsR * WR + Wv2 / (WR + R(1.0))) + prR * Wv2 + b2 * (WR * WR - R(0.5)) -
-                   alphaR * alphaR * b0 * b0;
-        } else {
-            taup = rhohs * WR * WR - pstar - alphaR * alphaR * b0 * b0 - Dp;
-        }
+        const R Wv2 = WR * WR * (v_d[0] * vR[0] + v_d[1] * vR[1] + v_d[2] * vR[2]);
+        const R taup = rhoR * WR * (epsR * WR + Wv2 / (WR + R(1.0))) + prR * Wv2 + b2 * (WR * WR - R(0.5)) -
+                       alphaR * alphaR * b0 * b0;
         // ---- densitized fluxes [dir][var]
         R vt[3];
         for (int i = 0; i < 3; i++) vt[i] = alphaR * vR[i] - betaR[i];
@@ -450,6 +521,7 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
         for (int m = 0; m < 4; m++)
             for (int k = m; k < 4; k++, n++)
                 tmn[n * P + p] = widen(rhohs * u4[m] * u4[k] + pstar * gu[m][k] - b4[m] * b4[k]);
+        }
         lam[p] = fabs(beta[0]) + alpha * sqrt(gi[0][0]);
     }
     // warp-aggregated failure count
@@ -461,25 +533,27 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
 // the 6 second-derivative pairs rr, rth, rph, thth, thph, phph use the same packing
 #define c_pair_idx(i, j) sym_idx(i, j)
 
-// The FP32-algebra instance is capped at 170 registers (3 blocks per SM): its spills cost
-// less than the latency its extra warps hide (measured 0.23 -> 0.18 ms on 393k nodes); the
-// FP64 instance is FP64-pipe bound and keeps 255.
-template <typename DT, typename R, bool HAM>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 1) k_rhs(Dims d, PhysParams pp, const double* __restrict__ U0,
+// The mixed modes' right-hand side (FP32 algebra; FP64 runs k_rhs64 below).  Bound by memory
+// and latency, not by arithmetic, so it keeps the four-dimensional form of the matter terms.
+// Capped at 170 registers (3 blocks per SM): its spills cost less than the latency its
+// extra warps hide (measured 0.23 -> 0.18 ms on 393k nodes).
+template <bool HAM>
+__global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const double* __restrict__ U0,
                                              const double* __restrict__ Us,
                                              const double* __restrict__ prim,
                                              const double* __restrict__ flux,
                                              const double* __restrict__ tmn,
                                              const double* __restrict__ lam,
                                              const double* __restrict__ met,
-                                             const DT* __restrict__ d1,
-                                             const DT* __restrict__ d2,
-                                             const DT* __restrict__ divF,
-                                             const DT* __restrict__ divB,
+                                             const float* __restrict__ d1,
+                                             const float* __restrict__ d2,
+                                             const float* __restrict__ divF,
+                                             const float* __restrict__ divB,
                                              const double* __restrict__ r_scale,
                                              const double* __restrict__ dt_dev, RKCoef co,
                                              double* __restrict__ out, double* __restrict__ acc,
                                              double* __restrict__ ham) {
+    using R = float;
     long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long P = d.P;
     if (p >= P) return;
@@ -885,6 +959,464 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? 3 : 1) k_rhs(Dims d, Phy
     }
 }
 
+// --------------------------------------------------------------------------- k_rhs64
+// The FP64 right-hand side.  GB300's FP64 pipe (2 instructions per SM clock) bounds it, so
+// the algebra is arranged for the fewest FP64 instructions (~950 per node and stage, 1,567
+// in the form of k_rhs below; the arrangement is the same system of equations):
+//   * matter as densitized Eulerian projections (see k_prep): the Valencia sources contract
+//     S^ij alone, 1/2 S^ij d_k gamma_ij + S_i d_k beta^i - E d_k alpha (T^00 beta beta +
+//     2 T^0i beta + T^ij is S^ij), and S_ij needs no lowering;
+//   * C_kij = 2 Gammatilde_kij from d_i gammatilde_jk: nine of its 18 components are single
+//     derivatives (C_iij = d_j gammatilde_ii), the others take 1 or 2 operations;
+//   * Gammatilde^k d_k gammatilde_ij replaces Gammatilde^k (Gammatilde_ijk + Gammatilde_jik);
+//   * only the trace-free part of X_ij is used, so its terms proportional to gammatilde_ij
+//     (Laplacian of phi, (d phi)^2, d phi . d alpha, the pressure) are left out;
+//   * - 2/3 div beta goes into the diagonal of d_j beta^k, alpha (K/2 - Atilde) beside it;
+//   * every gammatilde^ij v_j term of the Gammatilde equation shares one product.
+// A variable is written as soon as its right-hand side is known (no array of 33 in local
+// memory: 254 registers without spills, against 904 B of spills per thread).  Measured on
+// 393,216 nodes, per launch: 1.085 -> 0.603 ms.  MODE: 0 the plain right-hand side, 1 the first SSP-RK3 stage Us + dt L, 2 the
+// others a U0 + b (Us + dt L), 3 RK4 stages.
+template <int MODE>
+struct Emit {
+    const double *U0, *Us;
+    double *out, *acc;
+    long long P, p;
+    double a, b, bdt, cdt, wdt;
+    int acc_mode;
+    bool frozen;
+    __device__ __forceinline__ void operator()(int v, double L) const {
+        const long long ix = v * P + p;
+        if (frozen) L = 0.0;
+        if (MODE == 0) out[ix] = L;
+        else if (MODE == 1) out[ix] = fma(bdt, L, Us[ix]);
+        else if (MODE == 2) out[ix] = fma(bdt, L, fma(b, Us[ix], a * U0[ix]));
+        else {
+            // next stage input U0 + c dt L, accumulator acc (+)= w dt L; final stage U0 + acc + w dt L
+            const double u0 = U0[ix];
+            if (acc_mode == 1) { acc[ix] = wdt * L; out[ix] = fma(cdt, L, u0); }
+            else if (acc_mode == 2) { acc[ix] = fma(wdt, L, acc[ix]); out[ix] = fma(cdt, L, u0); }
+            else out[ix] = u0 + fma(wdt, L, acc[ix]);
+        }
+    }
+};
+
+template <int MODE, bool HAM>
+__global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const double* __restrict__ U0,
+                                               const double* __restrict__ Us, const double* __restrict__ flux,
+                                               const double* __restrict__ mat, const double* __restrict__ lam,
+                                               const double* __restrict__ met, const double* __restrict__ d1,
+                                               const double* __restrict__ d2, const double* __restrict__ divF,
+                                               const double* __restrict__ divB, const double* __restrict__ r_scale,
+                                               const double* __restrict__ dt_dev, RKCoef co,
+                                               double* __restrict__ out, double* __restrict__ acc,
+                                               double* __restrict__ ham) {
+    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long P = d.P;
+    if (p >= P) return;
+    const int e = (int)(p / d.elem);
+    const long long ir = (p / d.NtNp) % d.Nr;
+    const double dt = MODE == 0 ? 0.0 : dt_dev[d.elem_inst[e]];
+    // the outer boundary node of each instance is frozen
+    const Emit<MODE> emit = {U0, Us, out, acc, P, p, co.a, co.b, co.b * dt, co.c * dt, co.w * dt, co.acc_mode,
+                             ir == d.Nr - 1 && !d.iface_next[e]};
+#define LD(a, k) __ldg((a) + (long long)(k) * P + p)
+#define D1(f, dd) LD(d1, (f) * 3 + (dd))
+#define D2(f, q) LD(d2, (f) * 6 + (q))
+    const double alpha = LD(Us, V_ALPHA), K = LD(Us, V_K);
+    double beta[3], gt[6], At[6], gti[6], dgt[3][6], dphi[3], dal[3], dbe[3][3];
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+        gt[q] = LD(Us, V_GT + q);
+        At[q] = LD(Us, V_AT + q);
+        gti[q] = LD(met, 3 + q);
+    }
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        beta[k] = LD(Us, V_BETA + k);
+        dphi[k] = D1(V_PHI, k);
+        dal[k] = D1(V_ALPHA, k);
+#pragma unroll
+        for (int q = 0; q < 6; q++) dgt[k][q] = D1(V_GT + q, k);
+#pragma unroll
+        for (int i = 0; i < 3; i++) dbe[k][i] = D1(V_BETA + i, k);
+    }
+    const double e4m = LD(met, 1);
+    const double third = 1.0 / 3.0;
+
+    // ------------------------------------------------------------ Valencia
+    // mat: sqrt(gamma) times E, S_i, E + S, S^ij, Z v_i v_j - b_i b_j
+    double S_u[3];  // sqrt(gamma) gammatilde^ij S_j
+    {
+        double S_d[3];
+#pragma unroll
+        for (int i = 0; i < 3; i++) S_d[i] = LD(mat, 1 + i);
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+            S_u[i] = gti[SI(i, 0)] * S_d[0] + gti[SI(i, 1)] * S_d[1] + gti[SI(i, 2)] * S_d[2];
+        if (pp.evolve_fluid) {
+            double r[8];
+#pragma unroll
+            for (int v = 0; v < 8; v++) r[v] = -LD(divF, v);
+            // V^ij = 1/2 alpha e^{4phi} S^ij, twice that off the diagonal (symmetric sums)
+            const double ae = alpha * LD(met, 0), hae = 0.5 * ae;
+            double V[6], tr = 0.0, VA = 0.0;
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+#pragma unroll
+                for (int j = i; j < 3; j++) {
+                    const int q = SI(i, j);
+                    V[q] = (i == j ? hae : ae) * LD(mat, 5 + q);
+                    tr = fma(V[q], gt[q], tr);
+                    VA = fma(V[q], At[q], VA);
+                }
+            const double E = LD(mat, 0), f4 = 4.0 * tr;
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                // d_k gamma_ij = e^{4phi} (d_k gammatilde_ij + 4 gammatilde_ij d_k phi)
+                double s = r[1 + k];
+#pragma unroll
+                for (int q = 0; q < 6; q++) s = fma(V[q], dgt[k][q], s);
+                s = fma(f4, dphi[k], s);
+#pragma unroll
+                for (int i = 0; i < 3; i++) s = fma(S_d[i], dbe[k][i], s);
+                r[1 + k] = fma(-E, dal[k], s);
+            }
+            // alpha S^ij K_ij - S^i d_i alpha, K_ij = e^{4phi} (Atilde_ij + gammatilde_ij K / 3)
+            r[4] = fma(2.0, fma(K * third, tr, VA), r[4]);
+            r[4] = fma(-e4m, S_u[0] * dal[0] + S_u[1] * dal[1] + S_u[2] * dal[2], r[4]);
+            if (pp.glm) {
+                // GLM cleaning: see k_rhs
+                double dpsi[3];
+#pragma unroll
+                for (int k = 0; k < 3; k++) dpsi[k] = D1(N_D1, k);
+                const double as = alpha * LD(met, 2) * e4m;
+#pragma unroll
+                for (int i = 0; i < 3; i++)
+                    r[5 + i] -= as * (gti[SI(i, 0)] * dpsi[0] + gti[SI(i, 1)] * dpsi[1] + gti[SI(i, 2)] * dpsi[2]);
+                emit(V_PSI, -alpha * fma(pp.glm_ch2 * divB[p], LD(met, 9), LD(Us, V_PSI) * pp.glm_itau));
+            }
+            // interface penalty (Rusanov flux, strong form) at duplicated element-end nodes
+            int side = 0;
+            if (ir == d.Nr - 1 && d.iface_next[e]) side = +1;
+            if (ir == 0 && e > 0 && d.iface_next[e - 1]) side = -1;
+            if (side != 0) {
+                const long long pl = side > 0 ? p : p - d.NtNp, pr = pl + d.NtNp;
+                const double hl = 0.5 * fmax(lam[pl], lam[pr]);
+                const double fac = r_scale[e] / pp.w_end;
+#pragma unroll
+                for (int v = 0; v < 8; v++) {
+                    const double FL = flux[v * P + pl], FR = flux[v * P + pr];
+                    const double UL = Us[(V_D + v) * P + pl], UR = Us[(V_D + v) * P + pr];
+                    const double Fs = 0.5 * (FL + FR) - hl * (UR - UL);
+                    r[v] = side > 0 ? fma(FL - Fs, fac, r[v]) : fma(Fs - FR, fac, r[v]);
+                }
+            }
+#pragma unroll
+            for (int v = 0; v < 8; v++) emit(V_D + v, r[v]);
+        } else {
+            for (int v = V_D; v < NV + pp.glm; v++) emit(v, 0.0);
+        }
+    }
+    if (!pp.evolve_metric) {
+        for (int v = 0; v < N_BSSN; v++) emit(v, 0.0);
+        return;
+    }
+
+    // ------------------------------------------------------------ gammatilde, phi, lapse, shift
+    const double bdal = beta[0] * dal[0] + beta[1] * dal[1] + beta[2] * dal[2];
+    const double aK = alpha * K;
+    const double divb = dbe[0][0] + dbe[1][1] + dbe[2][2], db3 = divb * third;
+    emit(V_PHI, fma(-1.0 / 6.0, aK, fma(0.5, db3, beta[0] * dphi[0] + beta[1] * dphi[1] + beta[2] * dphi[2])));
+    if (pp.gauge == 0) {
+        emit(V_ALPHA, fma(-2.0, aK, bdal));
+#pragma unroll
+        for (int i = 0; i < 3; i++) emit(V_BETA + i, 0.75 * LD(Us, V_BG + i));
+    } else {
+        emit(V_ALPHA, 0.0);
+#pragma unroll
+        for (int i = 0; i < 3; i++) emit(V_BETA + i, 0.0);
+    }
+    // trace-free d_j beta^k: carries the -2/3 div beta terms of the conformal tensors
+#pragma unroll
+    for (int i = 0; i < 3; i++) dbe[i][i] -= db3;
+    const double m2a = -2.0 * alpha;
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = i; j < 3; j++) {
+            const int q = SI(i, j);
+            double s = m2a * At[q];
+#pragma unroll
+            for (int k = 0; k < 3; k++) s = fma(beta[k], dgt[k][q], s);
+            if (i == j) {
+                s = fma(2.0, gt[SI(i, 0)] * dbe[i][0] + gt[SI(i, 1)] * dbe[i][1] + gt[SI(i, 2)] * dbe[i][2], s);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    s = fma(gt[SI(i, k)], dbe[j][k], s);
+                    s = fma(gt[SI(j, k)], dbe[i][k], s);
+                }
+            }
+            emit(V_GT + q, s);
+        }
+
+    // ------------------------------------------------------------ Christoffel symbols, Ricci tensor
+    double Cu[3][6], Gd[3], R2[6], gw[6];  // Gammatilde^k_ij, its trace, 2 Rtilde_ij, weighted inverse
+    {
+        double C[3][6];
+#pragma unroll
+        for (int k = 0; k < 3; k++)
+#pragma unroll
+            for (int i = 0; i < 3; i++)
+#pragma unroll
+                for (int j = i; j < 3; j++) {
+                    const int q = SI(i, j);
+                    if (k == i) C[k][q] = dgt[j][SI(i, i)];
+                    else if (k == j) C[k][q] = dgt[i][SI(j, j)];
+                    else if (i == j) C[k][q] = fma(2.0, dgt[i][SI(k, i)], -dgt[k][q]);
+                    else C[k][q] = dgt[i][SI(k, j)] + dgt[j][SI(k, i)] - dgt[k][q];
+                }
+        double hg[6];
+#pragma unroll
+        for (int q = 0; q < 6; q++) hg[q] = 0.5 * gti[q];
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = i; j < 3; j++) gw[SI(i, j)] = i == j ? gti[SI(i, j)] : gti[SI(i, j)] + gti[SI(i, j)];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            double s = 0.0;
+#pragma unroll
+            for (int q = 0; q < 6; q++) {
+                Cu[k][q] = hg[SI(k, 0)] * C[0][q] + hg[SI(k, 1)] * C[1][q] + hg[SI(k, 2)] * C[2][q];
+                s = q == 0 ? gw[0] * Cu[k][0] : fma(gw[q], Cu[k][q], s);
+            }
+            Gd[k] = s;
+        }
+#pragma unroll
+        for (int q = 0; q < 6; q++) R2[q] = Gd[0] * dgt[0][q] + Gd[1] * dgt[1][q] + Gd[2] * dgt[2][q];
+        // the quadratic part, gti^lm (Gamma^k_li Gamma_jkm + Gamma^k_lj Gamma_ikm + Gamma^k_im Gamma_klj)
+        // twice: P_ij + P_ji + Q_ij with T_i^km = Gamma^k_il gti^lm, P_ij = T_i^km C_jkm (T
+        // symmetrised: C is symmetric there), Q_ij = T_i^km C_kmj (symmetric in i, j)
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            double T[3][3];
+#pragma unroll
+            for (int k = 0; k < 3; k++)
+#pragma unroll
+                for (int m = 0; m < 3; m++)
+                    T[k][m] = Cu[k][SI(i, 0)] * gti[SI(0, m)] + Cu[k][SI(i, 1)] * gti[SI(1, m)] +
+                              Cu[k][SI(i, 2)] * gti[SI(2, m)];
+            const double t01 = T[0][1] + T[1][0], t02 = T[0][2] + T[2][0], t12 = T[1][2] + T[2][1];
+#pragma unroll
+            for (int j = 0; j < 3; j++) {
+                const int q = SI(i, j);
+                const double* c = C[j];
+                if (i == j) {
+                    const double s = T[0][0] * c[0] + t01 * c[1] + t02 * c[2] + T[1][1] * c[3] + t12 * c[4] + T[2][2] * c[5];
+                    R2[q] = fma(2.0, s, R2[q]);
+                } else {
+                    R2[q] = fma(T[0][0], c[0], R2[q]);
+                    R2[q] = fma(t01, c[1], R2[q]);
+                    R2[q] = fma(t02, c[2], R2[q]);
+                    R2[q] = fma(T[1][1], c[3], R2[q]);
+                    R2[q] = fma(t12, c[4], R2[q]);
+                    R2[q] = fma(T[2][2], c[5], R2[q]);
+                }
+                if (j >= i)
+#pragma unroll
+                    for (int k = 0; k < 3; k++)
+#pragma unroll
+                        for (int m = 0; m < 3; m++) R2[q] = fma(T[k][m], C[k][SI(m, j)], R2[q]);
+            }
+        }
+    }
+    double dGam[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int i = 0; i < 3; i++) dGam[k][i] = D1(V_GAM + i, k);
+
+    // ------------------------------------------------------------ X_ij, trace-free part
+    // X_ij = -D_i D_j alpha + alpha (R_ij - 8 pi S_ij) up to multiples of gammatilde_ij:
+    // -d_i d_j alpha - 2 alpha d_i d_j phi + Gamma^k_ij (d_k alpha + 2 alpha d_k phi)
+    // + 2 d_i phi (d_j alpha + alpha d_j phi) + (i <-> j) + alpha (Rtilde_ij - 8 pi S_ij)
+    const double m8 = 8.0 * 3.141592653589793 * alpha * LD(met, 9);
+    double X[6], trX = 0.0, ddal_tr = 0.0, ddphi_tr = 0.0;
+    {
+        const double ha = 0.5 * alpha;
+        double qv[3], pv[3], tv[3];
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            qv[k] = fma(-m2a, dphi[k], dal[k]);
+            tv[k] = fma(alpha, dphi[k], dal[k]);
+            pv[k] = 2.0 * dphi[k];
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = i; j < 3; j++) {
+                const int q = SI(i, j);
+                double R = R2[q];
+#pragma unroll
+                for (int l = 0; l < 6; l++) R = fma(-gw[l], D2(q, l), R);
+                if (i == j) {
+                    R = fma(2.0, gt[SI(i, 0)] * dGam[i][0] + gt[SI(i, 1)] * dGam[i][1] + gt[SI(i, 2)] * dGam[i][2], R);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 3; k++) {
+                        R = fma(gt[SI(k, i)], dGam[j][k], R);
+                        R = fma(gt[SI(k, j)], dGam[i][k], R);
+                    }
+                }
+                const double dda = D2(7, q), ddp = D2(6, q);
+                ddal_tr = fma(gw[q], dda, ddal_tr);
+                if (HAM) ddphi_tr = fma(gw[q], ddp, ddphi_tr);
+                double s = fma(m2a, ddp, -dda);
+#pragma unroll
+                for (int k = 0; k < 3; k++) s = fma(Cu[k][q], qv[k], s);
+                s = fma(pv[i], tv[j], s);
+                s = fma(pv[j], tv[i], s);
+                s = fma(ha, R, s);
+                X[q] = fma(-m8, LD(mat, 11 + q), s);
+                trX = fma(gw[q], X[q], trX);
+            }
+    }
+    // gammatilde^ij d_i phi d_j alpha; D^i D_i alpha
+    double dphi_u[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+        dphi_u[k] = gti[SI(k, 0)] * dphi[0] + gti[SI(k, 1)] * dphi[1] + gti[SI(k, 2)] * dphi[2];
+    const double gpa = dphi_u[0] * dal[0] + dphi_u[1] * dal[1] + dphi_u[2] * dal[2];
+    double lap = fma(2.0, gpa, ddal_tr);
+#pragma unroll
+    for (int k = 0; k < 3; k++) lap = fma(-Gd[k], dal[k], lap);
+    lap *= e4m;
+
+    // ------------------------------------------------------------ Atilde, K
+    double Aud[3][3], Auu[6], AA = 0.0;  // Atilde^k_j; Atilde^ij (twice off the diagonal below)
+#pragma unroll
+    for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+            Aud[k][j] = gti[SI(k, 0)] * At[SI(0, j)] + gti[SI(k, 1)] * At[SI(1, j)] + gti[SI(k, 2)] * At[SI(2, j)];
+#pragma unroll
+    for (int i = 0; i < 3; i++)
+#pragma unroll
+        for (int j = i; j < 3; j++)
+            Auu[SI(i, j)] = Aud[i][0] * gti[SI(0, j)] + Aud[i][1] * gti[SI(1, j)] + Aud[i][2] * gti[SI(2, j)];
+    // 2 alpha (Atilde^ij (6 d_j phi) ) - 2 Atilde^ij d_j alpha
+    double rG[3];
+    {
+        double w[3];
+        const double a12 = 12.0 * alpha;
+#pragma unroll
+        for (int k = 0; k < 3; k++) w[k] = fma(a12, dphi[k], -2.0 * dal[k]);
+#pragma unroll
+        for (int i = 0; i < 3; i++) rG[i] = Auu[SI(i, 0)] * w[0] + Auu[SI(i, 1)] * w[1] + Auu[SI(i, 2)] * w[2];
+    }
+    Auu[1] += Auu[1];
+    Auu[2] += Auu[2];
+    Auu[4] += Auu[4];
+#pragma unroll
+    for (int q = 0; q < 6; q++) AA = fma(At[q], Auu[q], AA);
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+        double s = 0.0;
+#pragma unroll
+        for (int q = 0; q < 6; q++) s = q == 0 ? Cu[i][0] * Auu[0] : fma(Cu[i][q], Auu[q], s);
+        rG[i] = fma(-m2a, s, rG[i]);
+    }
+    double dK[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) dK[k] = D1(V_K, k);
+    {
+        double s = fma(alpha, fma(K * third, K, AA), -lap);
+        s = fma(0.5 * m8, LD(mat, 4), s);
+#pragma unroll
+        for (int k = 0; k < 3; k++) s = fma(beta[k], dK[k], s);
+        emit(V_K, s);
+    }
+    if (HAM) {
+        // Hamiltonian constraint R + (2/3) K^2 - Atilde.Atilde - 16 pi E with e^{4phi} R =
+        // gammatilde^ij R_ij: trX holds alpha (its part without the gammatilde_ij terms) minus
+        // the lapse and matter terms, which are taken out again
+        double gdp2 = dphi_u[0] * dphi[0] + dphi_u[1] * dphi[1] + dphi_u[2] * dphi[2];
+        double lapphi = ddphi_tr, pl = ddal_tr, mt = 0.0;
+#pragma unroll
+        for (int k = 0; k < 3; k++) {
+            lapphi = fma(-Gd[k], dphi[k], lapphi);
+            pl = fma(-Gd[k], dal[k], pl);
+        }
+#pragma unroll
+        for (int q = 0; q < 6; q++) mt = fma(gw[q], LD(mat, 11 + q), mt);
+        const double trR = (trX + pl - 4.0 * gpa + m8 * mt) / alpha - 6.0 * lapphi - 12.0 * gdp2;
+        ham[p] = e4m * trR + 2.0 * third * K * K - AA - 16.0 * 3.141592653589793 * LD(mat, 0) * LD(met, 9);
+    }
+    {
+        const double c1 = -(e4m * trX) * third, hk = 0.5 * aK;
+        // d_j beta^k - alpha Atilde^k_j + 1/2 alpha K delta: the Lie, quadratic and K terms of Atilde
+        double H[3][3];
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                H[j][k] = fma(-alpha, Aud[k][j], dbe[j][k]);
+                if (j == k) H[j][k] += hk;
+            }
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+#pragma unroll
+            for (int j = i; j < 3; j++) {
+                const int q = SI(i, j);
+                double s = fma(e4m, X[q], c1 * gt[q]);
+#pragma unroll
+                for (int k = 0; k < 3; k++) s = fma(beta[k], D1(V_AT + q, k), s);
+                if (i == j) {
+                    s = fma(2.0, At[SI(i, 0)] * H[i][0] + At[SI(i, 1)] * H[i][1] + At[SI(i, 2)] * H[i][2], s);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 3; k++) {
+                        s = fma(At[SI(i, k)], H[j][k], s);
+                        s = fma(At[SI(j, k)], H[i][k], s);
+                    }
+                }
+                emit(V_AT + q, s);
+            }
+    }
+
+    // ------------------------------------------------------------ Gammatilde, driver
+    {
+        const double a43 = -4.0 * third * alpha;
+        double v[3];
+#pragma unroll
+        for (int j = 0; j < 3; j++) {
+            // d_j d_k beta^k
+            const double t = D2(8, SI(j, 0)) + D2(9, SI(j, 1)) + D2(10, SI(j, 2));
+            v[j] = fma(a43, dK[j], t * third);
+        }
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            double s = fma(-2.0 * m8, S_u[i], rG[i]);
+#pragma unroll
+            for (int q = 0; q < 6; q++) s = fma(gw[q], D2(8 + i, q), s);
+#pragma unroll
+            for (int k = 0; k < 3; k++) {
+                s = fma(gti[SI(i, k)], v[k], s);
+                s = fma(beta[k], dGam[k][i], s);
+                s = fma(-LD(Us, V_GAM + k), dbe[k][i], s);
+            }
+            s = fma(db3, LD(Us, V_GAM + i), s);
+            emit(V_GAM + i, s);
+            emit(V_BG + i, pp.gauge == 0 ? fma(-pp.eta, LD(Us, V_BG + i), s) : 0.0);
+        }
+    }
+#undef LD
+#undef D1
+#undef D2
+}
+
 // --------------------------------------------------------------------------- launchers
 cudaError_t launch_prep(const Dims& d, const PhysParams& pp, const double* U, double* prim,
                         double* flux, double* tmn, double* lam, unsigned long long* nfail, double* met,
@@ -904,14 +1436,21 @@ cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, co
                        double* ham) {
     int bs = 128;
     long long nb = (d.P + bs - 1) / bs;
-#define RHS_ARGS(T) d, pp, U0, Us, prim, flux, tmn, lam, met, (const T*)d1, (const T*)d2, (const T*)divF, \
-                    (const T*)divB, r_scale_dev, dt_dev, co, out, acc, ham
+#define RHS_ARGS d, pp, U0, Us, prim, flux, tmn, lam, met, (const float*)d1, (const float*)d2, (const float*)divF, \
+                    (const float*)divB, r_scale_dev, dt_dev, co, out, acc, ham
     if (deriv_fp32) {
-        if (ham) k_rhs<float, float, true><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS(float));
-        else k_rhs<float, float, false><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS(float));
+        if (ham) k_rhs<true><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
+        else k_rhs<false><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
     } else {
-        if (ham) k_rhs<double, double, true><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS(double));
-        else k_rhs<double, double, false><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS(double));
+#define RHS64_ARGS d, pp, U0, Us, flux, tmn, lam, met, (const double*)d1, (const double*)d2, (const double*)divF, \
+                   (const double*)divB, r_scale_dev, dt_dev, co, out, acc, ham
+        const unsigned g = (unsigned)nb;
+        if (ham) k_rhs64<0, true><<<g, bs, 0, s>>>(RHS64_ARGS);
+        else if (co.acc_mode < 0) k_rhs64<0, false><<<g, bs, 0, s>>>(RHS64_ARGS);
+        else if (co.acc_mode > 0) k_rhs64<3, false><<<g, bs, 0, s>>>(RHS64_ARGS);
+        else if (co.a == 0.0 && co.b == 1.0) k_rhs64<1, false><<<g, bs, 0, s>>>(RHS64_ARGS);
+        else k_rhs64<2, false><<<g, bs, 0, s>>>(RHS64_ARGS);
+#undef RHS64_ARGS
     }
 #undef RHS_ARGS
     return cudaGetLastError();
