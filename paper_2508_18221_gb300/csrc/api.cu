@@ -717,8 +717,11 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
                 c->tc_fy[src32][h] = (int)tj.size();
                 if (c->ft)
                     for (int i = 0; i < c->nfold; i++) {
+                        // FP32 fields of Y sit at the byte offset of the FP64 field of the same
+                        // number: the second derivatives (FP32, side stream) and the flux
+                        // divergence (FP64, main stream) fold at the same time
                         const long long o = (long long)i * P + h * (P / 2);
-                        addt(src32 ? (const void*)(Yf + o) : (const void*)(c->Y + o), Zf + o, 0);
+                        addt(src32 ? (const void*)(Yf + (o + (long long)i * P)) : (const void*)(c->Y + o), Zf + o, 0);
                     }
             }
         if (cudaMalloc(&c->tcjobs, tj.size() * sizeof(TcJob)) != cudaSuccess ||
@@ -767,7 +770,7 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
             for (int x = 0; x < 2; x++) {
                 const long long i = n1 + 2 * q + x, so = ((long long)v2[q] * 3 + 1 + x) * P;
                 const int par = x == 0 ? -kThetaParity[v2[q]] : kThetaParity[v2[q]];
-                if (mixed) addf(reinterpret_cast<const float*>(c->d1) + so, Yf + i * P, par, 0);
+                if (mixed) addf(reinterpret_cast<const float*>(c->d1) + so, Yf + 2 * i * P, par, 0);
                 else addf(c->d1 + so, c->Y + i * P, par, 0);
             }
         c->fj_second_u = (int)fj.size();
