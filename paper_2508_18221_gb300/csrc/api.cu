@@ -1297,7 +1297,7 @@ extern "C" int grmhd_con2prim(grmhd_ctx* c, double* prim_out, int on_device, lon
     NvtxRange nvtx_range("grmhd_con2prim");
     if (!c) return GRMHD_EINVAL;
     CK(cudaMemsetAsync(c->nfail, 0, sizeof(unsigned long long), c->stream));
-    CK(launch_prep(c->d, c->pp, c->U[0], c->prim, c->flux, c->tmn, c->lam, c->nfail, c->met, c->stream));
+    CK(launch_con2prim(c->d, c->pp, c->U[0], c->prim, c->nfail, c->stream));
     if (prim_out) {
         int st = copy_out(c, prim_out, c->prim, (size_t)N_PRIM * c->d.P, on_device);
         if (st) return st;
@@ -1395,7 +1395,7 @@ extern "C" int grmhd_diag(grmhd_ctx* c, double out[GRMHD_NDIAG]) {
         if (st) return st;
     }
     CK(cudaMemsetAsync(c->nfail, 0, sizeof(unsigned long long), c->stream));
-    CK(launch_prep(c->d, c->pp, c->U[0], c->prim, c->flux, c->tmn, c->lam, c->nfail, c->met, c->stream));
+    CK(launch_con2prim(c->d, c->pp, c->U[0], c->prim, c->nfail, c->stream));
     // divergence of the densitized field into scratch
     const long long P = c->d.P;
     DerivJob jb[3];

@@ -93,6 +93,9 @@ cudaError_t tc_init();
 cudaError_t launch_prep(const Dims& d, const PhysParams& pp, const double* U, double* prim,
                         double* flux, double* tmn, double* lam, unsigned long long* nfail, double* met,
                         cudaStream_t s, int fp32_algebra = 0);
+// the primitives of U alone (prim, nfail)
+cudaError_t launch_con2prim(const Dims& d, const PhysParams& pp, const double* U, double* prim,
+                            unsigned long long* nfail, cudaStream_t s);
 struct RKCoef { double a, b, c, w; int acc_mode; };  // out = a U0 + b Us + c dt L (+acc)
 // d1, d2, divF are double (FP64 mode) or float (deriv_fp32 = 1, mixed modes); ham != null
 // also writes the Hamiltonian constraint per node (diagnostics)

@@ -24,166 +24,191 @@ __host__ __device__ constexpr int sym_idx(int i, int j) {
 #define SI(i, j) sym_idx(i, j)
 
 // --------------------------------------------------------------------------- helpers
-__device__ __forceinline__ double det3(const double g[3][3]) {
-    return g[0][0] * (g[1][1] * g[2][2] - g[1][2] * g[2][1]) -
-           g[0][1] * (g[1][0] * g[2][2] - g[1][2] * g[2][0]) +
-           g[0][2] * (g[1][0] * g[2][1] - g[1][1] * g[2][0]);
+// Reciprocal and reciprocal square root: the hardware's 20-bit seeds (rcp / rsqrt.approx.f64)
+// with one Householder step of third order, y (1 + e + e^2), e = 1 - x y, and
+// y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2: the seed's error cubed is below 2^-56, so the results
+// are correctly rounded but for rare ties, in 3 and 5 FP64 instructions (1.0 / x and rsqrt(x) take about twice
+// as many, and the FP64 pipe bounds the kernels here).  Operands near the ends of the
+// exponent range, zero, Inf, NaN and negative ones take the library functions.
+__device__ __noinline__ double rcp64_any(double x) { return 1.0 / x; }
+__device__ __noinline__ double rsqrt64_any(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rcp64(double x) {
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
+    if (ex - 64u > 1918u) return rcp64_any(x);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
 }
-
-// inverse of a symmetric 3x3 matrix by cofactors; returns the determinant
-__device__ __forceinline__ double inv3sym(const double g[3][3], double gi[3][3]) {
-    double c00 = g[1][1] * g[2][2] - g[1][2] * g[1][2];
-    double c01 = g[0][2] * g[1][2] - g[0][1] * g[2][2];
-    double c02 = g[0][1] * g[1][2] - g[0][2] * g[1][1];
-    double c11 = g[0][0] * g[2][2] - g[0][2] * g[0][2];
-    double c12 = g[0][1] * g[0][2] - g[0][0] * g[1][2];
-    double c22 = g[0][0] * g[1][1] - g[0][1] * g[0][1];
-    double det = g[0][0] * c00 + g[0][1] * c01 + g[0][2] * c02;
-    double id = 1.0 / det;
-    gi[0][0] = c00 * id; gi[0][1] = gi[1][0] = c01 * id; gi[0][2] = gi[2][0] = c02 * id;
-    gi[1][1] = c11 * id; gi[1][2] = gi[2][1] = c12 * id; gi[2][2] = c22 * id;
-    return det;
+__device__ __forceinline__ double rsqrt64(double x) {
+    const unsigned ex = (unsigned)__double2hiint(x) >> 20;    // with the sign: negative is out of range
+    if (ex - 64u > 1918u) return rsqrt64_any(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y * y, 1.0);                      // y * y is exact: the seed's low word is zero
+    return fma(y, e * fma(0.375, e, 0.5), y);
 }
-
-// forward-mode dual number (value, d/dmu) for the Newton derivative of the master function
-struct Dual {
-    double v, d;
-};
-__device__ __forceinline__ Dual mk(double v, double d = 0.0) { Dual r; r.v = v; r.d = d; return r; }
-__device__ __forceinline__ Dual operator+(Dual a, Dual b) { return mk(a.v + b.v, a.d + b.d); }
-__device__ __forceinline__ Dual operator-(Dual a, Dual b) { return mk(a.v - b.v, a.d - b.d); }
-__device__ __forceinline__ Dual operator*(Dual a, Dual b) { return mk(a.v * b.v, a.d * b.v + a.v * b.d); }
-__device__ __forceinline__ Dual operator/(Dual a, Dual b) {
-    double iv = 1.0 / b.v;
-    double q = a.v * iv;
-    return mk(q, (a.d - q * b.d) * iv);
-}
-__device__ __forceinline__ Dual operator+(Dual a, double b) { return mk(a.v + b, a.d); }
-__device__ __forceinline__ Dual operator+(double a, Dual b) { return mk(a + b.v, b.d); }
-__device__ __forceinline__ Dual operator-(Dual a, double b) { return mk(a.v - b, a.d); }
-__device__ __forceinline__ Dual operator-(double a, Dual b) { return mk(a - b.v, -b.d); }
-__device__ __forceinline__ Dual operator*(Dual a, double b) { return mk(a.v * b, a.d * b); }
-__device__ __forceinline__ Dual operator*(double a, Dual b) { return mk(a * b.v, a * b.d); }
-__device__ __forceinline__ Dual operator/(double a, Dual b) {
-    double iv = 1.0 / b.v;
-    double q = a * iv;
-    return mk(q, -q * b.d * iv);
-}
-// 1/sqrt(a) and its derivative -a'/(2 a^{3/2}) = -a' r^3 / 2 (no division)
-__device__ __forceinline__ Dual drsqrt(Dual a) {
-    double r = rsqrt(a.v);
-    return mk(r, -0.5 * a.d * r * r * r);
-}
-__device__ __forceinline__ double drsqrt(double a) { return rsqrt(a); }
-__device__ __forceinline__ Dual dmin(Dual a, Dual b) { return a.v <= b.v ? a : b; }
-__device__ __forceinline__ Dual dmax(Dual a, Dual b) { return a.v >= b.v ? a : b; }
-__device__ __forceinline__ double dmin(double a, double b) { return fmin(a, b); }
-__device__ __forceinline__ double dmax(double a, double b) { return fmax(a, b); }
-__device__ __forceinline__ double val(double a) { return a; }
-__device__ __forceinline__ double val(Dual a) { return a.v; }
-template <class T> __device__ __forceinline__ T cst(double v);
-template <> __device__ __forceinline__ double cst<double>(double v) { return v; }
-template <> __device__ __forceinline__ Dual cst<Dual>(double v) { return mk(v); }
 
 // Scalar invariants of the conserved state entering the one-variable master function
 // in mu = 1/(h W) (Kastaun, Kalinani & Ciolfi 2021): q = tau/D, r^2 = S^2/D^2,
-// bb = B^2/D, rb2 = (S.B)^2/D^3.
+// bb = B^2/D, rb2 = (S.B)^2/D^3.  For the Gamma law h = 1 + Gamma eps, and the two
+// estimates of h/W whose larger one the method takes are equal except where eps is clamped
+// to eps_min, where h(eps_min)/W is the larger.  So the function is
+//   g(mu) = mu z - 1,  z = h/W + mu rbar^2 = 1 + qbar + (Gamma - 1) eps / W  (eps not clamped),
+// with the same sign and root as mu - 1/z and no further division.
+template <class T>
 struct C2PScal {
-    double D, q, r2, bb, rb2, gam, eps_min;
-    double v2max;   // r^2 / (1 + r^2), the largest admissible v^2
+    T r2, bb, rb2;
+    T c0, c1;       // qbar = c0 - c1 (mu x)^2: q - bb/2 and (bb r^2 - rb2)/2
+    T g1, eps_min;  // Gamma - 1
+    T v2max;        // r^2 / (1 + r^2), the largest admissible v^2
 };
 
-// One evaluation of the master function (value, or value and d/dmu for T = Dual):
-// 1/W = sqrt(1 - v^2) = (1 - v^2) W, so W comes from one reciprocal square root and h/W
-// needs no division.
-template <class T>
-__device__ __forceinline__ T master(T mu, const C2PScal& c, T* W_o, T* eps_o, T* x_o) {
-    T x = 1.0 / (1.0 + mu * c.bb);
-    T rbar2 = c.r2 * x * x + mu * x * (1.0 + x) * c.rb2;
-    T qbar = c.q - 0.5 * c.bb - 0.5 * mu * mu * x * x * (c.bb * c.r2 - c.rb2);
-    T v2 = dmin(mu * mu * rbar2, cst<T>(c.v2max));
-    T om = 1.0 - v2;
-    T W = drsqrt(om);
-    T eps = W * (qbar - mu * rbar2) + v2 * W * W / (1.0 + W);
-    T eps_c = dmax(eps, cst<T>(c.eps_min));
-    T ahat = (c.gam - 1.0) * eps_c / (1.0 + eps_c);
-    T h = (1.0 + eps_c) * (1.0 + ahat);
-    T nu = dmax(h * (om * W), (1.0 + ahat) * (1.0 + qbar - mu * rbar2));
-    if (W_o) *W_o = W;
-    if (eps_o) *eps_o = eps;
-    if (x_o) *x_o = x;
-    return mu - 1.0 / (nu + mu * rbar2);
+// g and its slope in FP32, with the derivatives the final correction needs
+struct Master32 {
+    float g, dg, dx, dv2, dqm;
+};
+__device__ __forceinline__ Master32 master32(float mu, const C2PScal<float>& c) {
+    Master32 r;
+    const float x = __fdividef(1.f, fmaf(mu, c.bb, 1.f)), mx = mu * x, x2 = x * x;    // d(mu x) = x^2
+    r.dx = -c.bb * x2;
+    const float rb = c.r2 * x2 + mx * (1.f + x) * c.rb2;
+    const float drb = 2.f * c.r2 * x * r.dx + c.rb2 * (x2 * (1.f + x) + mx * r.dx);
+    const float m1 = mu * rb, dm1 = fmaf(mu, drb, rb);
+    const float qb = c.c0 - c.c1 * mx * mx, dqb = -2.f * c.c1 * mx * x2;
+    r.dqm = dqb - dm1;
+    float v2 = mu * m1;
+    r.dv2 = fmaf(mu, dm1, m1);
+    if (!(v2 <= c.v2max)) { v2 = c.v2max; r.dv2 = 0.f; }
+    const float om = 1.f - v2, W = rsqrtf(om), iW = om * W, diW = -0.5f * r.dv2 * W;
+    const float e = fmaf(W, 1.f + (qb - m1), -1.f);
+    float z, dz;
+    if (e >= c.eps_min) {
+        const float de = 0.5f * r.dv2 * W * W * W * (1.f + (qb - m1)) + W * r.dqm;
+        z = fmaf(c.g1 * e, iW, 1.f + qb);
+        dz = dqb + c.g1 * (de * iW + e * diW);
+    } else {
+        const float h = 1.f + (1.f + c.g1) * c.eps_min;
+        z = fmaf(h, iW, m1);
+        dz = fmaf(h, diW, dm1);
+    }
+    r.g = fmaf(mu, z, -1.f);
+    r.dg = fmaf(mu, dz, z);
+    return r;
 }
 
-// Primitive recovery at one point: safeguarded Newton-Raphson on the master function,
-// bracket [0, 1] (h >= 1), started from the previous primitives.  Returns 1 on success
-// without floor, 0 if eps was floored or the iteration did not converge.
-__device__ int con2prim_point(double D, const double S_d[3], double tau, const double B_u[3],
-                              const double g[3][3], const double gi[3][3], double gam,
-                              double eps_min, int maxit, double tol, double guess_mu,
-                              double* rho, double v_u[3], double* eps, double* pr, double* Wout) {
-    double S_u[3];
-    for (int i = 0; i < 3; i++) S_u[i] = gi[i][0] * S_d[0] + gi[i][1] * S_d[1] + gi[i][2] * S_d[2];
-    double iD = 1.0 / D;
-    double S2 = S_d[0] * S_u[0] + S_d[1] * S_u[1] + S_d[2] * S_u[2];
-    double B2 = 0.0;
-    for (int i = 0; i < 3; i++)
-        for (int j = 0; j < 3; j++) B2 += g[i][j] * B_u[i] * B_u[j];
-    double SB = S_d[0] * B_u[0] + S_d[1] * B_u[1] + S_d[2] * B_u[2];
-    C2PScal c;
-    c.D = D;
-    c.q = tau * iD;
-    c.r2 = S2 * iD * iD;
-    c.bb = B2 * iD;
-    c.rb2 = SB * SB * iD * iD * iD;
-    c.gam = gam;
-    c.eps_min = eps_min;
-    c.v2max = c.r2 / (1.0 + c.r2);
+// g in FP64 and the quantities that the primitives are made of
+struct Master64 {
+    double g, x, v2, m1, q2;     // q2 = (mu x)^2
+};
+__device__ __forceinline__ Master64 master64(double mu, const C2PScal<double>& c) {
+    Master64 r;
+    r.x = rcp64(fma(mu, c.bb, 1.0));
+    const double mx = mu * r.x, u = mx * c.rb2;
+    r.q2 = mx * mx;
+    r.m1 = mu * fma(r.x, c.r2 * r.x, fma(u, r.x, u));
+    const double zb = fma(-c.c1, r.q2, 1.0 + c.c0);
+    const double v2 = mu * r.m1;
+    r.v2 = v2 <= c.v2max ? v2 : c.v2max;
+    const double om = 1.0 - r.v2, W = rsqrt64(om), iW = om * W;
+    const double e = fma(W, zb - r.m1, -1.0);
+    const double z = e >= c.eps_min ? fma(c.g1 * e, iW, zb) : fma(fma(1.0 + c.g1, c.eps_min, 1.0), iW, r.m1);
+    r.g = fma(mu, z, -1.0);
+    return r;
+}
 
-    double lo = 0.0, hi = 1.0;
-    int ok = 1;
-    double mu = (guess_mu > 0.0 && guess_mu < 1.0) ? guess_mu : 0.5;
+// Primitive recovery at one point: the root of g in the bracket [0, 1] (h >= 1).  FP32 finds
+// it to FP32's accuracy from the guess (its pipe is idle: 64 FP32 instructions issue in the
+// time of one FP64 instruction); then Newton steps with the residual in FP64 and the slope in
+// FP32, so that each step leaves about 1e-6 of the last one's error: two FP64 evaluations
+// of 27 instructions in place of three or four of ~110 with the derivative carried in
+// FP64.  Safeguarded by bisection throughout.  Returns 1 on success without floor, 0 if
+// eps was floored or the iteration did not converge; *mu_o, *x_o, *W_o, *iW_o, *eps_o
+// (floored) at the root.
+__device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit, double tol, float guess,
+                                             double* mu_o, double* x_o, double* W_o, double* iW_o, double* eps_o) {
+    const C2PScal<float> cf = {d2f_rn(c.r2), d2f_rn(c.bb), d2f_rn(c.rb2),     d2f_rn(c.c0),
+                               d2f_rn(c.c1), d2f_rn(c.g1), d2f_rn(c.eps_min), d2f_rn(c.v2max)};
+    float m = (guess > 0.f && guess < 1.f) ? guess : 0.5f;
+    {
+        // until the step is within a few units of FP32's noise; else the iterate of least |g|
+        float lo = 0.f, hi = 1.f, best = m, gbest = 3e38f;
+        for (int it = 0; it < 12; it++) {
+            const Master32 f = master32(m, cf);
+            if (fabsf(f.g) < gbest) { gbest = fabsf(f.g); best = m; }
+            const float mn = m - __fdividef(f.g, f.dg);
+            if (fabsf(mn - m) <= 4e-6f * m) {
+                best = mn;
+                break;
+            }
+            if (f.g < 0.f) lo = m; else hi = m;
+            m = (mn > lo && mn < hi) ? mn : 0.5f * (lo + hi);
+        }
+        m = best;
+    }
+    double lo = 0.0, hi = 1.0, mu = f2d(fminf(m, 1.f)), delta = 0.0;
+    float dprev = 0.f;
     int conv = 0;
+    Master64 f;
+    Master32 s;
+    const float tolf = (float)tol;
     // f(0+) < 0 and f(1) >= 0 for every admissible state (h >= 1); a state without a root
-    // never converges and is flagged below.  Stop when the Newton step is below tol, or
-    // when two consecutive Newton steps d_{k-1} > d_k (d_k <= 1e-3 mu) predict the next one,
-    // (d_k / d_{k-1}^2) d_k^2 for quadratic convergence, below tol / 100.
-    double dprev = 0.0;
-    for (int it = 0; it < maxit; it++) {
-        Dual f = master<Dual>(mk(mu, 1.0), c, nullptr, nullptr, nullptr);
-        if (f.v == 0.0) { conv = 1; break; }
-        if (f.v < 0.0) lo = mu; else hi = mu;
-        double mn = mu - f.v / f.d;
-        bool newton = true;
-        if (!(mn > lo && mn < hi)) { mn = 0.5 * (lo + hi); newton = false; }
-        const double dk = fabs(mn - mu);
-        if (dk <= tol * mn) { mu = mn; conv = 1; break; }
-        if (newton && dprev > dk && dk <= 1e-3 * mn && (dk / (dprev * dprev)) * dk * dk <= 0.01 * tol * mn) {
-            mu = mn;
+    // never converges and is flagged below.  Stop when the Newton step is below tol, or when
+    // two consecutive steps d_{k-1} > d_k predict the next one, d_k (d_k / d_{k-1}) for linear
+    // convergence, below tol / 100, or when a step of rounding size leaves the bracket.  The
+    // limit counts the FP64 evaluations after the first two.
+    for (int it = 0;; it++) {
+        f = master64(mu, c);
+        s = master32(d2f_rn(mu), cf);
+        delta = 0.0;
+        if (f.g == 0.0) { conv = 1; break; }
+        if (it >= maxit + 1) break;
+        if (f.g < 0.0) lo = mu; else hi = mu;
+        double mn = fma(-f.g, f2d(__fdividef(1.f, s.dg)), mu);
+        const bool newton = mn > lo && mn < hi;
+        if (!newton) {
+            if (fabsf(d2f_rn(mn - mu)) <= 4e-15f * d2f_rn(mu)) { conv = 1; break; }
+            mn = 0.5 * (lo + hi);
+        }
+        delta = mn - mu;
+        const float dk = fabsf(d2f_rn(delta)), mf = d2f_rn(mn);
+        if (dk <= tolf * mf) { conv = 1; break; }
+        if (newton && dprev > dk && dk <= 1e-3f * mf && __fdividef(dk, dprev) * dk <= 0.01f * tolf * mf) {
             conv = 1;
             break;
         }
-        dprev = newton ? dk : 0.0;
+        dprev = newton ? dk : 0.f;
         mu = mn;
-        if (hi - lo <= tol * hi) { conv = 1; break; }
+        if (hi - lo <= tol * hi) {
+            conv = 1;
+            f = master64(mu, c);
+            delta = 0.0;
+            break;
+        }
     }
-    if (!conv) ok = 0;
-    double W, e, x;
-    master<double>(mu, c, &W, &e, &x);
-    *Wout = W;
-    *rho = D / W;
-    if (!(e >= eps_min)) ok = 0;
-    e = fmax(e, eps_min);
-    *eps = e;
-    *pr = (gam - 1.0) * (*rho) * e;
-    // v_i = mu x (S_i/D + mu (S.B) B_i / D^2)
-    double B_d[3];
-    for (int i = 0; i < 3; i++) B_d[i] = g[i][0] * B_u[0] + g[i][1] * B_u[1] + g[i][2] * B_u[2];
-    double v_d[3];
-    double fac = mu * SB * iD * iD;
-    for (int i = 0; i < 3; i++) v_d[i] = mu * x * (S_d[i] * iD + fac * B_d[i]);
-    for (int i = 0; i < 3; i++) v_u[i] = gi[i][0] * v_d[0] + gi[i][1] * v_d[1] + gi[i][2] * v_d[2];
-    return ok;
+    double qm = fma(-c.c1, f.q2, c.c0) - f.m1;    // qbar - mu rbar^2
+    if (delta != 0.0) {
+        // the last step is not evaluated any more: to first order, or, where tol let it be
+        // large, after all
+        mu += delta;
+        if (fabs(delta) > 1e-9 * mu) {
+            f = master64(mu, c);
+            qm = fma(-c.c1, f.q2, c.c0) - f.m1;
+        } else {
+            f.x = fma(f2d(s.dx), delta, f.x);
+            f.v2 = fma(f2d(s.dv2), delta, f.v2);
+            qm = fma(f2d(s.dqm), delta, qm);
+        }
+    }
+    const double om = 1.0 - f.v2, W = rsqrt64(om);
+    // eps without the cancellation of W (1 + qm) - 1: W - 1 = W^2 v^2 / (1 + W)
+    const double e = fma(W, qm, f.v2 * W * W * rcp64(1.0 + W));
+    *mu_o = mu;
+    *x_o = f.x;
+    *W_o = W;
+    *iW_o = om * W;
+    *eps_o = fmax(e, c.eps_min);
+    return conv && e >= c.eps_min;
 }
 
 // The paper's primitive recovery (Methods, "The Primitive Variable Recovery") as an option
@@ -301,18 +326,13 @@ __device__ int con2prim_damped_point(double D, const double S_d[3], double tau, 
 // that the FP64 pipe bounds.  mat (densitized): E, S_i, E + S, S^ij, Z v_i v_j - b_i b_j (the
 // right-hand side needs S_ij only up to multiples of gamma_ij; S = E - rho (1 + eps) + 3 p).
 __device__ __forceinline__ void fluxes64(long long p, long long P, double alpha, const double beta[3],
-                                         const double g[3][3], const double gi[3][3], double e4, double sqg,
-                                         double rho, const double v[3], double eps, double pr, double W,
-                                         const double B[3], const double* __restrict__ U, double* __restrict__ flux,
-                                         double* __restrict__ mat) {
-    double v_d[3], B_d[3], b_u[3], b_d[3], vt[3];
-    for (int i = 0; i < 3; i++) {
-        v_d[i] = g[i][0] * v[0] + g[i][1] * v[1] + g[i][2] * v[2];
-        B_d[i] = g[i][0] * B[0] + g[i][1] * B[1] + g[i][2] * B[2];
-    }
-    const double iW = 1.0 / W;
+                                         const double gti[6], double e4m, double sqg, double rho, const double v[3],
+                                         const double v_d[3], double eps, double pr, double W, double iW,
+                                         const double B[3], const double B_d[3], double B2, const double Bs[3],
+                                         double* __restrict__ flux, double* __restrict__ mat) {
+    double b_u[3], b_d[3], vt[3];
     const double vB = v_d[0] * B[0] + v_d[1] * B[1] + v_d[2] * B[2], WvB = W * vB;
-    const double b2 = (B_d[0] * B[0] + B_d[1] * B[1] + B_d[2] * B[2]) * (iW * iW) + vB * vB;
+    const double b2 = B2 * (iW * iW) + vB * vB;
     for (int i = 0; i < 3; i++) {
         b_u[i] = B[i] * iW + WvB * v[i];
         b_d[i] = B_d[i] * iW + WvB * v_d[i];
@@ -321,12 +341,11 @@ __device__ __forceinline__ void fluxes64(long long p, long long P, double alpha,
     const double r1 = rho + rho * eps, ps = pr + 0.5 * b2;
     const double Z = (r1 + pr + b2) * (W * W);
     const double D = sqg * (rho * W), E = sqg * (Z - ps - WvB * WvB), tau = E - D;
-    const double sZ = sqg * Z, aps = alpha * (sqg * ps), sW = sqg * WvB;
-    double S[3], Bw[3], Bs[3];
+    const double sZ = sqg * Z, sp = sqg * ps, aps = alpha * sp, sW = sqg * WvB;
+    double S[3], Bw[3];
     const double aw = alpha * iW;
     for (int i = 0; i < 3; i++) {
         S[i] = sZ * v_d[i] - sW * b_d[i];
-        Bs[i] = U[(V_B + i) * P + p];
         Bw[i] = aw * Bs[i];
     }
     for (int i = 0; i < 3; i++) {
@@ -348,7 +367,7 @@ __device__ __forceinline__ void fluxes64(long long p, long long P, double alpha,
     mat[0 * P + p] = E;
     for (int i = 0; i < 3; i++) mat[(1 + i) * P + p] = S[i];
     mat[4 * P + p] = 2.0 * E - sqg * (r1 - 3.0 * pr);
-    const double sp = sqg * ps;
+    const double spe = sp * e4m;
     double zv[3], zd[3], sb[3], sd[3];
     for (int i = 0; i < 3; i++) {
         zv[i] = sZ * v[i];
@@ -358,13 +377,21 @@ __device__ __forceinline__ void fluxes64(long long p, long long P, double alpha,
     }
     for (int i = 0; i < 3; i++)
         for (int j = i; j < 3; j++) {
-            mat[(5 + SI(i, j)) * P + p] = zv[i] * v[j] + (sp * gi[i][j] - sb[i] * b_u[j]);
+            mat[(5 + SI(i, j)) * P + p] = zv[i] * v[j] + (spe * gti[SI(i, j)] - sb[i] * b_u[j]);
             mat[(11 + SI(i, j)) * P + p] = zd[i] * v_d[j] - sd[i] * b_d[j];
         }
 }
 
-template <typename R>
-__global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const double* __restrict__ U,
+// What a launch computes: the primitives alone, or also the fluxes and matter terms in FP64
+// or FP32.  Bound by the FP64 pipe (87 % busy): 346 FP64 instructions per node against 707
+// in FP64, so the launch inside the stepping of 393,216 nodes went from 545 to 283 us (ncu),
+// the FP32 form from 340 to 234 us, the recovery of a newly loaded state (grmhd_con2prim,
+// whole call) from 807 to 247 us.  Three blocks per SM (168 registers) hide the serial
+// chains of the root finding better than two of 182 registers do.
+enum { PREP_PRIM = 0, PREP_F64 = 1, PREP_F32 = 2 };
+
+template <int WHAT>
+__global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const double* __restrict__ U,
                                               double* __restrict__ prim, double* __restrict__ flux,
                                               double* __restrict__ tmn, double* __restrict__ lam,
                                               unsigned long long* __restrict__ nfail, double* __restrict__ met) {
@@ -375,67 +402,101 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
         // gamma = e^{4phi} gammatilde, gamma^-1 = e^{-4phi} gammatilde^-1, det gamma =
         // e^{12phi} det gammatilde, computed as the right-hand side uses them and kept in met
         // (e^{4phi}, e^{-4phi}, sqrt(gamma), gammatilde^ij) so that k_rhs reads them: GB300's
-        // FP64 pipe bounds both kernels, and the exponential, the cofactor inverse with its
-        // division and the square root are ~75 FP64 instructions per node
+        // FP64 pipe bounds both kernels
         const double e4 = exp(4.0 * U[V_PHI * P + p]);
-        const double e4m = 1.0 / e4;
-        double gt[3][3], gti[3][3], g[3][3], gi[3][3];
-        for (int i = 0; i < 3; i++)
-            for (int j = i; j < 3; j++) gt[i][j] = gt[j][i] = U[(V_GT + SI(i, j)) * P + p];
-        const double detgt = inv3sym(gt, gti);
-        for (int i = 0; i < 3; i++)
-            for (int j = 0; j < 3; j++) {
-                g[i][j] = e4 * gt[i][j];
-                gi[i][j] = e4m * gti[i][j];
-            }
-        const double sqg = sqrt(e4 * e4 * e4 * detgt);
-        double isq = 1.0 / sqg;
-        met[0 * P + p] = e4;
-        met[1 * P + p] = e4m;
-        met[2 * P + p] = sqg;
-        for (int i = 0; i < 3; i++)
-            for (int j = i; j < 3; j++) met[(3 + SI(i, j)) * P + p] = gti[i][j];
-        double alpha = U[V_ALPHA * P + p];
-        double beta[3] = {U[V_BETA * P + p], U[(V_BETA + 1) * P + p], U[(V_BETA + 2) * P + p]};
-        double Dc = U[V_D * P + p] * isq;
-        double S_d[3], B_u[3];
+        const double e4m = rcp64(e4);
+        double gt[6], gti[6];
+        for (int q = 0; q < 6; q++) gt[q] = U[(V_GT + q) * P + p];
+        const double c00 = gt[3] * gt[5] - gt[4] * gt[4], c01 = gt[2] * gt[4] - gt[1] * gt[5],
+                     c02 = gt[1] * gt[4] - gt[2] * gt[3];
+        const double detgt = gt[0] * c00 + gt[1] * c01 + gt[2] * c02;
+        const double id = rcp64(detgt);
+        gti[0] = c00 * id; gti[1] = c01 * id; gti[2] = c02 * id;
+        gti[3] = (gt[0] * gt[5] - gt[2] * gt[2]) * id;
+        gti[4] = (gt[1] * gt[2] - gt[0] * gt[4]) * id;
+        gti[5] = (gt[0] * gt[3] - gt[1] * gt[1]) * id;
+        const double detg = e4 * e4 * e4 * detgt;
+        const double isq = rsqrt64(detg), sqg = detg * isq;
+        double Us[3], Bs[3], B_u[3], B_d[3];
+        const double Ud = U[V_D * P + p], Ut = U[V_TAU * P + p];
         for (int i = 0; i < 3; i++) {
-            S_d[i] = U[(V_S + i) * P + p] * isq;
-            B_u[i] = U[(V_B + i) * P + p] * isq;
+            Us[i] = U[(V_S + i) * P + p];
+            Bs[i] = U[(V_B + i) * P + p];
+            B_u[i] = Bs[i] * isq;
         }
-        double tau = U[V_TAU * P + p] * isq;
+        for (int i = 0; i < 3; i++)
+            B_d[i] = e4 * (gt[SI(i, 0)] * B_u[0] + gt[SI(i, 1)] * B_u[1] + gt[SI(i, 2)] * B_u[2]);
+        const double B2 = B_d[0] * B_u[0] + B_d[1] * B_u[1] + B_d[2] * B_u[2];
+        const double Dc = Ud * isq, tau = Ut * isq;
 
-        // guess mu = 1/(h W) from the stored primitives
-        double Wg = prim[6 * P + p], eg = prim[4 * P + p];
-        double mu0 = 1.0 / ((1.0 + pp.gam * eg) * Wg);
-        double rho, v[3], eps, pr, W;
+        double rho, v[3], v_d[3], eps, pr, W, iW;
         int ok;
-        if (Dc > pp.rho_atm && isfinite(Dc) && isfinite(tau) && pp.c2p_lambda > 0.0) {
-            // the paper's damped iteration from the stored primitives, or (after a reset)
-            // from the dust estimates v^i = gamma^ij S_j / (tau + D), eps = (tau + D)/(D W) - 1
-            if (Wg >= 1.0 && prim[0 * P + p] > 0.0) {
-                rho = prim[0 * P + p];
-                for (int i = 0; i < 3; i++) v[i] = prim[(1 + i) * P + p];
-                eps = eg;
-            } else {
-                const double ie = 1.0 / (tau + Dc);
-                for (int i = 0; i < 3; i++)
-                    v[i] = (gi[i][0] * S_d[0] + gi[i][1] * S_d[1] + gi[i][2] * S_d[2]) * ie;
-                eps = 0.0;
-                damped_clamp(v, &eps, g, 1.0 - 1.0 / (10.0 * 10.0), 0.0);
-                const double W0 = lorentz_w(v, g);
-                eps = fmax((tau + Dc) / (Dc * W0) - 1.0, pp.eps_atm);
-                rho = Dc / W0;
+        const bool gas = Dc > pp.rho_atm && isfinite(Dc) && isfinite(tau);
+        if (gas && !(pp.c2p_lambda > 0.0)) {
+            // ratios to D straight from the densitized variables
+            const double iU = rcp64(Ud), iD = iU * sqg;
+            double s[3], su[3];
+            for (int i = 0; i < 3; i++) s[i] = Us[i] * iU;
+            for (int i = 0; i < 3; i++)
+                su[i] = e4m * (gti[SI(i, 0)] * s[0] + gti[SI(i, 1)] * s[1] + gti[SI(i, 2)] * s[2]);
+            const double sB = s[0] * B_u[0] + s[1] * B_u[1] + s[2] * B_u[2];
+            C2PScal<double> c;
+            c.r2 = s[0] * su[0] + s[1] * su[1] + s[2] * su[2];
+            c.bb = B2 * iD;
+            c.rb2 = sB * sB * iD;
+            c.c0 = Ut * iU - 0.5 * c.bb;
+            c.c1 = 0.5 * (c.bb * c.r2 - c.rb2);
+            c.g1 = pp.gam - 1.0;
+            c.eps_min = pp.eps_atm;
+            c.v2max = c.r2 * rcp64(1.0 + c.r2);
+            // guess mu = 1/(h W) from the stored primitives
+            const float guess = __fdividef(1.f, (1.f + (float)pp.gam * d2f_rn(prim[4 * P + p])) * d2f_rn(prim[6 * P + p]));
+            double mu, x;
+            ok = con2prim_root(c, pp.c2p_maxit, pp.c2p_tol, guess, &mu, &x, &W, &iW, &eps);
+            rho = Dc * iW;
+            pr = c.g1 * rho * eps;
+            // v_i = mu x (S_i/D + mu (S.B) B_i / D^2)
+            const double mx = mu * x, fac = mu * (sB * iD);
+            for (int i = 0; i < 3; i++) {
+                v_d[i] = mx * (s[i] + fac * B_d[i]);
+                v[i] = mx * (su[i] + fac * B_u[i]);
             }
-            ok = con2prim_damped_point(Dc, S_d, tau, B_u, g, gi, pp.gam, pp.eps_atm, pp.c2p_maxit, pp.c2p_tol,
-                                       pp.c2p_lambda, &rho, v, &eps, &pr, &W);
-        } else if (Dc > pp.rho_atm && isfinite(Dc) && isfinite(tau)) {
-            ok = con2prim_point(Dc, S_d, tau, B_u, g, gi, pp.gam, pp.eps_atm, pp.c2p_maxit,
-                                pp.c2p_tol, mu0, &rho, v, &eps, &pr, &W);
         } else {
-            ok = 0;
-            rho = pp.rho_atm; v[0] = v[1] = v[2] = 0.0; eps = pp.eps_atm;
-            pr = (pp.gam - 1.0) * rho * eps; W = 1.0;
+            double g[3][3];
+            for (int i = 0; i < 3; i++)
+                for (int j = 0; j < 3; j++) g[i][j] = e4 * gt[SI(i, j)];
+            if (gas) {
+                double gi[3][3], S_d[3];
+                for (int i = 0; i < 3; i++) {
+                    S_d[i] = Us[i] * isq;
+                    for (int j = 0; j < 3; j++) gi[i][j] = e4m * gti[SI(i, j)];
+                }
+                // the paper's damped iteration from the stored primitives, or (after a reset)
+                // from the dust estimates v^i = gamma^ij S_j / (tau + D), eps = (tau + D)/(D W) - 1
+                const double Wg = prim[6 * P + p];
+                if (Wg >= 1.0 && prim[0 * P + p] > 0.0) {
+                    rho = prim[0 * P + p];
+                    for (int i = 0; i < 3; i++) v[i] = prim[(1 + i) * P + p];
+                    eps = prim[4 * P + p];
+                } else {
+                    const double ie = 1.0 / (tau + Dc);
+                    for (int i = 0; i < 3; i++)
+                        v[i] = (gi[i][0] * S_d[0] + gi[i][1] * S_d[1] + gi[i][2] * S_d[2]) * ie;
+                    eps = 0.0;
+                    damped_clamp(v, &eps, g, 1.0 - 1.0 / (10.0 * 10.0), 0.0);
+                    const double W0 = lorentz_w(v, g);
+                    eps = fmax((tau + Dc) / (Dc * W0) - 1.0, pp.eps_atm);
+                    rho = Dc / W0;
+                }
+                ok = con2prim_damped_point(Dc, S_d, tau, B_u, g, gi, pp.gam, pp.eps_atm, pp.c2p_maxit, pp.c2p_tol,
+                                           pp.c2p_lambda, &rho, v, &eps, &pr, &W);
+            } else {
+                ok = 0;
+                rho = pp.rho_atm; v[0] = v[1] = v[2] = 0.0; eps = pp.eps_atm;
+                pr = (pp.gam - 1.0) * rho * eps; W = 1.0;
+            }
+            iW = 1.0 / W;
+            for (int i = 0; i < 3; i++) v_d[i] = g[i][0] * v[0] + g[i][1] * v[1] + g[i][2] * v[2];
         }
         bad = !ok;
         prim[0 * P + p] = rho;
@@ -446,10 +507,27 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
         prim[5 * P + p] = pr;
         prim[6 * P + p] = W;
 
-        if constexpr (sizeof(R) == 8) {
-            fluxes64(p, P, alpha, beta, g, gi, e4, sqg, rho, v, eps, pr, W, B_u, U, flux, tmn);
+        if constexpr (WHAT != PREP_PRIM) {
+        met[0 * P + p] = e4;
+        met[1 * P + p] = e4m;
+        met[2 * P + p] = sqg;
+        for (int q = 0; q < 6; q++) met[(3 + q) * P + p] = gti[q];
+        const double alpha = U[V_ALPHA * P + p];
+        const double beta[3] = {U[V_BETA * P + p], U[(V_BETA + 1) * P + p], U[(V_BETA + 2) * P + p]};
+        // the light-cone speed is read at the element ends (interface penalty) only
+        const uint32_t ir = ((uint32_t)p / (uint32_t)d.NtNp) % (uint32_t)d.Nr;
+        if (ir == 0 || ir == (uint32_t)d.Nr - 1) lam[p] = fabs(beta[0]) + alpha * sqrt(e4m * gti[0]);
+        if constexpr (WHAT == PREP_F64) {
             met[9 * P + p] = isq;
+            fluxes64(p, P, alpha, beta, gti, e4m, sqg, rho, v, v_d, eps, pr, W, iW, B_u, B_d, B2, Bs, flux, tmn);
         } else {
+        using R = float;
+        double g[3][3], gi[3][3];
+        for (int i = 0; i < 3; i++)
+            for (int j = 0; j < 3; j++) {
+                g[i][j] = e4 * gt[SI(i, j)];
+                gi[i][j] = e4m * gti[SI(i, j)];
+            }
         // ---- four-vectors, fluxes and T^{mu nu} of the mixed modes in FP32 (their consumers,
         // the tensor-core contractions and the FP32 right-hand side, keep about 24 bits); the
         // primitive recovery above stays FP64
@@ -461,13 +539,13 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
             BR[i] = narrow<R>(B_u[i]);
             for (int j = 0; j < 3; j++) gR[i][j] = narrow<R>(g[i][j]);
         }
-        R v_d[3];
-        for (int i = 0; i < 3; i++) v_d[i] = gR[i][0] * vR[0] + gR[i][1] * vR[1] + gR[i][2] * vR[2];
+        R vR_d[3];
+        for (int i = 0; i < 3; i++) vR_d[i] = gR[i][0] * vR[0] + gR[i][1] * vR[1] + gR[i][2] * vR[2];
         R ia = R(1.0) / alphaR;
         R u0 = WR * ia;
         R uu[3];
         for (int i = 0; i < 3; i++) uu[i] = WR * (vR[i] - betaR[i] * ia);
-        R b0 = WR * (v_d[0] * BR[0] + v_d[1] * BR[1] + v_d[2] * BR[2]) * ia;
+        R b0 = WR * (vR_d[0] * BR[0] + vR_d[1] * BR[1] + vR_d[2] * BR[2]) * ia;
         R iW = R(1.0) / WR;
         R bu[3];
         for (int i = 0; i < 3; i++) bu[i] = (BR[i] + alphaR * b0 * uu[i]) * iW;
@@ -487,12 +565,12 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
         // conserved variables from the primitives (undensitized)
         R Dp = rhoR * WR;
         R Sp[3];
-        for (int j = 0; j < 3; j++) Sp[j] = rhohs * WR * WR * v_d[j] - alphaR * b0 * bd[j];
+        for (int j = 0; j < 3; j++) Sp[j] = rhohs * WR * WR * vR_d[j] - alphaR * b0 * bd[j];
         // tau = rho h* W^2 - p* - alpha^2 b0^2 - D without its cancellation: with
         // W^2 - 1 = W^2 v^2 and W - 1 = W^2 v^2 / (W + 1),
         // tau = rho W (eps W + W^2 v^2 / (W + 1)) + p W^2 v^2 + b^2 (W^2 - 1/2) - alpha^2 b0^2
         // (tau ~ 1e-3 D for a cold gas: the direct form loses 3 digits, all of FP32's margin)
-        const R Wv2 = WR * WR * (v_d[0] * vR[0] + v_d[1] * vR[1] + v_d[2] * vR[2]);
+        const R Wv2 = WR * WR * (vR_d[0] * vR[0] + vR_d[1] * vR[1] + vR_d[2] * vR[2]);
         const R taup = rhoR * WR * (epsR * WR + Wv2 / (WR + R(1.0))) + prR * Wv2 + b2 * (WR * WR - R(0.5)) -
                        alphaR * alphaR * b0 * b0;
         // ---- densitized fluxes [dir][var]
@@ -522,7 +600,7 @@ __global__ void __launch_bounds__(128) k_prep(Dims d, PhysParams pp, const doubl
             for (int k = m; k < 4; k++, n++)
                 tmn[n * P + p] = widen(rhohs * u4[m] * u4[k] + pstar * gu[m][k] - b4[m] * b4[k]);
         }
-        lam[p] = fabs(beta[0]) + alpha * sqrt(gi[0][0]);
+        }
     }
     // warp-aggregated failure count
     unsigned m = __ballot_sync(0xffffffffu, bad);
@@ -1423,8 +1501,16 @@ cudaError_t launch_prep(const Dims& d, const PhysParams& pp, const double* U, do
                         cudaStream_t s, int fp32_algebra) {
     int bs = 128;
     long long nb = (d.P + bs - 1) / bs;
-    if (fp32_algebra) k_prep<float><<<(unsigned)nb, bs, 0, s>>>(d, pp, U, prim, flux, tmn, lam, nfail, met);
-    else k_prep<double><<<(unsigned)nb, bs, 0, s>>>(d, pp, U, prim, flux, tmn, lam, nfail, met);
+    if (fp32_algebra) k_prep<PREP_F32><<<(unsigned)nb, bs, 0, s>>>(d, pp, U, prim, flux, tmn, lam, nfail, met);
+    else k_prep<PREP_F64><<<(unsigned)nb, bs, 0, s>>>(d, pp, U, prim, flux, tmn, lam, nfail, met);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_con2prim(const Dims& d, const PhysParams& pp, const double* U, double* prim,
+                            unsigned long long* nfail, cudaStream_t s) {
+    int bs = 128;
+    long long nb = (d.P + bs - 1) / bs;
+    k_prep<PREP_PRIM><<<(unsigned)nb, bs, 0, s>>>(d, pp, U, prim, nullptr, nullptr, nullptr, nfail, nullptr);
     return cudaGetLastError();
 }
 
