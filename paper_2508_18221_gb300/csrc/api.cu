@@ -4,7 +4,7 @@
 // streams joined before the right-hand side:
 //   side stream: deriv r, theta, phi (first derivatives of 21 BSSN fields) | interface mean
 //                of d_r | deriv r, theta, phi (second derivatives of 11 fields) | interface
-//                mean of d_rr
+//                mean of d_rr  (small grids: the three directions in one launch)
 //   main stream: prep | deriv r, theta, phi (flux divergence) | (join) | rhs (+ RK stage
 //                combination)
 // A time step adds the filter (3 directional contractions + interface mean of the BSSN
@@ -33,6 +33,12 @@ struct NvtxRange {
     explicit NvtxRange(const char* name) { nvtxRangePushA(name); }
     ~NvtxRange() { nvtxRangePop(); }
 };
+
+// nodes x (N_r + N_theta + N_phi) up to which a grid's contractions run on the integer units.
+// A time step in us, integer units / tensor cores: 4,608 nodes (2 x 12 x 12 x 16) 224 / 351,
+// 18,432 (8 x 12 x 12 x 16) 318 / 461, 36,864 (2 x 24 x 24 x 32: 2.9e6) 615 / 662, 32,768
+// (1 x 32 x 32 x 32: 3.1e6) 594 / 590, 65,536 (8 x 16 x 16 x 32: 4.2e6) 1,046 / 1,032
+static const long long FXS_MAX_WORK = 3000000;
 
 struct grmhd_ctx {
     grmhd_grid grid;
@@ -113,6 +119,14 @@ struct grmhd_ctx {
     uint8_t* fx_dt[2];       // digit-slice images (nullptr: FP64 units)
     uint8_t* fx_ft[2];
     uint8_t* tc_t[2];        // mixed-precision images of the derivative operators
+    // small grids: the digit-slice contractions of every direction in one launch on the integer
+    // units (kernels_fxs.cu), derivatives (FP64 mode) and filter
+    int small_d, small_f;
+    uint8_t* fxs_d[4];       // images: r (one per element), theta or even extension, phi, odd extension
+    uint8_t* fxs_f[4];
+    long long fxs_estride;
+    FxsJob* sjobs;
+    int sj_first[3], sj_flux[3], sj_second, sj_filter[3][3][2];
     FoldJob* fjobs;          // fold / unfold job lists (offsets below)
     int fj_first[3], fj_first_u[3], fj_second, fj_second_u, fj_filter[3][2], fj_filter_u[3][2];
     int fj_dbg, fj_dbg_u;
@@ -276,6 +290,11 @@ static void free_ctx(grmhd_ctx* c) {
         if (c->tc_t[k]) cudaFree(c->tc_t[k]);
     }
     if (c->fjobs) cudaFree(c->fjobs);
+    for (int k = 0; k < 4; k++) {
+        if (c->fxs_d[k]) cudaFree(c->fxs_d[k]);
+        if (c->fxs_f[k]) cudaFree(c->fxs_f[k]);
+    }
+    if (c->sjobs) cudaFree(c->sjobs);
     if (c->s2) cudaStreamDestroy(c->s2);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);
@@ -458,6 +477,14 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
             }
         }
 
+    // small grids take the one-launch contractions: where a launch of the tensor-core kernel,
+    // 10-15 us however small, costs more than the products on the integer units.  The bits
+    // are the same, so an instance evolves alike alone and in a batch
+    c->small_f = P * (Nr + Nt + Np) <= FXS_MAX_WORK && opts->contraction == 0 && fxs_supported(Nr) && fxs_supported(Nt) &&
+                 fxs_supported(Np) && (!c->ft || (Np / 2) % 2 == 0);
+    c->small_d = c->small_f && opts->precision == 0;
+    const int ndiv = c->small_d ? 3 : 1;
+
     // device memory
     cudaError_t ce = cudaSuccess;
 #define AL(ptr, n) if (ce == cudaSuccess) ce = dalloc(&(ptr), (size_t)(n))
@@ -470,7 +497,7 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
     AL(c->d1, (N_D1 + glm) * 3 * P);
     if (glm) AL(c->divB, P);
     AL(c->d2, N_D2 * 6 * P);
-    AL(c->divF, 8 * P);
+    AL(c->divF, ndiv * 8 * P);
     AL(c->ham, P);
     AL(c->met, N_MET * P);
     AL(c->scratch, nv * P);
@@ -528,13 +555,28 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
     for (int s = 0; s < N_D2; s++)
         add(c->d1 + ((long long)vars2[s] * 3 + 2) * P, c->d2 + ((long long)s * 6 + 5) * P, 0);
     c->job_second_n[2] = N_D2;
-    // filter chains: r: U[b] -> scratch; theta: scratch -> U[b]; phi: U[b] -> U[0]
+    // filter: a group's active directions in turn, the last one into U[0]; with three, r:
+    // U[b] -> scratch, theta: scratch -> U[b], phi: U[b] -> U[0]; with two, the first goes to
+    // scratch.  (Directions a group is not filtered in keep the three-direction buffers, for
+    // timing.)
+    auto filter_link = [&](int b, int dir, int grp, const double** src, double** dst) {
+        int act = 0, k = 0;
+        for (int q = 0; q < 3; q++) {
+            const int on = (opts->filter >> (3 * grp + q)) & 1;
+            act += on;
+            if (q < dir) k += on;
+        }
+        if (!((opts->filter >> (3 * grp + dir)) & 1)) { act = 3; k = dir; }
+        *src = k == 0 ? c->U[b] : (k == 1 ? c->scratch : c->U[b]);
+        *dst = k == act - 1 ? c->U[0] : (k == 0 ? c->scratch : c->U[b]);
+    };
     for (int b = 0; b < 3; b++)
         for (int dir = 0; dir < 3; dir++)
             for (int grp = 0; grp < 2; grp++) {
                 c->job_filter[b][dir][grp] = (int)jobs.size();
-                const double* src = dir == 0 ? c->U[b] : (dir == 1 ? c->scratch : c->U[b]);
-                double* dst = dir == 0 ? c->scratch : (dir == 1 ? c->U[b] : c->U[0]);
+                const double* src;
+                double* dst;
+                filter_link(b, dir, grp, &src, &dst);
                 int v0 = grp == 0 ? V_D : 0, ng = grp == 0 ? 8 + glm : N_BSSN;
                 for (int v = v0; v < v0 + ng; v++) add(src + (long long)v * P, dst + (long long)v * P, 0);
             }
@@ -781,16 +823,15 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
                 if (mixed) addf(Zf + i * P, reinterpret_cast<float*>(c->d2) + dof, par, 0);
                 else addf(c->Z + i * P, c->d2 + dof, par, 0);
             }
-        // filter, theta link of the chain scratch -> U[b] (FP64 at every precision)
+        // filter, theta link of the chain (FP64 at every precision)
         for (int b = 0; b < 3; b++)
             for (int grp = 0; grp < 2; grp++) {
                 const int v0 = grp == 0 ? V_D : 0, ng = grp == 0 ? 8 + glm : N_BSSN;
                 c->fj_filter[b][grp] = (int)fj.size();
-                for (int i = 0; i < ng; i++)
-                    addf(c->scratch + (long long)(v0 + i) * P, c->Y + (long long)i * P, kThetaParity[v0 + i], 0);
+                const DerivJob* jl = &jobs[c->job_filter[b][1][grp]];
+                for (int i = 0; i < ng; i++) addf(jl[i].src, c->Y + (long long)i * P, kThetaParity[v0 + i], 0);
                 c->fj_filter_u[b][grp] = (int)fj.size();
-                for (int i = 0; i < ng; i++)
-                    addf(c->Z + (long long)i * P, c->U[b] + (long long)(v0 + i) * P, kThetaParity[v0 + i], 0);
+                for (int i = 0; i < ng; i++) addf(c->Z + (long long)i * P, jl[i].dst, kThetaParity[v0 + i], 0);
             }
         // test hook and diagnostics entries, filled per call
         c->fj_dbg = (int)fj.size();
@@ -803,6 +844,74 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
             free_ctx(c);
             return GRMHD_ENOMEM;
         }
+    }
+    // small grids: operator images and job lists of the one-launch contractions
+    if (c->small_f) {
+        const int Ns[3] = {Nr, Nt, Np};
+        std::vector<double> dense_d[3] = {Dr, Dt, circulant(Dp)};
+        std::vector<double> dense_f[3] = {Fr, Ft, circulant(Fp)};
+        auto put = [&](uint8_t** dst, const std::vector<uint8_t>& img) {
+            return cudaMalloc(dst, img.size()) == cudaSuccess &&
+                   cudaMemcpyAsync(*dst, img.data(), img.size(), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+                   cudaStreamSynchronize(s) == cudaSuccess;
+        };
+        bool ok = true;
+        for (int k = 0; k < 3 && ok; k++) {
+            if (k == 1 && c->ft) {
+                for (int h = 0; h < 2 && ok; h++)
+                    ok = put(&c->fxs_d[1 + 2 * h], fxs_operator_image(ext_d[h], Nt, 1.0)) &&
+                         put(&c->fxs_f[1 + 2 * h], fxs_operator_image(ext_f[h], Nt, 1.0));
+                continue;
+            }
+            std::vector<uint8_t> img;
+            for (int e = 0; e < (k == 0 ? E : 1); e++) {
+                const std::vector<uint8_t> one = fxs_operator_image(dense_d[k], Ns[k], k == 0 ? c->rscale_h[e] : 1.0);
+                if (k == 0) c->fxs_estride = (long long)one.size();
+                img.insert(img.end(), one.begin(), one.end());
+            }
+            ok = put(&c->fxs_d[k], img) && put(&c->fxs_f[k], fxs_operator_image(dense_f[k], Ns[k], 1.0));
+        }
+        // the jobs of the lists above, directions one after the other; the flux divergence of a
+        // direction into its own part of divF; the field divergence (GLM), whose interface mean
+        // is taken of the sum, accumulates over three launches
+        std::vector<FxsJob> sj;
+        auto adds = [&](const DerivJob& j, int dir, int par, double* dst = nullptr) {
+            FxsJob x;
+            x.src = j.src; x.dst = dst ? dst : j.dst; x.dir = dir == 1 && c->ft ? 3 : dir; x.parity = par;
+            x.accumulate = dst ? 0 : j.accumulate; x.pad = 0;
+            sj.push_back(x);
+        };
+        const int nB = N_D1 + glm;
+        for (int b = 0; b < 3; b++) {
+            c->sj_first[b] = (int)sj.size();
+            for (int dir = 0; dir < 3; dir++)
+                for (int i = 0; i < nB; i++)
+                    adds(jobs[c->job_first[b][dir] + i], dir, kThetaParity[i < N_D1 ? i : V_PSI]);
+            c->sj_flux[b] = (int)sj.size();
+            for (int dir = 0; dir < 3; dir++)
+                for (int v = 0; v < 8; v++)
+                    adds(jobs[c->job_first[b][dir] + nB + v], dir, -kThetaParity[V_D + v], c->divF + ((long long)dir * 8 + v) * P);
+            for (int dir = 0; dir < 3 && glm; dir++)
+                adds(jobs[c->job_first[b][dir] + nB + 8], dir, kThetaParity[V_B + 1]);
+            for (int dir = 0; dir < 3; dir++)
+                for (int grp = 0; grp < 2; grp++) {
+                    c->sj_filter[b][dir][grp] = (int)sj.size();
+                    const int v0 = grp == 0 ? V_D : 0, ng = grp == 0 ? 8 + glm : N_BSSN;
+                    for (int i = 0; i < ng; i++) adds(jobs[c->job_filter[b][dir][grp] + i], dir, kThetaParity[v0 + i]);
+                }
+        }
+        c->sj_second = (int)sj.size();
+        const int v2[N_D2] = {0, 1, 2, 3, 4, 5, 6, 17, 18, 19, 20};
+        for (int dir = 0; dir < 3; dir++)
+            for (int i = 0; i < c->job_second_n[dir]; i++) {
+                // theta list: theta-theta (of d_theta u, parity -s) and theta-phi (parity s) per field
+                const int par = kThetaParity[v2[dir == 1 ? i / 2 : 0]];
+                adds(jobs[c->job_second[dir] + i], dir, dir == 1 && i % 2 == 0 ? -par : par);
+            }
+        ok = ok && cudaMalloc(&c->sjobs, sj.size() * sizeof(FxsJob)) == cudaSuccess &&
+             cudaMemcpyAsync(c->sjobs, sj.data(), sj.size() * sizeof(FxsJob), cudaMemcpyHostToDevice, s) == cudaSuccess &&
+             cudaStreamSynchronize(s) == cudaSuccess;
+        if (!ok) { free_ctx(c); return GRMHD_ENOMEM; }
     }
     *out = c;
     return GRMHD_OK;
@@ -910,13 +1019,29 @@ static cudaError_t theta_fourier(grmhd_ctx* c, int filter, int stage, int fold_o
     return launch_theta_unfold(c->d, c->fjobs + unfold_off, n, stage >= 0, c->stream);
 }
 
+// The one-launch contraction of a small grid: n jobs of sjobs from offset off
+static cudaError_t small_contract(grmhd_ctx* c, int filter, int off, int n) {
+    FxsOps o;
+    for (int k = 0; k < 4; k++) o.img[k] = filter ? c->fxs_f[k] : c->fxs_d[k];
+    o.estride = filter ? 0 : c->fxs_estride;
+    return launch_contract_small(c->d, c->sjobs + off, n, c->ft ? 13 : 7, o, c->stream);
+}
+
 // First derivatives from buffer b.  part 0: the BSSN fields (+ psi) and their interface
 // means; part 1: the flux divergence (+ the field divergence with GLM), which needs the
 // fluxes of k_prep.
 static int enqueue_first_derivs(grmhd_ctx* c, int b, int part) {
     const int nB = N_D1 + c->pp.glm, off = part == 0 ? 0 : nB, n = part == 0 ? nB : c->job_first_n - nB;
     const int mixed = c->opts.precision > 0, tf32 = c->opts.precision == 2;
-    for (int dir = 0; dir < 3; dir++) {
+    if (c->small_d) {
+        CK(small_contract(c, 0, part == 0 ? c->sj_first[b] : c->sj_flux[b], part == 0 ? 3 * n : 24));
+        c->launches_tmp++;
+        for (int dir = 0; dir < 3 && part == 1 && c->pp.glm; dir++) {
+            CK(small_contract(c, 0, c->sj_flux[b] + 24 + dir, 1));
+            c->launches_tmp++;
+        }
+    }
+    for (int dir = 0; dir < 3 && !c->small_d; dir++) {
         if (dir == 1 && c->ft)
             CK(theta_fourier(c, 0, mixed ? 0 : -1, c->fj_first[b] + off, c->fj_first_u[b] + off, n, off));
         else if (mixed)
@@ -950,20 +1075,23 @@ static int enqueue_second_derivs(grmhd_ctx* c) {
                                       c->r_scale, c->tc_err, c->stream));
             c->launches_tmp++;
         }
-        for (int x = 0; x < 3; x++)
-            CK(launch_iface_avg_f(c->d, reinterpret_cast<float*>(c->d2) + x * c->d.P, 6 * c->d.P, N_D2, c->stream));
-        if (c->d.E > 1) c->launches_tmp += 3;
+        // the three radial results (slots 0 .. 2 of each field) in one launch
+        CK(launch_iface_avg_f(c->d, reinterpret_cast<float*>(c->d2), c->d.P, 3 * N_D2, c->stream, 3, 6 * c->d.P));
+        if (c->d.E > 1) c->launches_tmp++;
         return GRMHD_OK;
     }
-    for (int dir = 0; dir < 3; dir++) {
+    if (c->small_d) {
+        CK(small_contract(c, 0, c->sj_second, 6 * N_D2));
+        c->launches_tmp++;
+    }
+    for (int dir = 0; dir < 3 && !c->small_d; dir++) {
         if (dir == 1 && c->ft)
             CK(theta_fourier(c, 0, -1, c->fj_second, c->fj_second_u, c->job_second_n[dir], c->job_first_n));
         else CK(contract(c, dir, 0, c->jobs + c->job_second[dir], c->job_second_n[dir]));
         c->launches_tmp++;
     }
-    for (int x = 0; x < 3; x++)
-        CK(launch_iface_avg(c->d, c->d2 + x * c->d.P, 6 * c->d.P, N_D2, c->stream));
-    if (c->d.E > 1) c->launches_tmp += 3;
+    CK(launch_iface_avg(c->d, c->d2, c->d.P, 3 * N_D2, c->stream, 3, 6 * c->d.P));
+    if (c->d.E > 1) c->launches_tmp++;
     return GRMHD_OK;
 }
 
@@ -1000,7 +1128,7 @@ static int enqueue_stage(grmhd_ctx* c, int b, RKCoef co, double* out, const Phys
     CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
     CK(launch_rhs(c->d, pp, c->U[0], c->U[b], c->prim, c->flux, c->tmn, c->lam, c->met, c->d1, c->d2,
                   c->divF, c->divB, c->opts.precision > 0, c->r_scale, c->dt, co, out, c->acc, c->stream,
-                  c->ham_out));
+                  c->ham_out, c->small_d ? 3 : 1));
     c->launches_tmp++;
     return GRMHD_OK;
 }
@@ -1009,22 +1137,31 @@ static int enqueue_stage(grmhd_ctx* c, int b, RKCoef co, double* out, const Phys
 static int enqueue_filter(grmhd_ctx* c, int b) {
     const long long P = c->d.P;
     const int m = c->opts.filter;
+    const int n0 = 8 + c->pp.glm;   // the Valencia group carries psi (variable 32, right after them) with GLM
     for (int dir = 0; dir < 3; dir++) {
-        const double* src = dir == 0 ? c->U[b] : (dir == 1 ? c->scratch : c->U[b]);
-        double* dst = dir == 0 ? c->scratch : (dir == 1 ? c->U[b] : c->U[0]);
-        for (int grp = 0; grp < 2; grp++) {
-            int bit = (grp == 0 ? 1 : 8) << dir;
-            // the Valencia group carries psi (variable 32, right after them) with GLM
-            int v0 = grp == 0 ? V_D : 0, ng = grp == 0 ? 8 + c->pp.glm : N_BSSN;
-            if (m & bit) {
-                if (dir == 1 && c->ft) CK(theta_fourier(c, 1, -1, c->fj_filter[b][grp], c->fj_filter_u[b][grp], ng));
-                else CK(contract(c, dir, 1, c->jobs + c->job_filter[b][dir][grp], ng));
-                c->launches_tmp++;
-            } else if (src != dst) {
-                CK(cudaMemcpyAsync(dst + v0 * P, src + v0 * P, sizeof(double) * ng * P, cudaMemcpyDeviceToDevice, c->stream));
-            }
+        const bool on0 = m & (1 << dir), on1 = m & (8 << dir);
+        // the two groups' lists are adjacent: both in one launch where both are filtered
+        const int g = on0 ? 0 : 1, n = (on0 ? n0 : 0) + (on1 ? N_BSSN : 0);
+        if (!n) continue;
+        if (c->small_f) {
+            CK(small_contract(c, 1, c->sj_filter[b][dir][g], n));
+            c->launches_tmp++;
+        } else if (dir == 1 && c->ft) {
+            for (int grp = 0; grp < 2; grp++)
+                if (grp == 0 ? on0 : on1) {
+                    CK(theta_fourier(c, 1, -1, c->fj_filter[b][grp], c->fj_filter_u[b][grp], grp == 0 ? n0 : N_BSSN));
+                    c->launches_tmp++;
+                }
+        } else {
+            CK(contract(c, dir, 1, c->jobs + c->job_filter[b][dir][g], n));
+            c->launches_tmp++;
         }
     }
+    // a group filtered in no direction
+    if (!(m & 7))
+        CK(cudaMemcpyAsync(c->U[0] + V_D * P, c->U[b] + V_D * P, sizeof(double) * n0 * P, cudaMemcpyDeviceToDevice, c->stream));
+    if (!(m & 56))
+        CK(cudaMemcpyAsync(c->U[0], c->U[b], sizeof(double) * N_BSSN * P, cudaMemcpyDeviceToDevice, c->stream));
     CK(launch_iface_avg(c->d, c->U[0], P, N_BSSN, c->stream));
     c->launches_tmp++;
     if (c->pp.glm) {
@@ -1485,7 +1622,14 @@ extern "C" int grmhd_kernel_times(grmhd_ctx* c, int reps, double* ms_out, double
                                         mixed);
             else if (k >= 1 && k <= 3) {
                 int dir = k - 1;
-                if (dir == 1 && c->ft) {
+                if (c->small_d) {
+                    const int nB = N_D1 + c->pp.glm;
+                    e = small_contract(c, 0, c->sj_first[1] + dir * nB, nB);
+                    if (e == cudaSuccess) e = small_contract(c, 0, c->sj_flux[1] + dir * 8, 8);
+                    if (e == cudaSuccess && c->pp.glm) e = small_contract(c, 0, c->sj_flux[1] + 24 + dir, 1);
+                    fl[k] = contraction_flops(c, dir, 0) * c->job_first_n;
+                    by[k] = (double)P * c->job_first_n * 16.0;
+                } else if (dir == 1 && c->ft) {
                     e = theta_fourier(c, 0, mixed ? 0 : -1, c->fj_first[1], c->fj_first_u[1], c->job_first_n);
                     fl[k] = mixed ? tc_flops(c, dir) * c->job_first_n : contraction_flops(c, dir, 0) * c->job_first_n;
                     by[k] = (double)P * c->job_first_n * (mixed ? 8.0 + 4.0 : 16.0) + 8.0 * 8.0 * P;
@@ -1505,7 +1649,11 @@ extern "C" int grmhd_kernel_times(grmhd_ctx* c, int reps, double* ms_out, double
             } else if (k >= 5 && k <= 7) {
                 int dir = k - 5;
                 const int nj[3] = {3 * N_D2, 2 * N_D2, N_D2};
-                if (dir == 1 && c->ft) {
+                if (c->small_d) {
+                    e = small_contract(c, 0, c->sj_second + (dir > 0 ? nj[0] : 0) + (dir > 1 ? nj[1] : 0), nj[dir]);
+                    fl[k] = contraction_flops(c, dir, 0) * nj[dir];
+                    by[k] = (double)P * nj[dir] * 16.0;
+                } else if (dir == 1 && c->ft) {
                     e = theta_fourier(c, 0, mixed ? 1 : -1, c->fj_second, c->fj_second_u, nj[dir], c->job_first_n);
                     fl[k] = (mixed ? tc_flops(c, dir) : contraction_flops(c, dir, 0)) * nj[dir];
                     by[k] = (double)P * nj[dir] * (mixed ? 8.0 : 16.0);
@@ -1520,23 +1668,23 @@ extern "C" int grmhd_kernel_times(grmhd_ctx* c, int reps, double* ms_out, double
                     by[k] = (double)P * c->job_second_n[dir] * 16.0;
                 }
             } else if (k == 8) {
-                for (int x = 0; x < 3 && e == cudaSuccess; x++)
-                    e = mixed ? launch_iface_avg_f(c->d, reinterpret_cast<float*>(c->d2) + x * P, 6 * P, N_D2, c->stream)
-                              : launch_iface_avg(c->d, c->d2 + x * P, 6 * P, N_D2, c->stream);
+                e = mixed ? launch_iface_avg_f(c->d, reinterpret_cast<float*>(c->d2), P, 3 * N_D2, c->stream, 3, 6 * P)
+                          : launch_iface_avg(c->d, c->d2, P, 3 * N_D2, c->stream, 3, 6 * P);
             }
             else if (k == 9) e = launch_rhs(c->d, c->pp, c->U[0], c->U[1], c->prim, c->flux, c->tmn, c->lam, c->met, c->d1, c->d2,
                                             c->divF, c->divB, c->opts.precision > 0, c->r_scale, c->dt, co, c->scratch,
-                                            c->acc, c->stream);
+                                            c->acc, c->stream, nullptr, c->small_d ? 3 : 1);
             else {
                 int dir = k - 10;
-                // filter contraction of all 32 variables of U[1] (scratch <-> U[1] chain)
-                if (dir == 1 && c->ft) {
+                // filter contraction of all 32 variables, buffers of the filter chain from U[1]
+                if (c->small_f) {
+                    e = small_contract(c, 1, c->sj_filter[1][dir][0], c->nv);
+                } else if (dir == 1 && c->ft) {
                     e = theta_fourier(c, 1, -1, c->fj_filter[1][1], c->fj_filter_u[1][1], N_BSSN);
                     if (e == cudaSuccess)
                         e = theta_fourier(c, 1, -1, c->fj_filter[1][0], c->fj_filter_u[1][0], 8 + c->pp.glm);
                 } else {
-                    e = contract(c, dir, 1, c->jobs + c->job_filter[1][dir][1], N_BSSN);
-                    if (e == cudaSuccess) e = contract(c, dir, 1, c->jobs + c->job_filter[1][dir][0], 8 + c->pp.glm);
+                    e = contract(c, dir, 1, c->jobs + c->job_filter[1][dir][0], c->nv);
                 }
                 fl[k] = contraction_flops(c, dir, 1) * c->nv;
                 by[k] = (double)P * c->nv * 16.0;

@@ -98,13 +98,14 @@ cudaError_t launch_con2prim(const Dims& d, const PhysParams& pp, const double* U
                             unsigned long long* nfail, cudaStream_t s);
 struct RKCoef { double a, b, c, w; int acc_mode; };  // out = a U0 + b Us + c dt L (+acc)
 // d1, d2, divF are double (FP64 mode) or float (deriv_fp32 = 1, mixed modes); ham != null
-// also writes the Hamiltonian constraint per node (diagnostics)
+// also writes the Hamiltonian constraint per node (diagnostics); div_parts: 1, or 3 when divF
+// holds the three directions' terms one after the other (small grids, FP64)
 cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, const double* Us,
                        const double* prim, const double* flux, const double* tmn,
                        const double* lam, const double* met, const void* d1, const void* d2,
                        const void* divF, const void* divB, int deriv_fp32, const double* r_scale_dev,
                        const double* dt_dev, RKCoef co, double* out, double* acc, cudaStream_t s,
-                       double* ham = nullptr);
+                       double* ham = nullptr, int div_parts = 1);
 // tensor-core contraction (kernels_tc.cu); op_img in the kernel's shared-memory layout
 cudaError_t launch_contract_tc(int dir, int in_fp32, const Dims& d, const TcJob* jobs, int njobs,
                                const uint8_t* op_img, int tf32, const double* r_scale, int* err,
@@ -128,6 +129,26 @@ cudaError_t launch_contract_fx(int dir, const Dims& d, const DerivJob* jobs, int
 void fx_tune_set(int dir, int N, int kind, int tsets);
 int fx_tune_get(int dir, int N, int kind);
 bool fx_two_sets_possible(int dir, int N);
+// the same contraction, bit for bit, for small grids on the integer units (kernels_fxs.cu):
+// one launch for the jobs of every direction.  dir 0 r, 1 theta (Chebyshev), 2 phi, 3 theta
+// (Fourier basis, parity +1 / -1); dirs: bit mask of the directions in the list.  Images from
+// fxs_operator_image; img[0] one per element at estride bytes (0: one for all); dir 3 takes
+// the even (img[1]) and odd (img[3]) extension operators
+struct FxsJob {
+    const double* src;
+    double* dst;
+    int dir, parity;
+    int accumulate;       // 0: dst = D src, 1: dst += D src
+    int pad;
+};
+struct FxsOps {
+    const uint8_t* img[4];
+    long long estride;
+};
+bool fxs_supported(int N);
+cudaError_t fxs_init();
+cudaError_t launch_contract_small(const Dims& d, const FxsJob* jobs, int njobs, int dirs, const FxsOps& ops,
+                                  cudaStream_t s);
 cudaError_t launch_deriv(int dir, const Dims& d, const DerivJob* jobs_dev, int njobs,
                          const double* mat_dev, const double* r_scale_dev, cudaStream_t s);
 // reflection-split contraction (kernels_eo.cu): cudaErrorNotSupported when N has no
@@ -136,15 +157,16 @@ bool eo_supported(int dir, int N);
 cudaError_t launch_deriv_eo(int dir, const Dims& d, const DerivJob* jobs, int njobs,
                             const double* op_split, int sign, const double* r_scale,
                             cudaStream_t s);
+// interface means of nfields fields, field f at base + (f / group) group_stride + (f % group) field_stride
 cudaError_t launch_iface_avg(const Dims& d, double* base, long long field_stride, int nfields,
-                             cudaStream_t s);
+                             cudaStream_t s, int group = 1 << 30, long long group_stride = 0);
 // Fourier theta: fold the phi pairs (l, l + N_phi/2) of every job's field into two halves
 // [E][Nr][Nt][N_phi/2] (first the half the even extension operator takes), and the
 // inverse; d are the full grid's dims; fp32 selects float values
 cudaError_t launch_theta_fold(const Dims& d, const FoldJob* jobs, int njobs, int fp32, cudaStream_t s);
 cudaError_t launch_theta_unfold(const Dims& d, const FoldJob* jobs, int njobs, int fp32, cudaStream_t s);
 cudaError_t launch_iface_avg_f(const Dims& d, float* base, long long field_stride, int nfields,
-                               cudaStream_t s);
+                               cudaStream_t s, int group = 1 << 30, long long group_stride = 0);
 // per instance: dt[i] = cfl * hmin[i] / max over its nodes of lambda
 cudaError_t launch_cfl(const Dims& d, int n_inst, const double* U, const double* hmin_dev, double cfl,
                        double* dt_dev, unsigned long long* lam_bits, cudaStream_t s);

@@ -291,6 +291,34 @@ std::vector<uint8_t> fx_operator_image(const std::vector<double>& D, int N, doub
     return img;
 }
 
+std::vector<uint8_t> fxs_operator_image(const std::vector<double>& D, int N, double scale) {
+    const int K4 = (N + 3) / 4;
+    const size_t words = (size_t)N * K4 * 8;
+    std::vector<uint8_t> img((words * 4 + (size_t)N * 4 + 15) / 16 * 16, 0);
+    for (int n = 0; n < N; n++) {
+        int F = 0;
+        for (int k = 0; k < N; k++) {
+            const double x = D[(size_t)n * N + k] * scale;
+            if (x != 0.0) {
+                int ex;
+                std::frexp(x, &ex);
+                F = std::max(F, ex + 1022);
+            }
+        }
+        const int32_t f32 = F;
+        std::memcpy(&img[words * 4 + (size_t)n * 4], &f32, 4);
+        if (F <= 0) continue;
+        for (int k = 0; k < N; k++) {
+            const long long Y = std::llround(std::ldexp(D[(size_t)n * N + k] * scale, 1076 - F));
+            const unsigned long long Z = (unsigned long long)(Y + 0x80808080808080LL);
+            for (int q = 1; q <= 7; q++)
+                img[(((size_t)n * K4 + k / 4) * 8 + (q - 1)) * 4 + k % 4] =
+                    (uint8_t)(((Z >> (8 * (7 - q))) & 0xFF) ^ 0x80);
+        }
+    }
+    return img;
+}
+
 std::vector<double> circulant(const std::vector<double>& row) {
     int n = (int)row.size();
     std::vector<double> M((size_t)n * n);

@@ -31,6 +31,9 @@ std::vector<uint8_t> tc_operator_image(const std::vector<double>& D, int N, int 
 // integer in [-128, 127]); then the Np row exponents (int32); size a multiple of 16 bytes
 std::vector<uint8_t> fx_operator_image(const std::vector<double>& D, int N, double scale, int Np, int Kp,
                                        int KC);
+// the same digits for kernels_fxs.cu: signed bytes, words[row][k / 4][8] (slice l in word l - 1,
+// column k in byte k % 4), then the N row exponents; size a multiple of 16 bytes
+std::vector<uint8_t> fxs_operator_image(const std::vector<double>& D, int N, double scale);
 // BSSN variables 0..23 of the Kerr-Schild slice at (r, theta)
 void ks_bssn_point(double M, double a, double r, double th, double out[24]);
 void prim_to_cons_point(double rho, double p, const double v_u[3], const double B_u[3],

@@ -78,12 +78,13 @@ cudaError_t kernels_init() {
     if ((e = cudaFuncSetAttribute(k_deriv<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 8)) != cudaSuccess) return e;
     if ((e = eo_init()) != cudaSuccess) return e;
     if ((e = fx_init()) != cudaSuccess) return e;
+    if ((e = fxs_init()) != cudaSuccess) return e;
     return tc_init();
 }
 
 // Replace both copies of each duplicated interface node by their mean.
 template <typename T>
-__global__ void k_iface_avg(Dims d, T* base, long long fstride, int nfields) {
+__global__ void k_iface_avg(Dims d, T* base, long long fstride, int nfields, int group, long long gstride) {
     long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     long long nif = (long long)(d.E - 1) * d.NtNp;
     if (t >= nif * nfields) return;
@@ -92,7 +93,7 @@ __global__ void k_iface_avg(Dims d, T* base, long long fstride, int nfields) {
     int e = (int)(r / d.NtNp);
     long long kl = r % d.NtNp;
     if (!d.iface_next[e]) return;  // instance boundary inside a batch group
-    T* u = base + f * fstride;
+    T* u = base + (f / group) * gstride + (f % group) * fstride;
     long long pl = (long long)e * d.elem + (long long)(d.Nr - 1) * d.NtNp + kl;
     long long pr = pl + d.NtNp;
     T m = (T)0.5 * (u[pl] + u[pr]);
@@ -101,20 +102,20 @@ __global__ void k_iface_avg(Dims d, T* base, long long fstride, int nfields) {
 }
 
 cudaError_t launch_iface_avg(const Dims& d, double* base, long long fstride, int nfields,
-                             cudaStream_t s) {
+                             cudaStream_t s, int group, long long gstride) {
     if (d.E < 2 || nfields <= 0) return cudaSuccess;
     long long n = (long long)(d.E - 1) * d.NtNp * nfields;
     int bs = 256;
-    k_iface_avg<double><<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(d, base, fstride, nfields);
+    k_iface_avg<double><<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(d, base, fstride, nfields, group, gstride);
     return cudaGetLastError();
 }
 
 cudaError_t launch_iface_avg_f(const Dims& d, float* base, long long fstride, int nfields,
-                               cudaStream_t s) {
+                               cudaStream_t s, int group, long long gstride) {
     if (d.E < 2 || nfields <= 0) return cudaSuccess;
     long long n = (long long)(d.E - 1) * d.NtNp * nfields;
     int bs = 256;
-    k_iface_avg<float><<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(d, base, fstride, nfields);
+    k_iface_avg<float><<<(unsigned)((n + bs - 1) / bs), bs, 0, s>>>(d, base, fstride, nfields, group, gstride);
     return cudaGetLastError();
 }
 

@@ -36,6 +36,7 @@
 #include <mutex>
 #include <tuple>
 
+#include "fx_digits.cuh"
 #include "grmhd_internal.h"
 
 namespace gk {
@@ -44,7 +45,6 @@ namespace {
 
 constexpr int NDIG = 7;                                      // base-256 digits per operand
 constexpr int NACC = 7;                                      // TMEM accumulators: s = 2..8
-constexpr unsigned long long DIG_BIAS = 0x80808080808080ull;  // 128 in each digit
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -69,21 +69,6 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t da, uint64_t db,
                  "l"(da), "l"(db), "r"(id), "r"(acc));
 }
 
-// Digit word of one value: Z = X + bias with X = round(2 m 2^(e - EL)) the value as a
-// signed fixed-point integer relative to the line exponent EL (|X| <= 2^54; the value is
-// X 2^(EL - 1076)); byte b of Z minus 128 is the balanced digit of weight 256^b.  Branch-
-// free (the values of a thread overlap): round(2 m / 2^sh) = ((4 m >> sh) + 1) >> 1 for
-// sh = EL - e in 0 .. 63 (4 m < 2^56, so every sh >= 56 gives 0), zero for e = 0.
-__device__ __forceinline__ unsigned long long digit_word(double u, int EL) {
-    const long long bits = __double_as_longlong(u);
-    const int e = (int)((bits >> 52) & 0x7FF);
-    const unsigned long long m4 = (((unsigned long long)bits & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 2;
-    const int sh = min(EL - e, 63);
-    const unsigned long long mag = e != 0 ? ((m4 >> sh) + 1) >> 1 : 0ull;
-    const long long x = bits < 0 ? -(long long)mag : (long long)mag;
-    return (unsigned long long)(x + (long long)DIG_BIAS);
-}
-
 // Digit words of a value pair (u0, u1) for the A operand: FP16x2 words holding digit q of
 // u0 (low half) and of u1 (high half).  A biased digit byte b is placed under the byte
 // 0x64, giving the FP16 number 1024 + b, and one packed FP16 add of -1152 leaves b - 128
@@ -102,34 +87,6 @@ __device__ __forceinline__ uint32_t unbias(uint32_t w) {
     uint32_t r;
     asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(w), "r"(0xE480E480u));  // -1152 in both halves
     return r;
-}
-
-// R * 2^X: one correctly rounded integer-to-double conversion, then the power of two is
-// added to the exponent field; *ok false when the result leaves the normal range or R = 0
-// (the caller then takes ldexp_int below).  Branch-free, so that the eight outputs of a
-// column block overlap their conversions.
-__device__ __forceinline__ double ldexp_int(long long R, int X);
-__device__ __forceinline__ double scale_int_fast(long long R, int X, bool* ok) {
-    const double v = __ll2double_rn(R);
-    const int lo = __double2loint(v), hi = __double2hiint(v);
-    const int e = (hi >> 20) & 0x7FF;
-    *ok = e != 0 && (unsigned)(e + X - 1) < 2046u;
-    return __hiloint2double(hi + (X << 20), lo);
-}
-
-// R * 2^X as an IEEE double built with integer instructions (|R| < 2^62; ties away)
-__device__ __forceinline__ double ldexp_int(long long R, int X) {
-    if (R == 0) return 0.0;
-    const unsigned long long sgn = R < 0 ? (1ull << 63) : 0ull;
-    const unsigned long long a = R < 0 ? (unsigned long long)(-R) : (unsigned long long)R;
-    const int p = 63 - __clzll((long long)a);
-    unsigned long long mant;
-    if (p <= 52) mant = a << (52 - p);
-    else { const int sh = p - 52; mant = (a + (1ull << (sh - 1))) >> sh; }
-    const int be = p + X + 1023;
-    if (be <= 0) return __longlong_as_double((long long)sgn);
-    if (be >= 2047) return __longlong_as_double((long long)(sgn | 0x7FF0000000000000ull));
-    return __longlong_as_double((long long)(sgn | ((((unsigned long long)(be - 1)) << 52) + mant)));
 }
 
 // T = sum_s n_s 2^(-8 (s - 2)) as the integer R = round(T 2^40), n_s = acc[s - 2] the exact

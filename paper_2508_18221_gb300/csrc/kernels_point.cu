@@ -1088,7 +1088,7 @@ __global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const doub
                                                const double* __restrict__ divB, const double* __restrict__ r_scale,
                                                const double* __restrict__ dt_dev, RKCoef co,
                                                double* __restrict__ out, double* __restrict__ acc,
-                                               double* __restrict__ ham) {
+                                               double* __restrict__ ham, int div_parts) {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long P = d.P;
     if (p >= P) return;
@@ -1135,7 +1135,8 @@ __global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const doub
         if (pp.evolve_fluid) {
             double r[8];
 #pragma unroll
-            for (int v = 0; v < 8; v++) r[v] = -LD(divF, v);
+            for (int v = 0; v < 8; v++)
+                r[v] = div_parts == 1 ? -LD(divF, v) : -(LD(divF, v) + LD(divF, 8 + v) + LD(divF, 16 + v));
             // V^ij = 1/2 alpha e^{4phi} S^ij, twice that off the diagonal (symmetric sums)
             const double ae = alpha * LD(met, 0), hae = 0.5 * ae;
             double V[6], tr = 0.0, VA = 0.0;
@@ -1519,7 +1520,7 @@ cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, co
                        const double* lam, const double* met, const void* d1, const void* d2,
                        const void* divF, const void* divB, int deriv_fp32, const double* r_scale_dev,
                        const double* dt_dev, RKCoef co, double* out, double* acc, cudaStream_t s,
-                       double* ham) {
+                       double* ham, int div_parts) {
     int bs = 128;
     long long nb = (d.P + bs - 1) / bs;
 #define RHS_ARGS d, pp, U0, Us, prim, flux, tmn, lam, met, (const float*)d1, (const float*)d2, (const float*)divF, \
@@ -1529,7 +1530,7 @@ cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, co
         else k_rhs<false><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
     } else {
 #define RHS64_ARGS d, pp, U0, Us, flux, tmn, lam, met, (const double*)d1, (const double*)d2, (const double*)divF, \
-                   (const double*)divB, r_scale_dev, dt_dev, co, out, acc, ham
+                   (const double*)divB, r_scale_dev, dt_dev, co, out, acc, ham, div_parts
         const unsigned g = (unsigned)nb;
         if (ham) k_rhs64<0, true><<<g, bs, 0, s>>>(RHS64_ARGS);
         else if (co.acc_mode < 0) k_rhs64<0, false><<<g, bs, 0, s>>>(RHS64_ARGS);
