@@ -1054,7 +1054,7 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
 // A variable is written as soon as its right-hand side is known (no array of 33 in local
 // memory: 254 registers without spills, against 904 B of spills per thread).  Measured on
 // 393,216 nodes, per launch: 1.085 -> 0.603 ms.  MODE: 0 the plain right-hand side, 1 the first SSP-RK3 stage Us + dt L, 2 the
-// others a U0 + b (Us + dt L), 3 RK4 stages.
+// others a U0 + b (Us + dt L), 3 RK4 stages.  DIVP: parts of divF to add (1, or 3 on small grids).
 template <int MODE>
 struct Emit {
     const double *U0, *Us;
@@ -1079,7 +1079,7 @@ struct Emit {
     }
 };
 
-template <int MODE, bool HAM>
+template <int MODE, bool HAM, int DIVP>
 __global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const double* __restrict__ U0,
                                                const double* __restrict__ Us, const double* __restrict__ flux,
                                                const double* __restrict__ mat, const double* __restrict__ lam,
@@ -1088,7 +1088,7 @@ __global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const doub
                                                const double* __restrict__ divB, const double* __restrict__ r_scale,
                                                const double* __restrict__ dt_dev, RKCoef co,
                                                double* __restrict__ out, double* __restrict__ acc,
-                                               double* __restrict__ ham, int div_parts) {
+                                               double* __restrict__ ham) {
     const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const long long P = d.P;
     if (p >= P) return;
@@ -1136,7 +1136,7 @@ __global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const doub
             double r[8];
 #pragma unroll
             for (int v = 0; v < 8; v++)
-                r[v] = div_parts == 1 ? -LD(divF, v) : -(LD(divF, v) + LD(divF, 8 + v) + LD(divF, 16 + v));
+                r[v] = DIVP == 1 ? -LD(divF, v) : -(LD(divF, v) + LD(divF, 8 + v) + LD(divF, 16 + v));
             // V^ij = 1/2 alpha e^{4phi} S^ij, twice that off the diagonal (symmetric sums)
             const double ae = alpha * LD(met, 0), hae = 0.5 * ae;
             double V[6], tr = 0.0, VA = 0.0;
@@ -1529,15 +1529,18 @@ cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, co
         if (ham) k_rhs<true><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
         else k_rhs<false><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
     } else {
-#define RHS64_ARGS d, pp, U0, Us, flux, tmn, lam, met, (const double*)d1, (const double*)d2, (const double*)divF, \
-                   (const double*)divB, r_scale_dev, dt_dev, co, out, acc, ham, div_parts
         const unsigned g = (unsigned)nb;
-        if (ham) k_rhs64<0, true><<<g, bs, 0, s>>>(RHS64_ARGS);
-        else if (co.acc_mode < 0) k_rhs64<0, false><<<g, bs, 0, s>>>(RHS64_ARGS);
-        else if (co.acc_mode > 0) k_rhs64<3, false><<<g, bs, 0, s>>>(RHS64_ARGS);
-        else if (co.a == 0.0 && co.b == 1.0) k_rhs64<1, false><<<g, bs, 0, s>>>(RHS64_ARGS);
-        else k_rhs64<2, false><<<g, bs, 0, s>>>(RHS64_ARGS);
-#undef RHS64_ARGS
+        const auto run = [&](auto k) {
+            k<<<g, bs, 0, s>>>(d, pp, U0, Us, flux, tmn, lam, met, (const double*)d1, (const double*)d2,
+                               (const double*)divF, (const double*)divB, r_scale_dev, dt_dev, co, out, acc, ham);
+        };
+        // (a runtime branch on div_parts cost 4 %: the additions were issued either way)
+        const bool p3 = div_parts == 3;
+        if (ham) p3 ? run(k_rhs64<0, true, 3>) : run(k_rhs64<0, true, 1>);
+        else if (co.acc_mode < 0) p3 ? run(k_rhs64<0, false, 3>) : run(k_rhs64<0, false, 1>);
+        else if (co.acc_mode > 0) p3 ? run(k_rhs64<3, false, 3>) : run(k_rhs64<3, false, 1>);
+        else if (co.a == 0.0 && co.b == 1.0) p3 ? run(k_rhs64<1, false, 3>) : run(k_rhs64<1, false, 1>);
+        else p3 ? run(k_rhs64<2, false, 3>) : run(k_rhs64<2, false, 1>);
     }
 #undef RHS_ARGS
     return cudaGetLastError();
