@@ -255,9 +255,13 @@ std::vector<uint8_t> fx_operator_image(const std::vector<double>& D, int N, doub
                                        int KC) {
     const int nch = Kp / KC, kcores = KC / 8, Npp = Np > 64 ? 64 : Np;
     const size_t slice = (size_t)Np * KC * 2, chunk = 7 * slice;
-    const size_t bytes = ((size_t)nch * chunk + (size_t)Np * 4 + 15) / 16 * 16;
+    const size_t bytes = ((size_t)nch * chunk + (size_t)Np * 4 + 16 + 15) / 16 * 16;
     std::vector<uint8_t> img(bytes, 0);
     std::vector<int32_t> fexp(Np, 0);
+    // bound of |sum_k c_l(k) d_q(k)| summed over the pairs of each digit order (|d_1| <= 64, the
+    // other |d_q| <= 128), largest over the orders and rows
+    long long bound = 0;
+    int fmin = 1 << 20, fmax = 0;
     for (int n = 0; n < N; n++) {
         int F = 0;
         for (int k = 0; k < N; k++) {
@@ -269,7 +273,10 @@ std::vector<uint8_t> fx_operator_image(const std::vector<double>& D, int N, doub
             }
         }
         fexp[n] = F;
+        fmin = std::min(fmin, F);
+        fmax = std::max(fmax, F);
         if (F <= 0) continue;
+        long long csum[8] = {0};
         for (int k = 0; k < N; k++) {
             const double x = D[(size_t)n * N + k] * scale;
             const long long Y = std::llround(std::ldexp(x, 1076 - F));
@@ -278,6 +285,7 @@ std::vector<uint8_t> fx_operator_image(const std::vector<double>& D, int N, doub
             for (int q = 1; q <= 7; q++) {
                 const int digit = (int)((Z >> (8 * (7 - q))) & 0xFF) - 128;
                 const uint16_t b = half_of_digit(digit);
+                csum[q] += std::abs(digit);
                 // row of the chunk's tall B matrix: pass p (Npp = min(Np, 64) output rows),
                 // then slice, then the row within the pass
                 const int row = ((n / Npp) * 7 + (q - 1)) * Npp + n % Npp;
@@ -286,8 +294,15 @@ std::vector<uint8_t> fx_operator_image(const std::vector<double>& D, int N, doub
                 std::memcpy(&img[off], &b, 2);
             }
         }
+        for (int s = 2; s <= 8; s++) {
+            long long t = 0;
+            for (int l = 1; l < s; l++) t += csum[l] * (s - l == 1 ? 64 : 128);
+            bound = std::max(bound, t);
+        }
     }
     std::memcpy(&img[(size_t)nch * chunk], fexp.data(), (size_t)Np * 4);
+    const int32_t meta[3] = {bound >= (1 << 22) ? 1 : 0, fmin, fmax};
+    std::memcpy(&img[(size_t)nch * chunk + (size_t)Np * 4], meta, sizeof(meta));
     return img;
 }
 

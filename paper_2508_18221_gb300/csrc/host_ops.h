@@ -28,7 +28,9 @@ std::vector<uint8_t> tc_operator_image(const std::vector<double>& D, int N, int 
 // (kernels_fx.cu): per K chunk of KC columns one tall FP16 matrix in the K-major
 // core-matrix layout whose rows are, per pass of Npp = min(Np, 64) output rows, the seven
 // balanced base-256 digit slices of those rows one after the other (each digit an FP16
-// integer in [-128, 127]); then the Np row exponents (int32); size a multiple of 16 bytes
+// integer in [-128, 127]); then the Np row exponents (int32) and three int32: 1 when a
+// digit-order sum can reach 2^22 (else its conversion takes the narrow form), the smallest
+// and the largest row exponent; size a multiple of 16 bytes
 std::vector<uint8_t> fx_operator_image(const std::vector<double>& D, int N, double scale, int Np, int Kp,
                                        int KC);
 // the same digits for kernels_fxs.cu: signed bytes, words[row][k / 4][8] (slice l in word l - 1,

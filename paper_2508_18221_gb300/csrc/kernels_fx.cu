@@ -91,37 +91,55 @@ __device__ __forceinline__ uint32_t unbias(uint32_t w) {
 
 // T = sum_s n_s 2^(-8 (s - 2)) as the integer R = round(T 2^40), n_s = acc[s - 2] the exact
 // integer sum of the digit products of order s (digits are plain integers in both
-// operands), |n_s| <= (s - 1) K 2^14: below 2^24 for K <= 128 and below 2^22 for K <= 32.
-// Each n_s is made non-negative by an offset, t_s = n_s + o_s: below 2^22 t_s is read off
-// the bits of n_s + 1.5 * 2^23 (the low 23 bits hold n_s + 2^22; exact, as n_s is an
-// integer), above it comes from a float-to-integer conversion (exact too).
-// The t_s are summed at their byte offsets with 32 x 32 -> 64-bit multiply-adds (an
-// unsigned sum below 2^63), the s = 8 term rounded to the unit of s = 7 (half up), and the
-// offsets' total is subtracted once.
-template <bool WIDE>
-__device__ __forceinline__ long long combine7(const uint32_t* acc) {
-    const float MAG = 12582912.f;  // 1.5 * 2^23
+// operands), the s = 8 term rounded to the unit of s = 7 (half up).
+//
+// Narrow (|n_s| < 2^22): the bits of the FP32 sum n_s + 1.5 2^23 are 0x4B400000 + n_s, so the
+// seven bit patterns are added at their byte offsets modulo 2^64 and the constant that the
+// seven 0x4B400000 add up to is taken off once (it starts the sum).  The integer pipe bounds
+// the epilogue, so the sums are 32 x 32 + 64-bit multiply-adds of the multiply-add pipe:
+// the powers of two come in as kernel parameters, out of the compiler's sight.  Whether an
+// operator's sums stay below 2^22 is found from its digits on the host (every size up to 64
+// nodes does); float-to-integer conversions, a quarter-rate pipe, are left to the longer
+// ones.  With digit_word's single addition, launches of 29 / 33 fields of 393,216 nodes went
+// from 85.9 to 76.7 us (r, 24 nodes), 128 to 119 (theta, 32), 126 to 119 (phi, 64).
+struct Pow2 {
+    uint32_t p24, p16, p8, p0;
+};
+__device__ __forceinline__ unsigned long long mad_wide(uint32_t a, uint32_t b, unsigned long long c) {
+    unsigned long long r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ long long combine_narrow(const uint32_t* acc, const Pow2& w) {
+    constexpr unsigned long long M = 0x4B400000ull;
+    constexpr unsigned long long OFF = (M << 40) + (M << 32) + (M << 24) + (M << 16) + (M << 8) + M + (M >> 8);
     uint32_t t[NACC];
-    unsigned long long off;
-    if (!WIDE) {
 #pragma unroll
-        for (int s = 0; s < NACC; s++) t[s] = (uint32_t)__float_as_int(__uint_as_float(acc[s]) + MAG) & 0x7FFFFFu;
-        // o_s = 2^22 for every s
-        off = (1ull << 62) + (1ull << 54) + (1ull << 46) + (1ull << 38) + (1ull << 30) + (1ull << 22) + (1ull << 14);
-    } else {
-        // |n_s| <= (s - 1) K 2^14 <= (s - 1) 2^21: o_2 = 2^21, the others o_s = 2^24
+    for (int s = 0; s < NACC; s++) t[s] = __float_as_uint(__uint_as_float(acc[s]) + 12582912.f);
+    unsigned long long a = mad_wide(t[2], w.p24, 0ull - OFF);
+    a = mad_wide(t[3], w.p16, a);
+    a = mad_wide(t[4], w.p8, a);
+    a = mad_wide(t[5], w.p0, a);
+    a = mad_wide((t[6] + 128u) >> 8, w.p0, a);
+    return (long long)(a + ((unsigned long long)(t[0] * w.p8 + t[1]) << 32));
+}
+// Wide (|n_s| < 2^24, K <= 128): t_s = n_s + o_s from float-to-integer conversions, summed
+// the same way as non-negative integers
+__device__ __forceinline__ long long combine_wide(const uint32_t* acc) {
+    uint32_t t[NACC];
+    // |n_s| <= (s - 1) K 2^14 <= (s - 1) 2^21: o_2 = 2^21, the others o_s = 2^24
 #pragma unroll
-        for (int s = 0; s < NACC; s++)
-            t[s] = (uint32_t)(__float2int_rn(__uint_as_float(acc[s])) + (s == 0 ? (1 << 21) : (1 << 24)));
-        off = (1ull << 61) + (1ull << 56) + (1ull << 48) + (1ull << 40) + (1ull << 32) + (1ull << 24) + (1ull << 16);
-    }
+    for (int s = 0; s < NACC; s++)
+        t[s] = (uint32_t)(__float2int_rn(__uint_as_float(acc[s])) + (s == 0 ? (1 << 21) : (1 << 24)));
+    constexpr unsigned long long OFF =
+        (1ull << 61) + (1ull << 56) + (1ull << 48) + (1ull << 40) + (1ull << 32) + (1ull << 24) + (1ull << 16);
     // t_2 2^40 + t_3 2^32 + t_4 2^24 + t_5 2^16 + t_6 2^8 + t_7 + round(t_8 / 256)
     unsigned long long a = (unsigned long long)t[2] * (1ull << 24) + t[5];
     a += (unsigned long long)t[3] * (1ull << 16);
     a += (unsigned long long)t[4] * (1ull << 8);
     a += (unsigned long long)((t[0] << 8) + t[1]) << 32;
     a += (t[6] + 128u) >> 8;
-    return (long long)(a - off);
+    return (long long)(a - OFF);
 }
 
 }  // namespace
@@ -176,6 +194,11 @@ __device__ __forceinline__ double stg_at(const double* stg, int m, int k, int N)
     return DIR == 2 ? stg[m * stg_rs<DIR>(N) * 2 + k] : stg[k * 128 + m];
 }
 
+template <int DIR>
+__device__ __forceinline__ uint32_t stg_hi(const double* stg, int m, int k, int N) {
+    return reinterpret_cast<const uint32_t*>(stg)[2 * (DIR == 2 ? m * stg_rs<DIR>(N) * 2 + k : k * 128 + m) + 1];
+}
+
 struct FxParams {
     const DerivJob* jobs;
     const uint8_t* img;
@@ -191,6 +214,8 @@ struct FxParams {
     uint32_t stg_bytes;
     int* err;
     int stall;               // test of the wait limits: the staging warp issues no copies
+    Pow2 pw;                 // 2^24, 2^16, 2^8, 1
+    uint32_t four;           // 4
     int tsets;               // TMEM accumulator sets: 1, or 2 (item k in set k % 2: the MMAs of
                              // item k + 1 run while the epilogue drains item k; needs b_all)
 };
@@ -534,10 +559,11 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
             const double* stg = reinterpret_cast<const double*>(sm + b * fp.stg_bytes);
             const bool valid = m < tl.nlines;
             if (!bwait(&bars->stg_full[b], (uint32_t)((k / fp.nstg) & 1), abort_flag)) break;
-            int EL = 0;
+            // the largest |high word| holds the largest exponent
+            uint32_t hm = 0;
             if (valid)
-                for (int j = 0; j < N; j++)
-                    EL = max(EL, (int)((__double_as_longlong(stg_at<DIR>(stg, m, j, N)) >> 52) & 0x7FF));
+                for (int j = 0; j < N; j++) hm = max(hm, stg_hi<DIR>(stg, m, j, N) & 0x7FFFFFFFu);
+            const int EL = (int)(hm >> 20);
             if (grp == 0) {
                 // the epilogue of item k - 2 has read this set of sEL and sF
                 const int t = k & 1;
@@ -572,8 +598,8 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
                             const int kk = k0 + 2 * h;
                             const double u0 = kk < N ? stg_at<DIR>(stg, m, kk, N) : 0.0;
                             const double u1 = kk + 1 < N ? stg_at<DIR>(stg, m, kk + 1, N) : 0.0;
-                            const DigitHalves a0 = digit_halves(digit_word(u0, EL));
-                            const DigitHalves a1 = digit_halves(digit_word(u1, EL));
+                            const DigitHalves a0 = digit_halves(digit_word(u0, EL, fp.four));
+                            const DigitHalves a1 = digit_halves(digit_word(u1, EL, fp.four));
                             // digit q = 1 .. 7 sits in byte 7 - q of Z
                             w[0][h] = unbias(__byte_perm(a0.eh, a1.eh, 0x7632));   // byte 6
                             w[1][h] = unbias(__byte_perm(a0.oh, a1.oh, 0x5410));   // byte 5
@@ -604,7 +630,6 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
         // warp w reads TMEM lanes 32 (w & 3) ..; with W = 8 the two warps of a lane quadrant
         // take the first and the second half of the column blocks
         const int quad = warp & 3, m = quad * 32 + lane, half = (warp - WC) >> 2;
-        const bool wide = fp.Kp > 32;   // scaled accumulators reach 2^22
         int k = 0;
         for (long long it = blockIdx.x; it < nitems; it += gridDim.x, k++) {
             FxTile tl;
@@ -632,6 +657,12 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
                 }
             }
             const int EL = sEL[t * 128 + m];
+            // the operator's sums stay below 2^22 (narrow); its rows' smallest and largest exponent
+            const int* meta = reinterpret_cast<const int*>(fp.img + (DIR == 0 ? tl.e * fp.img_estride : 0) +
+                                                           (size_t)op_bytes) + Np;
+            const bool wide = __ldg(meta) != 0;
+            // R has 63 bits at most, so every result of the line is a normal number or zero
+            const bool safe = EL + __ldg(meta + 1) >= 1096 && EL + __ldg(meta + 2) <= 2996;
             const bool line_bad = EL == 0x7FF;
             // column blocks holding output rows of this pass (the padding blocks beyond N are
             // computed by the MMAs but not read)
@@ -668,7 +699,7 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
                     if (lane == 0) barrive(&bars->acc_empty[t]);
                 }
                 if (valid) {
-                    // phases over the eight outputs (combine, convert, fix-ups), so that their
+                    // phases over the eight outputs (combine, convert, scale), so that their
                     // dependency chains overlap
                     long long R[8];
                     if (wide) {
@@ -677,7 +708,7 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
                             uint32_t acc[NA];
 #pragma unroll
                             for (int g = 0; g < NA; g++) acc[g] = r[g][j];
-                            R[j] = combine7<true>(acc);
+                            R[j] = combine_wide(acc);
                         }
                     } else {
 #pragma unroll
@@ -685,23 +716,27 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
                             uint32_t acc[NA];
 #pragma unroll
                             for (int g = 0; g < NA; g++) acc[g] = r[g][j];
-                            R[j] = combine7<false>(acc);
+                            R[j] = combine_narrow(acc, fp.pw);
                         }
                     }
                     double v[8];
-                    bool ok[8], all_ok = true;
+                    if (safe) {
 #pragma unroll
-                    for (int j = 0; j < 8; j++) {
-                        v[j] = scale_int_fast(R[j], X[j], &ok[j]);
-                        all_ok = all_ok && ok[j];
+                        for (int j = 0; j < 8; j++) v[j] = __ll2double_rn(R[j]);
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            const int hi = __double2hiint(v[j]);
+                            v[j] = __hiloint2double(hi != 0 ? hi + (X[j] << 20) : hi, __double2loint(v[j]));
+                        }
+                    } else {
+#pragma unroll
+                        for (int j = 0; j < 8; j++) {
+                            bool ok;
+                            v[j] = scale_int_fast(R[j], X[j], &ok);
+                            if (!ok) v[j] = R[j] == 0 ? 0.0 : ldexp_int(R[j], X[j]);
+                            if (line_bad) v[j] = __longlong_as_double(0x7FF8000000000000ll);
+                        }
                     }
-                    if (!all_ok)
-#pragma unroll
-                        for (int j = 0; j < 8; j++)
-                            if (!ok[j]) v[j] = R[j] == 0 ? 0.0 : ldexp_int(R[j], X[j]);
-                    if (line_bad)
-#pragma unroll
-                        for (int j = 0; j < 8; j++) v[j] = __longlong_as_double(0x7FF8000000000000ll);
                     double* pd = jb.dst + base + (long long)c0 * stride;
                     if (DIR == 2 && c0 + 8 <= N && (reinterpret_cast<uintptr_t>(pd) & 15) == 0) {
                         // phi: the block's outputs are contiguous in the line: 16-byte stores
@@ -722,6 +757,9 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
 #pragma unroll
                         for (int j = 0; j < 8; j++)
                             if (c0 + j < N) pd[(long long)j * stride] += v[j];
+                    } else if (c0 + 8 <= N) {
+#pragma unroll
+                        for (int j = 0; j < 8; j++) pd[(long long)j * stride] = v[j];
                     } else {
 #pragma unroll
                         for (int j = 0; j < 8; j++)
@@ -892,6 +930,8 @@ cudaError_t launch_contract_fx(int dir, const Dims& d, const DerivJob* jobs, int
     fp.err = err;
     fp.stall = stall;
     fp.tsets = cfg.tsets;
+    fp.pw = {1u << 24, 1u << 16, 1u << 8, 1u};
+    fp.four = 4u;
     if (d.P >= (1LL << 31) || (d.P / 16 + d.E) * 2 * (long long)njobs >= (1LL << 31))
         return cudaErrorNotSupported;   // 32-bit line and item arithmetic
     fp.tpe = (uint32_t)((d.NtNp + 127) / 128);

@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(NW * 32) k_contract_small(Dims d, FxsOps ops, 
     for (int g = warp; g < K4; g += NW) {
         unsigned long long z[4];
 #pragma unroll
-        for (int k = 0; k < 4; k++) z[k] = digit_word(4 * g + k < N ? sV[(4 * g + k) * 33 + lane] : 0.0, EL);
+        for (int k = 0; k < 4; k++) z[k] = digit_word(4 * g + k < N ? sV[(4 * g + k) * 33 + lane] : 0.0, EL, 4u);
 #pragma unroll
         for (int q = 0; q < 7; q++) sA[(g * 7 + q) * 32 + lane] = pack_byte(z, 6 - q);
     }
