@@ -742,21 +742,25 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
                         // phi: the block's outputs are contiguous in the line: 16-byte stores
                         double2* p2 = reinterpret_cast<double2*>(pd);
                         if (jb.accumulate) {
+                            double2 o[4];
 #pragma unroll
-                            for (int h = 0; h < 4; h++) {
-                                double2 o = p2[h];
-                                o.x += v[2 * h];
-                                o.y += v[2 * h + 1];
-                                p2[h] = o;
-                            }
+                            for (int h = 0; h < 4; h++) o[h] = p2[h];
+#pragma unroll
+                            for (int h = 0; h < 4; h++)
+                                p2[h] = make_double2(o[h].x + v[2 * h], o[h].y + v[2 * h + 1]);
                         } else {
 #pragma unroll
                             for (int h = 0; h < 4; h++) p2[h] = make_double2(v[2 * h], v[2 * h + 1]);
                         }
                     } else if (jb.accumulate) {
+                        // all loads before the first store (the compiler cannot reorder them): one
+                        // trip to memory per block of columns instead of eight in turn
+                        double o[8];
+#pragma unroll
+                        for (int j = 0; j < 8; j++) o[j] = c0 + j < N ? pd[(long long)j * stride] : 0.0;
 #pragma unroll
                         for (int j = 0; j < 8; j++)
-                            if (c0 + j < N) pd[(long long)j * stride] += v[j];
+                            if (c0 + j < N) pd[(long long)j * stride] = o[j] + v[j];
                     } else if (c0 + 8 <= N) {
 #pragma unroll
                         for (int j = 0; j < 8; j++) pd[(long long)j * stride] = v[j];
