@@ -396,7 +396,11 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
         if (e != cudaSuccess) { free_ctx(c); return GRMHD_ECUDA; }
         c->own_stream = true;
     }
-    if (cudaStreamCreateWithFlags(&c->s2, cudaStreamNonBlocking) != cudaSuccess ||
+    // the side stream's kernels go first where both streams have blocks waiting: its chain is the
+    // longer one of a single right-hand side
+    int prio_low = 0, prio_high = 0;
+    cudaDeviceGetStreamPriorityRange(&prio_low, &prio_high);
+    if (cudaStreamCreateWithPriority(&c->s2, cudaStreamNonBlocking, prio_high) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess) {
         free_ctx(c);
@@ -975,14 +979,15 @@ extern "C" int grmhd_coords(const grmhd_ctx* c, double* r, double* th, double* p
 // against its largest value) reaches 1.5e-11 at 96 theta nodes, against 9.5e-12 for the
 // FP64 units, which take those derivatives.  force_fx (the test hook): the digit slices
 // whenever the image exists.
+// share: another kernel is to run on the same SMs (see launch_contract_fx).
 static cudaError_t contract(grmhd_ctx* c, int dir, int filter, const DerivJob* jobs, int njobs,
-                            bool force_fx = false) {
+                            bool force_fx = false, bool share = false) {
     if (dir == 1 && c->ft) return cudaErrorInvalidValue;   // theta_fourier below
     const int Ns[3] = {c->d.Nr, c->d.Nt, c->d.Np};
     const bool cheb_d = !filter && dir < 2;
     const uint8_t* fx = filter ? c->fx_f[dir] : ((cheb_d && Ns[dir] > 64 && !force_fx) ? nullptr : c->fx_d[dir]);
     if (fx) return launch_contract_fx(dir, c->d, jobs, njobs, fx, (dir == 0 && !filter) ? c->fx_estride : 0,
-                                      c->tc_err, c->stream, 0, filter ? 1 : 0);
+                                      c->tc_err, c->stream, 0, filter ? 1 : 0, 0, share);
     const double* split = filter ? c->Fs[dir] : c->Ds[dir];
     const double* rs = filter ? nullptr : c->r_scale;
     if (split) return launch_deriv_eo(dir, c->d, jobs, njobs, split, filter ? 1 : -1, rs, c->stream);
@@ -1030,7 +1035,14 @@ static cudaError_t small_contract(grmhd_ctx* c, int filter, int off, int n) {
 // First derivatives from buffer b.  part 0: the BSSN fields (+ psi) and their interface
 // means; part 1: the flux divergence (+ the field divergence with GLM), which needs the
 // fluxes of k_prep.
-static int enqueue_first_derivs(grmhd_ctx* c, int b, int part) {
+//
+// FP64, part 0: phi goes first, with its second derivatives d_phi d_phi (second = 1; they need
+// d_phi alone), in the form whose CTA leaves half of an SM's registers free: k_prep starts
+// with it on the main stream and its blocks share the SMs (FP64 pipe against tensor and
+// integer pipes).  Two k_prep and six 21-field phi launches of 393,216 nodes take 563 and
+// 495 us apart, 812 us together; the r and theta forms (two CTAs per SM) gain nothing
+// together (863 against 912, and one CTA per SM 828).  SSP-RK3 step 4.59 -> 4.45 ms.
+static int enqueue_first_derivs(grmhd_ctx* c, int b, int part, int second = 0) {
     const int nB = N_D1 + c->pp.glm, off = part == 0 ? 0 : nB, n = part == 0 ? nB : c->job_first_n - nB;
     const int mixed = c->opts.precision > 0, tf32 = c->opts.precision == 2;
     if (c->small_d) {
@@ -1041,15 +1053,20 @@ static int enqueue_first_derivs(grmhd_ctx* c, int b, int part) {
             c->launches_tmp++;
         }
     }
-    for (int dir = 0; dir < 3 && !c->small_d; dir++) {
+    for (int k = 0; k < 3 && !c->small_d; k++) {
+        const int dir = part == 0 && !mixed ? (k + 2) % 3 : k;
         if (dir == 1 && c->ft)
             CK(theta_fourier(c, 0, mixed ? 0 : -1, c->fj_first[b] + off, c->fj_first_u[b] + off, n, off));
         else if (mixed)
             CK(launch_contract_tc(dir, 0, c->d, c->tcjobs + c->tc_first[b][dir] + off, n, c->tc_img[dir], tf32,
                                   c->r_scale, c->tc_err, c->stream));
         else
-            CK(contract(c, dir, 0, c->jobs + c->job_first[b][dir] + off, n));
+            CK(contract(c, dir, 0, c->jobs + c->job_first[b][dir] + off, n, false, part == 0 && dir == 2));
         c->launches_tmp++;
+        if (second && dir == 2 && !mixed) {
+            CK(contract(c, 2, 0, c->jobs + c->job_second[2], c->job_second_n[2], false, true));
+            c->launches_tmp++;
+        }
     }
     if (part == 0) {
         if (mixed) CK(launch_iface_avg_f(c->d, reinterpret_cast<float*>(c->d1), 3 * c->d.P, nB, c->stream));
@@ -1084,7 +1101,7 @@ static int enqueue_second_derivs(grmhd_ctx* c) {
         CK(small_contract(c, 0, c->sj_second, 6 * N_D2));
         c->launches_tmp++;
     }
-    for (int dir = 0; dir < 3 && !c->small_d; dir++) {
+    for (int dir = 0; dir < 2 && !c->small_d; dir++) {   // phi: with the first derivatives
         if (dir == 1 && c->ft)
             CK(theta_fourier(c, 0, -1, c->fj_second, c->fj_second_u, c->job_second_n[dir], c->job_first_n));
         else CK(contract(c, dir, 0, c->jobs + c->job_second[dir], c->job_second_n[dir]));
@@ -1115,7 +1132,7 @@ static int enqueue_stage(grmhd_ctx* c, int b, RKCoef co, double* out, const Phys
     int st;
     {
         OnStream on(c, c->s2);
-        st = enqueue_first_derivs(c, b, 0);
+        st = enqueue_first_derivs(c, b, 0, pp.evolve_metric);
         if (!st && pp.evolve_metric) st = enqueue_second_derivs(c);
         if (!st) CK(cudaEventRecord(c->ev_join, c->s2));
     }

@@ -120,10 +120,11 @@ cudaError_t fx_init();
 // kernel runs out (about 0.5 s), the CTAs leave and *err is set.  kind: 0 derivative, 1
 // filter (the key of the tuning table; the arithmetic is the same).  tsets: TMEM accumulator
 // sets (1, or 2: the next item's MMAs run while the epilogue drains the previous one; one
-// CTA per SM); 0 takes the tuning table's choice for the class
+// CTA per SM); 0 takes the tuning table's choice for the class; share: where one CTA fills an
+// SM (33 nodes up), the smaller form that leaves room for another kernel's blocks
 cudaError_t launch_contract_fx(int dir, const Dims& d, const DerivJob* jobs, int njobs, const uint8_t* op_img,
                                long long img_estride, int* err, cudaStream_t s, int stall = 0, int kind = 0,
-                               int tsets = 0);
+                               int tsets = 0, bool share = false);
 // tuning table of the digit-slice contraction (process-wide): accumulator sets per
 // (direction, nodes, kind); 0 when the class was not tuned
 void fx_tune_set(int dir, int N, int kind, int tsets);

@@ -905,7 +905,8 @@ cudaError_t fx_init() {
 }
 
 cudaError_t launch_contract_fx(int dir, const Dims& d, const DerivJob* jobs, int njobs, const uint8_t* img,
-                               long long img_estride, int* err, cudaStream_t s, int stall, int kind, int tsets) {
+                               long long img_estride, int* err, cudaStream_t s, int stall, int kind, int tsets,
+                               bool share) {
     if (njobs <= 0) return cudaSuccess;
     if (kind != 0 && kind != 1) return cudaErrorNotSupported;
     const int N = dir == 0 ? d.Nr : (dir == 1 ? d.Nt : d.Np);
@@ -951,8 +952,10 @@ cudaError_t launch_contract_fx(int dir, const Dims& d, const DerivJob* jobs, int
     const long long grid = nitems < (long long)cfg.ctas * nsm ? nitems : (long long)cfg.ctas * nsm;
     const size_t sm = cfg.smem;
     // one CTA per SM: eight converter and eight epilogue warps (the register file holds
-    // them at up to 112 registers a thread); two: four of each (96 registers)
-    const bool w8 = cfg.ctas == 1;
+    // them at up to 112 registers a thread); two: four of each (96 registers).  One CTA of four of
+    // each is 7 % slower by itself (phi, 64 nodes, 21 fields: 82 -> 88 us) and leaves half of
+    // the register file to another kernel's blocks
+    const bool w8 = cfg.ctas == 1 && !share;
     const unsigned nt = (unsigned)(w8 ? fx_threads(8, 8) : fx_threads(4, 4));
     if (dir == 0) {
         if (w8) k_contract_fx<0, 8, 8><<<(unsigned)grid, nt, sm, s>>>(d, fp);
