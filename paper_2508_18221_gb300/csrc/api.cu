@@ -733,12 +733,13 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
         float* d1f = reinterpret_cast<float*>(c->d1);
         float* d2f = reinterpret_cast<float*>(c->d2);
         float* dFf = reinterpret_cast<float*>(c->divF);
+        const float* fxf = reinterpret_cast<const float*>(c->flux);   // FP32 values in these modes
         for (int b = 0; b < 3; b++)
             for (int dir = 0; dir < 3; dir++) {
                 c->tc_first[b][dir] = (int)tj.size();
                 for (int f = 0; f < N_D1; f++) addt(c->U[b] + (long long)f * P, d1f + ((long long)f * 3 + dir) * P, 0);
                 if (opts->glm) addt(c->U[b] + (long long)V_PSI * P, d1f + ((long long)N_D1 * 3 + dir) * P, 0);
-                for (int v = 0; v < 8; v++) addt(c->flux + ((long long)dir * 8 + v) * P, dFf + (long long)v * P, dir > 0);
+                for (int v = 0; v < 8; v++) addt(fxf + ((long long)dir * 8 + v) * P, dFf + (long long)v * P, dir > 0);
                 if (opts->glm) addt(c->U[b] + (long long)(V_B + dir) * P, reinterpret_cast<float*>(c->divB), dir > 0);
             }
         const int vars2[N_D2] = {0, 1, 2, 3, 4, 5, 6, 17, 18, 19, 20};
@@ -797,7 +798,12 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
         for (int b = 0; b < 3; b++) {
             const DerivJob* jl = &jobs[c->job_first[b][1]];
             c->fj_first[b] = (int)fj.size();
-            for (int i = 0; i < n1; i++) addf(jl[i].src, c->Y + (long long)i * P, par1[i], 0);
+            // (mixed: the fluxes are FP32, folded into FP32 fields)
+            for (int i = 0; i < n1; i++) {
+                const bool f32 = mixed && i >= N_D1 + glm && i < N_D1 + glm + 8;
+                if (f32) addf(tj[c->tc_first[b][1] + i].src, Yf + 2LL * i * P, par1[i], 0);
+                else addf(jl[i].src, c->Y + (long long)i * P, par1[i], 0);
+            }
             c->fj_first_u[b] = (int)fj.size();
             for (int i = 0; i < n1; i++) {
                 if (mixed) {
@@ -1024,6 +1030,25 @@ static cudaError_t theta_fourier(grmhd_ctx* c, int filter, int stage, int fold_o
     return launch_theta_unfold(c->d, c->fjobs + unfold_off, n, stage >= 0, c->stream);
 }
 
+// One direction of the mixed first derivatives: part 0 the FP64 fields of the state, part 1 the
+// FP32 fluxes and, with GLM, the FP64 field
+static cudaError_t first_mixed(grmhd_ctx* c, int b, int dir, int part) {
+    const int nB = N_D1 + c->pp.glm, tf32 = c->opts.precision == 2;
+    const auto run = [&](int fp32, int off, int n) {
+        if (dir == 1 && c->ft)
+            return theta_fourier(c, 0, fp32, c->fj_first[b] + off, c->fj_first_u[b] + off, n, off);
+        return launch_contract_tc(dir, fp32, c->d, c->tcjobs + c->tc_first[b][dir] + off, n, c->tc_img[dir], tf32,
+                                  c->r_scale, c->tc_err, c->stream);
+    };
+    if (part == 0) return run(0, 0, nB);
+    cudaError_t e = run(1, nB, 8);
+    if (e == cudaSuccess && c->pp.glm) {
+        c->launches_tmp++;
+        e = run(0, nB + 8, 1);
+    }
+    return e;
+}
+
 // The one-launch contraction of a small grid: n jobs of sjobs from offset off
 static cudaError_t small_contract(grmhd_ctx* c, int filter, int off, int n) {
     FxsOps o;
@@ -1044,7 +1069,7 @@ static cudaError_t small_contract(grmhd_ctx* c, int filter, int off, int n) {
 // together (863 against 912, and one CTA per SM 828).  SSP-RK3 step 4.59 -> 4.45 ms.
 static int enqueue_first_derivs(grmhd_ctx* c, int b, int part, int second = 0) {
     const int nB = N_D1 + c->pp.glm, off = part == 0 ? 0 : nB, n = part == 0 ? nB : c->job_first_n - nB;
-    const int mixed = c->opts.precision > 0, tf32 = c->opts.precision == 2;
+    const int mixed = c->opts.precision > 0;
     if (c->small_d) {
         CK(small_contract(c, 0, part == 0 ? c->sj_first[b] : c->sj_flux[b], part == 0 ? 3 * n : 24));
         c->launches_tmp++;
@@ -1055,13 +1080,13 @@ static int enqueue_first_derivs(grmhd_ctx* c, int b, int part, int second = 0) {
     }
     for (int k = 0; k < 3 && !c->small_d; k++) {
         const int dir = part == 0 && !mixed ? (k + 2) % 3 : k;
-        if (dir == 1 && c->ft)
-            CK(theta_fourier(c, 0, mixed ? 0 : -1, c->fj_first[b] + off, c->fj_first_u[b] + off, n, off));
-        else if (mixed)
-            CK(launch_contract_tc(dir, 0, c->d, c->tcjobs + c->tc_first[b][dir] + off, n, c->tc_img[dir], tf32,
-                                  c->r_scale, c->tc_err, c->stream));
-        else
+        if (mixed) {
+            CK(first_mixed(c, b, dir, part));
+        } else if (dir == 1 && c->ft) {
+            CK(theta_fourier(c, 0, -1, c->fj_first[b] + off, c->fj_first_u[b] + off, n, off));
+        } else {
             CK(contract(c, dir, 0, c->jobs + c->job_first[b][dir] + off, n, false, part == 0 && dir == 2));
+        }
         c->launches_tmp++;
         if (second && dir == 2 && !mixed) {
             CK(contract(c, 2, 0, c->jobs + c->job_second[2], c->job_second_n[2], false, true));
@@ -1646,15 +1671,15 @@ extern "C" int grmhd_kernel_times(grmhd_ctx* c, int reps, double* ms_out, double
                     if (e == cudaSuccess && c->pp.glm) e = small_contract(c, 0, c->sj_flux[1] + 24 + dir, 1);
                     fl[k] = contraction_flops(c, dir, 0) * c->job_first_n;
                     by[k] = (double)P * c->job_first_n * 16.0;
-                } else if (dir == 1 && c->ft) {
-                    e = theta_fourier(c, 0, mixed ? 0 : -1, c->fj_first[1], c->fj_first_u[1], c->job_first_n);
-                    fl[k] = mixed ? tc_flops(c, dir) * c->job_first_n : contraction_flops(c, dir, 0) * c->job_first_n;
-                    by[k] = (double)P * c->job_first_n * (mixed ? 8.0 + 4.0 : 16.0) + 8.0 * 8.0 * P;
                 } else if (mixed) {
-                    e = launch_contract_tc(dir, 0, c->d, c->tcjobs + c->tc_first[1][dir], c->job_first_n, c->tc_img[dir], tf32,
-                                           c->r_scale, c->tc_err, c->stream);
+                    e = first_mixed(c, 1, dir, 0);
+                    if (e == cudaSuccess) e = first_mixed(c, 1, dir, 1);
                     fl[k] = tc_flops(c, dir) * c->job_first_n;
-                    by[k] = (double)P * c->job_first_n * (8.0 + 4.0) + (dir > 0 ? (8.0 + c->pp.glm) * 4.0 * P : 0.0);
+                    by[k] = (double)P * (c->job_first_n * (8.0 + 4.0) - 8 * 4.0) + (dir > 0 ? (8.0 + c->pp.glm) * 4.0 * P : 0.0);
+                } else if (dir == 1 && c->ft) {
+                    e = theta_fourier(c, 0, -1, c->fj_first[1], c->fj_first_u[1], c->job_first_n);
+                    fl[k] = contraction_flops(c, dir, 0) * c->job_first_n;
+                    by[k] = (double)P * c->job_first_n * 16.0 + 8.0 * 8.0 * P;
                 } else {
                     e = contract(c, dir, 0, c->jobs + c->job_first[1][dir], c->job_first_n);
                     fl[k] = contraction_flops(c, dir, 0) * c->job_first_n;

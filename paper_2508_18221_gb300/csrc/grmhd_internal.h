@@ -23,7 +23,8 @@ enum {
     N_PRIM = 7,     // rho, v^r, v^th, v^ph, eps, p, W
     N_FLUX = 24,    // sqrt(gamma) scriptF^i_v  [dir][var]
     // matter terms.  FP64: sqrt(gamma) times E, S_i, E + S, S^ij, Z v_i v_j - b_i b_j (17);
-    // mixed modes: T^{00},T^{01},T^{02},T^{03},T^{11},T^{12},T^{13},T^{22},T^{23},T^{33} (10)
+    // mixed modes, FP32 (as the fluxes): T^{00},T^{01},T^{02},T^{03},T^{11},T^{12},T^{13},T^{22},
+    // T^{23},T^{33} (10)
     N_TMN = 17,
     N_MET = 10,     // e^{4phi}, e^{-4phi}, sqrt(gamma), gammatilde^ij (6), 1/sqrt(gamma) (FP64)
 };

@@ -577,14 +577,14 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
         R vt[3];
         for (int i = 0; i < 3; i++) vt[i] = alphaR * vR[i] - betaR[i];
         for (int i = 0; i < 3; i++) {
-            double* F = flux + (long long)(i * 8) * P + p;
-            F[0 * P] = widen(sqgR * (Dp * vt[i]));
+            // kept in FP32, as is T^{mu nu}: half the bytes, no conversion here and in the readers
+            R* F = reinterpret_cast<R*>(flux) + (long long)(i * 8) * P + p;
+            F[0 * P] = sqgR * (Dp * vt[i]);
             for (int j = 0; j < 3; j++)
-                F[(1 + j) * P] = widen(sqgR * (Sp[j] * vt[i] + (i == j ? alphaR * pstar : R(0.0)) -
-                                               alphaR * bd[j] * BR[i] * iW));
-            F[4 * P] = widen(sqgR * (taup * vt[i] + alphaR * pstar * vR[i] -
-                                     alphaR * alphaR * b0 * BR[i] * iW));
-            for (int k = 0; k < 3; k++) F[(5 + k) * P] = widen(sqgR * (vt[i] * BR[k] - vt[k] * BR[i]));
+                F[(1 + j) * P] = sqgR * (Sp[j] * vt[i] + (i == j ? alphaR * pstar : R(0.0)) -
+                                         alphaR * bd[j] * BR[i] * iW);
+            F[4 * P] = sqgR * (taup * vt[i] + alphaR * pstar * vR[i] - alphaR * alphaR * b0 * BR[i] * iW);
+            for (int k = 0; k < 3; k++) F[(5 + k) * P] = sqgR * (vt[i] * BR[k] - vt[k] * BR[i]);
         }
         // ---- T^{mu nu}
         R ia2 = ia * ia;
@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
         int n = 0;
         for (int m = 0; m < 4; m++)
             for (int k = m; k < 4; k++, n++)
-                tmn[n * P + p] = widen(rhohs * u4[m] * u4[k] + pstar * gu[m][k] - b4[m] * b4[k]);
+                reinterpret_cast<R*>(tmn)[n * P + p] = rhohs * u4[m] * u4[k] + pstar * gu[m][k] - b4[m] * b4[k];
         }
         }
     }
@@ -619,8 +619,8 @@ template <bool HAM>
 __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const double* __restrict__ U0,
                                              const double* __restrict__ Us,
                                              const double* __restrict__ prim,
-                                             const double* __restrict__ flux,
-                                             const double* __restrict__ tmn,
+                                             const float* __restrict__ flux,
+                                             const float* __restrict__ tmn,
                                              const double* __restrict__ lam,
                                              const double* __restrict__ met,
                                              const float* __restrict__ d1,
@@ -701,12 +701,12 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
 
     // ------------------------------------------------------------ Valencia
     {
-        R T00 = narrow<R>(tmn[0 * P + p]);
-        R T0i[3] = {narrow<R>(tmn[1 * P + p]), narrow<R>(tmn[2 * P + p]), narrow<R>(tmn[3 * P + p])};
+        R T00 = tmn[0 * P + p];
+        R T0i[3] = {tmn[1 * P + p], tmn[2 * P + p], tmn[3 * P + p]};
         R Tij[3][3];
-        Tij[0][0] = narrow<R>(tmn[4 * P + p]); Tij[0][1] = Tij[1][0] = narrow<R>(tmn[5 * P + p]);
-        Tij[0][2] = Tij[2][0] = narrow<R>(tmn[6 * P + p]); Tij[1][1] = narrow<R>(tmn[7 * P + p]);
-        Tij[1][2] = Tij[2][1] = narrow<R>(tmn[8 * P + p]); Tij[2][2] = narrow<R>(tmn[9 * P + p]);
+        Tij[0][0] = tmn[4 * P + p]; Tij[0][1] = Tij[1][0] = tmn[5 * P + p];
+        Tij[0][2] = Tij[2][0] = tmn[6 * P + p]; Tij[1][1] = tmn[7 * P + p];
+        Tij[1][2] = Tij[2][1] = tmn[8 * P + p]; Tij[2][2] = tmn[9 * P + p];
         R beta_d[3];
         for (int i = 0; i < 3; i++)
             beta_d[i] = g[i][0] * beta[0] + g[i][1] * beta[1] + g[i][2] * beta[2];
@@ -791,8 +791,8 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
             double J = 1.0 / r_scale[e];
             double fac = 1.0 / (pp.w_end * J);
             for (int v = 0; v < 8; v++) {
-                double FL = flux[(0 * 8 + v) * P + pl];
-                double FR = flux[(0 * 8 + v) * P + pr_];
+                double FL = widen(flux[(0 * 8 + v) * P + pl]);
+                double FR = widen(flux[(0 * 8 + v) * P + pr_]);
                 double UL = Us[(V_D + v) * P + pl];
                 double UR = Us[(V_D + v) * P + pr_];
                 double Fs = 0.5 * (FL + FR) - 0.5 * lmax * (UR - UL);
@@ -1523,7 +1523,7 @@ cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, co
                        double* ham, int div_parts) {
     int bs = 128;
     long long nb = (d.P + bs - 1) / bs;
-#define RHS_ARGS d, pp, U0, Us, prim, flux, tmn, lam, met, (const float*)d1, (const float*)d2, (const float*)divF, \
+#define RHS_ARGS d, pp, U0, Us, prim, (const float*)flux, (const float*)tmn, lam, met, (const float*)d1, (const float*)d2, (const float*)divF, \
                     (const float*)divB, r_scale_dev, dt_dev, co, out, acc, ham
     if (deriv_fp32) {
         if (ham) k_rhs<true><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
