@@ -22,8 +22,8 @@
 // tile's first loads are issued before the epilogue of the current one.  Several CTAs share
 // an SM up to 64 nodes; at 65 .. 128 their operands fill it, so one CTA of 16 warps
 // works alone.  Per launch on 4,194,304 nodes (32 x 64 x 128 per element), before and after:
-// first derivatives r 473 -> 323, theta 996 -> 449, phi 1,099 -> 657 us; second derivatives
-// 458 -> 262, 506 -> 245, 328 -> 211 us (bit-identical results).
+// first derivatives r 473 -> 292, theta 996 -> 381, phi 1,099 -> 585 us; second derivatives
+// 458 -> 229, 506 -> 190, 328 -> 196 us (bit-identical results).
 #include <cuda_bf16.h>
 #include <stdint.h>
 
@@ -121,13 +121,17 @@ __device__ __forceinline__ void load8(const float* p, uint32_t stride, int n, bo
 // Epilogue: warp w serves tensor-memory lanes 32 (w mod 4) .. and every W-th block of eight
 // columns.  Shared memory (bytes): [A slices | B image | 2 mbarriers | tmem address]
 //   A: nsl x 128 x Kp x es,  B: nsl x Np x Kp x es  (nsl = 3 for BF16 x3, 1 for TF32)
+// CTAs per SM that the registers are cut for
+template <typename TIn>
+__host__ __device__ constexpr int tc_ctas(int W) { return W == 1 ? (sizeof(TIn) == 4 ? 7 : 5) : (W == 2 ? 3 : 1); }
+
 template <int DIR, typename TIn, bool TF32, int W>
-__global__ void __launch_bounds__(128 * W, W == 1 ? 5 : (W == 2 ? 2 : 1))
+__global__ void __launch_bounds__(128 * W, tc_ctas<TIn>(W))
     k_contract_tc(Dims d, const TcJob* __restrict__ jobs, int njobs, const uint8_t* __restrict__ op_img, int N, int Np,
                   int Kp, int tmem_cols, const double* __restrict__ r_scale, int* __restrict__ err) {
     extern __shared__ __align__(1024) uint8_t sm[];
     constexpr int es = TF32 ? 4 : 2, nsl = TF32 ? 1 : 3, NT = 128 * W;
-    constexpr int NB = 2;                                // groups of eight per thread and batch
+    constexpr int NB = W == 4 ? 4 : 2;                                // groups of eight per thread and batch
     const int kcores = Kp * es / 16, ngr = Kp / 8;
     const uint32_t a_bytes = 128u * Kp * es;
     const uint32_t b_bytes = (uint32_t)Np * Kp * es;
@@ -359,9 +363,10 @@ static cudaError_t launch_w(const Dims& d, const TcJob* jobs, int njobs, const u
     const long long nlines = DIR == 0 ? (long long)d.E * d.NtNp : (DIR == 1 ? (long long)d.E * d.Nr * d.Np : d.P / N);
     if (d.P >= (1LL << 31)) return cudaErrorNotSupported;   // 32-bit line arithmetic
     const long long nb = (nlines + 127) / 128;
-    // jobs walked by a CTA: about two rounds of CTAs in all, so that set-up is amortised on
-    // large grids and small ones still fill the chip
-    const long long want = (W == 1 ? 5 : (W == 2 ? 2 : 1)) * 152LL * 2;
+    // jobs walked by a CTA: about eight rounds of CTAs in all.  Fewer rounds leave a longer last
+    // one, one job per CTA repeats the set-up (4.2M nodes, phi first derivatives: 620 us at two
+    // rounds, 618 at four, 585 at eight, 658 at one job each)
+    const long long want = tc_ctas<TIn>(W) * 152LL * 8;
     long long gy = (want + nb - 1) / nb;
     if (gy > njobs) gy = njobs;
     if (gy < 1) gy = 1;
