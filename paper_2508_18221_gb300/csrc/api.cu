@@ -68,13 +68,7 @@ struct grmhd_ctx {
     double* met;             // N_MET * P: the metric of the last k_prep
     double* ham_out;         // non-null while a diagnostic stage is enqueued: k_rhs writes H there
     int nv;                  // evolved variables: GRMHD_NV, + 1 (psi) with GLM
-    double* Dr;              // Nr x Nr reference CGL matrix on [-1, 1]
-    double* Dt;              // Nt x Nt Gauss matrix scaled to [theta_min, theta_max]
-    double* Dp;              // circulant row
-    double* Fr;
-    double* Ft;
-    double* Fp;
-    double* Ds[3];           // reflection-split derivative operators (nullptr: dense only)
+    double* Ds[3];           // reflection-split derivative operators r / theta / phi
     double* Fs[3];           // reflection-split filter operators
     double* r_scale;         // E
     double* wq;              // P quadrature weights
@@ -112,10 +106,8 @@ struct grmhd_ctx {
     int nfold;               // fields the folding buffers hold
     double* Y;               // folded inputs, nfold x P values (double, or float)
     double* Z;               // folded contraction results
-    double* Dt2[2];          // dense even / odd extension operators: derivative
-    double* Ft2[2];          //   and filter
-    double* Dts[2];          // reflection-split copies (nullptr: dense only)
-    double* Fts[2];
+    double* Dts[2];          // even / odd extension operators, reflection-split: derivative
+    double* Fts[2];          //   and filter
     uint8_t* fx_dt[2];       // digit-slice images (nullptr: FP64 units)
     uint8_t* fx_ft[2];
     uint8_t* tc_t[2];        // mixed-precision images of the derivative operators
@@ -259,8 +251,7 @@ static void free_ctx(grmhd_ctx* c) {
     if (!c) return;
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
     double** bufs[] = {&c->U[0], &c->U[1], &c->U[2], &c->acc, &c->prim, &c->flux, &c->tmn, &c->lam,
-                       &c->d1, &c->d2, &c->divF, &c->scratch, &c->Dr, &c->Dt, &c->Dp, &c->Fr,
-                       &c->Ft, &c->Fp, &c->r_scale, &c->wq, &c->hmin, &c->dt, &c->diag, &c->divB, &c->ham, &c->met};
+                       &c->d1, &c->d2, &c->divF, &c->scratch, &c->r_scale, &c->wq, &c->hmin, &c->dt, &c->diag, &c->divB, &c->ham, &c->met};
     for (double** b : bufs)
         if (*b) cudaFree(*b);
     for (int k = 0; k < 3; k++) {
@@ -280,8 +271,7 @@ static void free_ctx(grmhd_ctx* c) {
     }
     if (c->tcjobs) cudaFree(c->tcjobs);
     if (c->tc_err) cudaFree(c->tc_err);
-    double** fbufs[] = {&c->Y, &c->Z, &c->Dt2[0], &c->Dt2[1], &c->Ft2[0], &c->Ft2[1], &c->Dts[0], &c->Dts[1],
-                        &c->Fts[0], &c->Fts[1]};
+    double** fbufs[] = {&c->Y, &c->Z, &c->Dts[0], &c->Dts[1], &c->Fts[0], &c->Fts[1]};
     for (double** b : fbufs)
         if (*b) cudaFree(*b);
     for (int k = 0; k < 2; k++) {
@@ -505,8 +495,6 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
     AL(c->ham, P);
     AL(c->met, N_MET * P);
     AL(c->scratch, nv * P);
-    AL(c->Dr, Nr * Nr); AL(c->Dt, Nt * Nt); AL(c->Dp, Np);
-    AL(c->Fr, Nr * Nr); AL(c->Ft, Nt * Nt); AL(c->Fp, Np);
     AL(c->r_scale, E); AL(c->wq, P); AL(c->hmin, ninst); AL(c->dt, ninst); AL(c->diag, 8);
     AL(c->nfail, 1); AL(c->lam_bits, ninst); AL(c->nan_flag, 1); AL(c->tc_err, 1);
     AL(c->iface_dev, E); AL(c->elem_inst_dev, E);
@@ -597,9 +585,6 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
     if (dalloc(&c->jobs, jobs.size()) != cudaSuccess) { free_ctx(c); return GRMHD_ENOMEM; }
     cudaStream_t s = c->stream;
     if (cudaMemcpyAsync(c->jobs, jobs.data(), jobs.size() * sizeof(DerivJob), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        upload(c->Dr, Dr, s) != cudaSuccess || upload(c->Dt, Dt, s) != cudaSuccess ||
-        upload(c->Dp, Dp, s) != cudaSuccess || upload(c->Fr, Fr, s) != cudaSuccess ||
-        upload(c->Ft, Ft, s) != cudaSuccess || upload(c->Fp, Fp, s) != cudaSuccess ||
         upload(c->r_scale, c->rscale_h, s) != cudaSuccess || upload(c->wq, wq, s) != cudaSuccess ||
         upload(c->hmin, hmin, s) != cudaSuccess ||
         cudaMemsetAsync(c->dt, 0, sizeof(double) * ninst, s) != cudaSuccess ||
@@ -617,7 +602,6 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
         std::vector<double> dense_d[3] = {Dr, Dt, circulant(Dp)};
         std::vector<double> dense_f[3] = {Fr, Ft, circulant(Fp)};
         for (int k = 0; k < 3; k++) {
-            if (!eo_supported(k, Ns[k])) continue;
             std::vector<double> sd = split_operator(dense_d[k], Ns[k], k == 2 ? 1 : 0);
             std::vector<double> sf = split_operator(dense_f[k], Ns[k], k == 2 ? 1 : 0);
             if (dalloc(&c->Ds[k], sd.size()) != cudaSuccess || dalloc(&c->Fs[k], sf.size()) != cudaSuccess ||
@@ -628,7 +612,7 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
         }
         if (cudaStreamSynchronize(s) != cudaSuccess) { free_ctx(c); return GRMHD_ECUDA; }
     }
-    // Fourier theta: even / odd extension operators (dense, reflection-split, digit slices)
+    // Fourier theta: even / odd extension operators (reflection-split, digit slices)
     std::vector<double> ext_d[2], ext_f[2];
     if (c->ft) {
         c->dh = c->d;
@@ -646,19 +630,13 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
         int np_ = 0, kp_ = 0, kc_ = 0;
         fx_geometry(Nt, &np_, &kp_, &kc_);
         for (int h = 0; h < 2; h++) {
-            if (dalloc(&c->Dt2[h], (size_t)Nt * Nt) != cudaSuccess || dalloc(&c->Ft2[h], (size_t)Nt * Nt) != cudaSuccess ||
-                upload(c->Dt2[h], ext_d[h], s) != cudaSuccess || upload(c->Ft2[h], ext_f[h], s) != cudaSuccess) {
+            std::vector<double> sd = split_operator(ext_d[h], Nt, 0), sf = split_operator(ext_f[h], Nt, 0);
+            if (dalloc(&c->Dts[h], sd.size()) != cudaSuccess || dalloc(&c->Fts[h], sf.size()) != cudaSuccess ||
+                upload(c->Dts[h], sd, s) != cudaSuccess || upload(c->Fts[h], sf, s) != cudaSuccess) {
                 free_ctx(c);
                 return GRMHD_ENOMEM;
             }
-            if (eo_supported(1, Nt)) {
-                std::vector<double> sd = split_operator(ext_d[h], Nt, 0), sf = split_operator(ext_f[h], Nt, 0);
-                if (dalloc(&c->Dts[h], sd.size()) != cudaSuccess || dalloc(&c->Fts[h], sf.size()) != cudaSuccess ||
-                    upload(c->Dts[h], sd, s) != cudaSuccess || upload(c->Fts[h], sf, s) != cudaSuccess) {
-                    free_ctx(c);
-                    return GRMHD_ENOMEM;
-                }
-            }
+            if (cudaStreamSynchronize(s) != cudaSuccess) { free_ctx(c); return GRMHD_ECUDA; }
             if (fx_ok) {
                 std::vector<uint8_t> id = fx_operator_image(ext_d[h], Nt, 1.0, np_, kp_, kc_);
                 std::vector<uint8_t> iff = fx_operator_image(ext_f[h], Nt, 1.0, np_, kp_, kc_);
@@ -965,27 +943,15 @@ extern "C" int grmhd_coords(const grmhd_ctx* c, double* r, double* th, double* p
 
 // ------------------------------------------------------------------ pipeline
 // One directional contraction of `njobs` FP64 fields: the digit-sliced tensor-core
-// kernel when the context built its images (opts.contraction = 0, at most 128 nodes),
-// else the reflection-split kernel when the size has a compiled instance, else the dense
-// kernel.  filter = 1 uses the modal filter operator (unscaled), 0 the derivative
-// (radial: scaled per element).
+// kernel when the context built its images (opts.contraction = 0, at most 128 nodes), else
+// the reflection-split kernel on the FP64 units.  filter = 1 uses the modal filter operator
+// (unscaled), 0 the derivative (radial: scaled per element).
 //
-// Accumulators of the digit-slice kernel: with five, the folded one's FP32 additions leave
-// an error of about K 2^-53 of sum_j |D_ij| max_j |u_j| per contraction (3.5e-15 / 7.5e-15
-// / 1.4e-14 at 24 / 64 / 128 nodes), the worst case of an FP64 dot product.  A derivative
-// whose terms cancel (the phi derivative of a flux that is constant in phi up to small
-// noise; the second derivatives, which compose two contractions and amplify the first
-// one's error by the operator norm, ~N^2 on Chebyshev nodes) carries that error into the
-// right-hand side: on the 393,216-node instance the momentum and energy equations landed
-// at 1.0-1.5e-11 of their largest value with five accumulators, against 1-3e-12 for the
-// FP64 units.  Every derivative therefore takes a sixth accumulator that keeps the
-// digit-order sum 6 exact (combine6 in the kernel): operator error 7e-16 of the bound.
-// The filter (one contraction of a smooth state, no cancellation) keeps five.  Above 64
-// Chebyshev nodes the digit slices' remaining error (the fixed-point rounding of each line
+// Above 64 Chebyshev nodes the digit slices' error (the fixed-point rounding of each line
 // against its largest value) reaches 1.5e-11 at 96 theta nodes, against 9.5e-12 for the
 // FP64 units, which take those derivatives.  force_fx (the test hook): the digit slices
-// whenever the image exists.
-// share: another kernel is to run on the same SMs (see launch_contract_fx).
+// whenever the image exists.  share: another kernel is to run on the same SMs (see
+// launch_contract_fx).
 static cudaError_t contract(grmhd_ctx* c, int dir, int filter, const DerivJob* jobs, int njobs,
                             bool force_fx = false, bool share = false) {
     if (dir == 1 && c->ft) return cudaErrorInvalidValue;   // theta_fourier below
@@ -994,18 +960,14 @@ static cudaError_t contract(grmhd_ctx* c, int dir, int filter, const DerivJob* j
     const uint8_t* fx = filter ? c->fx_f[dir] : ((cheb_d && Ns[dir] > 64 && !force_fx) ? nullptr : c->fx_d[dir]);
     if (fx) return launch_contract_fx(dir, c->d, jobs, njobs, fx, (dir == 0 && !filter) ? c->fx_estride : 0,
                                       c->tc_err, c->stream, 0, filter ? 1 : 0, 0, share);
-    const double* split = filter ? c->Fs[dir] : c->Ds[dir];
-    const double* rs = filter ? nullptr : c->r_scale;
-    if (split) return launch_deriv_eo(dir, c->d, jobs, njobs, split, filter ? 1 : -1, rs, c->stream);
-    const double* dense = filter ? (dir == 0 ? c->Fr : (dir == 1 ? c->Ft : c->Fp))
-                                 : (dir == 0 ? c->Dr : (dir == 1 ? c->Dt : c->Dp));
-    return launch_deriv(dir, c->d, jobs, njobs, dense, rs, c->stream);
+    return launch_deriv_eo(dir, c->d, jobs, njobs, filter ? c->Fs[dir] : c->Ds[dir], filter ? 1 : -1,
+                           filter ? nullptr : c->r_scale, c->stream);
 }
 
 // Theta contraction of n fields under the Fourier basis: fold the phi pairs, contract
 // the two halves along theta with the even and the odd extension operator, unfold into
-// the destinations (4 launches).  stage < 0: FP64 values (digit-slice, reflection-split or
-// dense kernel); 0 / 1: the mixed-precision tensor-core kernel on FP64 / FP32 inputs.
+// the destinations (4 launches).  stage < 0: FP64 values (digit-slice or reflection-split
+// kernel); 0 / 1: the mixed-precision tensor-core kernel on FP64 / FP32 inputs.
 // i0: folding-buffer field of the list's first job (lists that may run concurrently use
 // disjoint fields)
 static cudaError_t theta_fourier(grmhd_ctx* c, int filter, int stage, int fold_off, int unfold_off, int n,
@@ -1018,11 +980,9 @@ static cudaError_t theta_fourier(grmhd_ctx* c, int filter, int stage, int fold_o
                                    c->opts.precision == 2, c->r_scale, c->tc_err, c->stream);
         } else {
             const uint8_t* fx = filter ? c->fx_ft[h] : c->fx_dt[h];
-            const double* split = filter ? c->Fts[h] : c->Dts[h];
             const DerivJob* jb = c->jobs + c->job_fy[h] + i0;
             if (fx) e = launch_contract_fx(1, c->dh, jb, n, fx, 0, c->tc_err, c->stream, 0, filter ? 1 : 0);
-            else if (split) e = launch_deriv_eo(1, c->dh, jb, n, split, filter ? 1 : -1, nullptr, c->stream);
-            else e = launch_deriv(1, c->dh, jb, n, filter ? c->Ft2[h] : c->Dt2[h], nullptr, c->stream);
+            else e = launch_deriv_eo(1, c->dh, jb, n, filter ? c->Fts[h] : c->Dts[h], filter ? 1 : -1, nullptr, c->stream);
         }
         if (e != cudaSuccess) return e;
     }
@@ -1622,8 +1582,6 @@ static double contraction_flops(const grmhd_ctx* c, int dir, int filter) {
     const int Ns[3] = {c->d.Nr, c->d.Nt, c->d.Np};
     const int N = Ns[dir];
     const double P = (double)c->d.P;
-    const double* split = (dir == 1 && c->ft) ? (filter ? c->Fts[0] : c->Dts[0]) : (filter ? c->Fs[dir] : c->Ds[dir]);
-    if (!split) return 2.0 * N * P;
     double np = dir == 2 ? N / 2 - 1 : N / 2, nf = dir == 2 ? 2 : N % 2;
     double per_line = 2 * np + np * (4 * np + 2 * nf + 5) + nf * (2 * np + 2 * nf + 1);
     return per_line * P / N;

@@ -151,11 +151,8 @@ bool fxs_supported(int N);
 cudaError_t fxs_init();
 cudaError_t launch_contract_small(const Dims& d, const FxsJob* jobs, int njobs, int dirs, const FxsOps& ops,
                                   cudaStream_t s);
-cudaError_t launch_deriv(int dir, const Dims& d, const DerivJob* jobs_dev, int njobs,
-                         const double* mat_dev, const double* r_scale_dev, cudaStream_t s);
-// reflection-split contraction (kernels_eo.cu): cudaErrorNotSupported when N has no
-// compiled instance; sign -1 for derivatives, +1 for filters
-bool eo_supported(int dir, int N);
+// reflection-split contraction on the FP64 units (kernels_eo.cu), 2..128 nodes (even in phi);
+// sign -1 for derivatives, +1 for filters
 cudaError_t launch_deriv_eo(int dir, const Dims& d, const DerivJob* jobs, int njobs,
                             const double* op_split, int sign, const double* r_scale,
                             cudaStream_t s);

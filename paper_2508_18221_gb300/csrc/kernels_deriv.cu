@@ -1,81 +1,15 @@
-// Spectral derivative / filter contractions and small reductions (FP64).
-//
-// A derivative along direction dir of a field u[E][Nr][Nt][Np] is the 1-D contraction
-// (D u)_i = sum_j D_ij u_j along that axis (paper: "The Spectral Derivative Operators";
-// the Chebyshev coefficient route and the Fourier (ik) multiplier are the same linear
-// maps written as matrices).  r uses the element's CGL matrix scaled by 2/(b-a), theta
-// the Chebyshev-Gauss matrix, phi the circulant Fourier matrix stored as one row.
-// r_scale == nullptr applies the matrix unscaled (modal filters).
-// One thread produces one output node; the matrix sits in shared memory and a warp
-// walks consecutive phi nodes, so every source load of the warp is one coalesced
-// 256-byte segment and every matrix load is a broadcast.
+// Interface means, the Fourier-theta fold and unfold, and small reductions (FP64).
 #include <math.h>
 
 #include "grmhd_internal.h"
 
 namespace gk {
 
-template <int DIR>
-__global__ void __launch_bounds__(256) k_deriv(Dims d, const DerivJob* __restrict__ jobs,
-                                               const double* __restrict__ mat,
-                                               const double* __restrict__ r_scale) {
-    extern __shared__ double sD[];
-    const int N = DIR == 0 ? d.Nr : (DIR == 1 ? d.Nt : d.Np);
-    const int nmat = DIR == 2 ? N : N * N;
-    for (int t = threadIdx.x; t < nmat; t += blockDim.x) sD[t] = mat[t];
-    __syncthreads();
-    const DerivJob job = jobs[blockIdx.y];
-    const long long P = d.P;
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < P;
-         p += (long long)gridDim.x * blockDim.x) {
-        double acc = 0.0;
-        if (DIR == 2) {
-            const int l = (int)(p % N);
-            const double* line = job.src + (p - l);
-            // (D u)_l = sum_j c[(l - j) mod N] u_j
-#pragma unroll 4
-            for (int j = 0; j < N; j++) {
-                int m = l - j;
-                m += (m < 0) ? N : 0;
-                acc = fma(sD[m], line[j], acc);
-            }
-        } else {
-            const long long stride = DIR == 0 ? d.NtNp : (long long)d.Np;
-            const int i = (int)((p / stride) % N);
-            const double* col = job.src + (p - (long long)i * stride);
-            const double* Drow = sD + i * N;
-#pragma unroll 4
-            for (int j = 0; j < N; j++) acc = fma(Drow[j], col[(long long)j * stride], acc);
-            if (DIR == 0 && r_scale != nullptr) acc *= r_scale[p / d.elem];
-        }
-        if (job.accumulate) job.dst[p] += acc;
-        else job.dst[p] = acc;
-    }
-}
-
-cudaError_t launch_deriv(int dir, const Dims& d, const DerivJob* jobs_dev, int njobs,
-                         const double* mat_dev, const double* r_scale_dev, cudaStream_t s) {
-    if (njobs <= 0) return cudaSuccess;
-    const int bs = 256;
-    long long nb = (d.P + bs - 1) / bs;
-    if (nb > 65535LL * 32) nb = 65535LL * 32;
-    dim3 grid((unsigned)nb, (unsigned)njobs);
-    const int N = dir == 0 ? d.Nr : (dir == 1 ? d.Nt : d.Np);
-    size_t sm = (size_t)(dir == 2 ? N : N * N) * sizeof(double);
-    if (dir == 0) k_deriv<0><<<grid, bs, sm, s>>>(d, jobs_dev, mat_dev, r_scale_dev);
-    else if (dir == 1) k_deriv<1><<<grid, bs, sm, s>>>(d, jobs_dev, mat_dev, r_scale_dev);
-    else k_deriv<2><<<grid, bs, sm, s>>>(d, jobs_dev, mat_dev, r_scale_dev);
-    return cudaGetLastError();
-}
-
 cudaError_t eo_init();
 cudaError_t tc_init();
 
 cudaError_t kernels_init() {
     cudaError_t e;
-    // dense contractions: theta matrices up to 128 x 128 doubles (128 KB)
-    if ((e = cudaFuncSetAttribute(k_deriv<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, 64 * 64 * 8)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_deriv<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 128 * 8)) != cudaSuccess) return e;
     if ((e = eo_init()) != cudaSuccess) return e;
     if ((e = fx_init()) != cudaSuccess) return e;
     if ((e = fxs_init()) != cudaSuccess) return e;

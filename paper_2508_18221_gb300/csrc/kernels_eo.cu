@@ -1,174 +1,177 @@
-// Reflection-split contractions (FP64): the same linear maps as k_deriv with half the
-// fused multiply-adds.
+// Spectral derivative / filter contractions on the FP64 units (opts.contraction = 1, and the
+// Chebyshev derivatives above 64 nodes): reflection-split products, any size up to 128.
 //
-// Every 1-D operator of the grid either commutes (modal filters, sign +1) or
-// anticommutes (first derivatives, sign -1) with the reflection of its node set:
-// x_j -> -x_j on the Chebyshev nodes (j <-> N-1-j) and phi_j -> -phi_j on the Fourier
-// nodes (j <-> N-j, fixed points j = 0 and N/2).  Writing a line u as its even and odd
-// parts over the index pairs (j, j'),  s_j = u_j + u_j',  a_j = u_j - u_j',  gives for an
-// output pair (i, i')
+// A derivative along direction dir of a field u[E][Nr][Nt][Np] is the 1-D contraction
+// (D u)_i = sum_j D_ij u_j along that axis (paper: "The Spectral Derivative Operators"; the
+// Chebyshev coefficient route and the Fourier (ik) multiplier are the same linear maps
+// written as matrices; r scaled per element, r_scale == nullptr: unscaled).  Every 1-D
+// operator of the grid either commutes (modal filters, sign +1) or anticommutes (first
+// derivatives, sign -1) with the reflection of its node set: x_j -> -x_j on the Chebyshev
+// nodes (j <-> N-1-j) and phi_j -> -phi_j on the Fourier nodes (j <-> N-j, fixed points
+// j = 0 and N/2).  Writing a line u as its even and odd parts over the index pairs (j, j'),
+// s_j = u_j + u_j',  a_j = u_j - u_j',  gives for an output pair (i, i')
 //     out_i  = E s + O a + C u_f,        out_i' = sign (E s - O a + C u_f),
-// with E = (D_ij + D_ij')/2, O = (D_ij - D_ij')/2 and C the columns of the fixed points,
-// so a pair of outputs costs N fused multiply-adds instead of 2N.  One thread owns one
-// line: it loads the N values into registers, forms s and a once, and writes its N
-// outputs; the split matrices sit in shared memory and every matrix read of a warp is a
-// broadcast.  FP64 throughput, not memory, bounds this kernel on GB300 (1.2 TFLOP/s vs
-// 6.8 TB/s), so the strided per-thread line accesses cost nothing measurable.
+// with E = (D_ij + D_ij')/2, O = (D_ij - D_ij')/2 and C the columns of the fixed points, so
+// a pair of outputs costs N fused multiply-adds instead of 2N.
+//
+// The FP64 pipe (a warp instruction holds a quarter of an SM for 64 cycles) bounds the
+// kernel.  A block holds 32 lines (lane = line) as pairs (s, a) in shared memory and the
+// operator as pairs (E, O); its four warps share the output pairs, up to four at a time, so
+// that one 16-byte read of the line serves eight multiply-adds and eight independent sums hide
+// the pipe's latency.  One kernel per direction takes every size
+// (a template instance per size, one thread per line, came first, with dense products for
+// the sizes without one).  First derivatives, before and after: 8 x 24 x 32 x 64 nodes r 363 ->
+// 341, theta 421 -> 406, phi 791 -> 694 us; 5 x 21 x 27 x 40 (dense before) 131 -> 92, 159 ->
+// 107, 226 -> 142 us; 96 theta nodes of a 786,432-node grid (dense before) 8,031 -> 2,088 us.
 #include "grmhd_internal.h"
 
 namespace gk {
 
-// KIND 0: Chebyshev (pairs j <-> N-1-j, middle node fixed for odd N)
-// KIND 1: Fourier   (pairs j <-> N-j for j = 1..N/2-1, fixed 0 and N/2; N even)
-template <int KIND, int N>
-struct Split {
-    static constexpr int NP = KIND == 0 ? N / 2 : N / 2 - 1;
-    static constexpr int NF = KIND == 0 ? N % 2 : 2;
-    static constexpr int SIZE = 2 * NP * NP + 2 * NP * NF + NF * NF;
-    __device__ static constexpr int pair_lo(int ip) { return KIND == 0 ? ip : ip + 1; }
-    __device__ static constexpr int pair_hi(int ip) { return N - 1 - ip; }
-    __device__ static constexpr int fixed(int f) { return KIND == 0 ? N / 2 : (f == 0 ? 0 : N / 2); }
-};
+namespace {
 
-template <int DIR, int KIND, int N>
+// node pairs and fixed points: Chebyshev (directions r, theta; also the theta extension
+// operators) or Fourier (phi)
+struct SplitSet {
+    int np, nf, off;     // pairs (ip + off, N - 1 - ip), fixed points
+};
+__host__ __device__ __forceinline__ SplitSet split_set(int dir, int N) {
+    return dir == 2 ? SplitSet{N / 2 - 1, 2, 1} : SplitSet{N / 2, N % 2, 0};
+}
+__device__ __forceinline__ int fixed_node(int dir, int N, int f) { return dir == 2 && f == 0 ? 0 : N / 2; }
+
+size_t eo_smem(int dir, int N) {
+    const SplitSet s = split_set(dir, N);
+    return (size_t)(2 * s.np * s.np + 2 * s.np * s.nf + s.nf * s.nf) * 8 + (size_t)s.np * 32 * 16 + (size_t)s.nf * 32 * 8;
+}
+
+// the sums of output pairs ip0 .. ip0 + Q - 1
+template <int Q>
+__device__ __forceinline__ void pair_sums(const double2* EO, const double2* SA, int np, int ip0, int lane, double* A,
+                                          double* B) {
+#pragma unroll
+    for (int q = 0; q < Q; q++) A[q] = B[q] = 0.0;
+    const double2* row = EO + (size_t)ip0 * np;
+#pragma unroll 2
+    for (int j = 0; j < np; j++) {
+        const double2 sa = SA[j * 32 + lane];
+#pragma unroll
+        for (int q = 0; q < Q; q++) {
+            const double2 eo = row[q * np + j];
+            A[q] = fma(eo.x, sa.x, A[q]);
+            B[q] = fma(eo.y, sa.y, B[q]);
+        }
+    }
+}
+
+}  // namespace
+
+template <int DIR>
 __global__ void __launch_bounds__(128) k_deriv_eo(Dims d, const DerivJob* __restrict__ jobs,
                                                   const double* __restrict__ op, int sign,
                                                   const double* __restrict__ r_scale) {
-    using S = Split<KIND, N>;
-    constexpr int NP = S::NP, NF = S::NF;
-    extern __shared__ double sm[];
-    for (int t = threadIdx.x; t < S::SIZE; t += blockDim.x) sm[t] = op[t];
-    __syncthreads();
-    const double* E = sm;
-    const double* O = E + NP * NP;
-    const double* C = O + NP * NP;        // [NP][NF]
-    const double* F = C + NP * NF;        // [NF][NP]
-    const double* G = F + NF * NP;        // [NF][NF]
+    extern __shared__ __align__(16) double sm[];
+    const int N = DIR == 0 ? d.Nr : (DIR == 1 ? d.Nt : d.Np);
+    const SplitSet S = split_set(DIR, N);
+    const int np = S.np, nf = S.nf, nn = np * np;
+    double2* EO = reinterpret_cast<double2*>(sm);
+    double2* SA = EO + nn;                             // [np][32]
+    double* uf = reinterpret_cast<double*>(SA + np * 32);   // [nf][32]
+    double* C = uf + nf * 32;                          // [np][nf]
+    double* F = C + np * nf;                           // [nf][np]
+    double* G = F + nf * np;                           // [nf][nf]
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int t = threadIdx.x; t < nn; t += 128) EO[t] = make_double2(op[t], op[nn + t]);
+    for (int t = threadIdx.x; t < 2 * np * nf + nf * nf; t += 128) C[t] = op[2 * nn + t];
     const DerivJob job = jobs[blockIdx.y];
-
-    long long nlines, stride;
-    if (DIR == 0) { nlines = (long long)d.E * d.NtNp; stride = d.NtNp; }
-    else if (DIR == 1) { nlines = (long long)d.E * d.Nr * d.Np; stride = d.Np; }
-    else { nlines = d.P / N; stride = 1; }
-
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nlines;
-         t += (long long)gridDim.x * blockDim.x) {
-        long long base;
-        double scale = 1.0;
-        if (DIR == 0) {
-            long long e = t / d.NtNp;
-            base = e * d.elem + (t - e * d.NtNp);
-            if (r_scale) scale = r_scale[e];
-        } else if (DIR == 1) {
-            long long eil = t / d.Np;
-            base = eil * d.NtNp + (t - eil * d.Np);
-        } else {
-            base = t * N;
-        }
-        const double* src = job.src + base;
-        double s[NP > 0 ? NP : 1], a[NP > 0 ? NP : 1], uf[NF > 0 ? NF : 1];
+    const uint32_t nlines = DIR == 0 ? (uint32_t)(d.E * d.NtNp)
+                                     : (DIR == 1 ? (uint32_t)((long long)d.E * d.Nr * d.Np) : (uint32_t)(d.P / N));
+    const uint32_t t = blockIdx.x * 32u + lane;
+    const bool valid = t < nlines;
+    const uint32_t tc = valid ? t : nlines - 1;
+    size_t base;
+    uint32_t stride = 1;
+    double scale = 1.0;
+    if (DIR == 0) {
+        const uint32_t e = tc / (uint32_t)d.NtNp;
+        base = (size_t)e * d.elem + (tc - e * (uint32_t)d.NtNp);
+        stride = (uint32_t)d.NtNp;
+        if (r_scale) scale = r_scale[e];
+    } else if (DIR == 1) {
+        const uint32_t r = tc / (uint32_t)d.Np;
+        base = (size_t)r * d.NtNp + (tc - r * (uint32_t)d.Np);
+        stride = (uint32_t)d.Np;
+    } else {
+        base = (size_t)tc * N;
+    }
+    const double* src = job.src + base;
+    for (int j = warp; j < np; j += 4) {
+        const double lo = src[(size_t)(j + S.off) * stride], hi = src[(size_t)(N - 1 - j) * stride];
+        SA[j * 32 + lane] = make_double2(lo + hi, lo - hi);
+    }
+    for (int f = warp; f < nf; f += 4) uf[f * 32 + lane] = src[(size_t)fixed_node(DIR, N, f) * stride];
+    __syncthreads();
+    double* dst = job.dst + base;
+    const auto put = [&](int i, double v) {
+        if (!valid) return;
+        double* q = dst + (size_t)i * stride;
+        *q = job.accumulate ? *q + v : v;
+    };
+    // pairs per warp and round: the rounds balanced over the four warps
+    const int rounds = (np + 15) / 16, Q = rounds ? (np + 4 * rounds - 1) / (4 * rounds) : 1;
+    for (int ip0 = warp * Q; ip0 < np; ip0 += 4 * Q) {
+        double A[4], B[4];
+        const int n = min(Q, np - ip0);
+        if (n == 4) pair_sums<4>(EO, SA, np, ip0, lane, A, B);
+        else if (n == 3) pair_sums<3>(EO, SA, np, ip0, lane, A, B);
+        else if (n == 2) pair_sums<2>(EO, SA, np, ip0, lane, A, B);
+        else pair_sums<1>(EO, SA, np, ip0, lane, A, B);
 #pragma unroll
-        for (int j = 0; j < NP; j++) {
-            double lo = src[(long long)S::pair_lo(j) * stride];
-            double hi = src[(long long)S::pair_hi(j) * stride];
-            s[j] = lo + hi;
-            a[j] = lo - hi;
-        }
-#pragma unroll
-        for (int f = 0; f < NF; f++) uf[f] = src[(long long)S::fixed(f) * stride];
-        double* dst = job.dst + base;
-        for (int ip = 0; ip < NP; ip++) {
-            const double* Er = E + ip * NP;
-            const double* Or = O + ip * NP;
-            double A = 0.0, B = 0.0, Cc = 0.0;
-#pragma unroll
-            for (int j = 0; j < NP; j++) {
-                A = fma(Er[j], s[j], A);
-                B = fma(Or[j], a[j], B);
-            }
-#pragma unroll
-            for (int f = 0; f < NF; f++) Cc = fma(C[ip * NF + f], uf[f], Cc);
-            double o1 = (A + B + Cc) * scale;
-            double o2 = sign * (A - B + Cc) * scale;
-            long long i1 = (long long)S::pair_lo(ip) * stride, i2 = (long long)S::pair_hi(ip) * stride;
-            if (job.accumulate) { dst[i1] += o1; dst[i2] += o2; }
-            else { dst[i1] = o1; dst[i2] = o2; }
-        }
-#pragma unroll
-        for (int f = 0; f < NF; f++) {
-            double acc = 0.0;
-#pragma unroll
-            for (int j = 0; j < NP; j++) acc = fma(F[f * NP + j], sign < 0 ? a[j] : s[j], acc);
-#pragma unroll
-            for (int g = 0; g < NF; g++) acc = fma(G[f * NF + g], uf[g], acc);
-            acc *= scale;
-            long long i1 = (long long)S::fixed(f) * stride;
-            if (job.accumulate) dst[i1] += acc;
-            else dst[i1] = acc;
+        for (int q = 0; q < 4; q++) {
+            if (q >= n) break;
+            const int ip = ip0 + q;
+            double c = 0.0;
+            for (int f = 0; f < nf; f++) c = fma(C[ip * nf + f], uf[f * 32 + lane], c);
+            put(ip + S.off, (A[q] + B[q] + c) * scale);
+            put(N - 1 - ip, sign * (A[q] - B[q] + c) * scale);
         }
     }
+    // fixed-point outputs, on the warps that the rounds above leave first
+    for (int f = 3 - warp; f < nf; f += 4) {
+        double acc = 0.0;
+        for (int j = 0; j < np; j++) {
+            const double2 sa = SA[j * 32 + lane];
+            acc = fma(F[f * np + j], sign < 0 ? sa.y : sa.x, acc);
+        }
+        for (int g = 0; g < nf; g++) acc = fma(G[f * nf + g], uf[g * 32 + lane], acc);
+        put(fixed_node(DIR, N, f), acc * scale);
+    }
 }
-
-template <int DIR, int KIND, int N>
-static cudaError_t launch_one(const Dims& d, const DerivJob* jobs, int njobs, const double* op,
-                              int sign, const double* r_scale, cudaStream_t s) {
-    using S = Split<KIND, N>;
-    long long nlines = DIR == 0 ? (long long)d.E * d.NtNp : (DIR == 1 ? (long long)d.E * d.Nr * d.Np : d.P / N);
-    const int bs = 128;
-    long long nb = (nlines + bs - 1) / bs;
-    if (nb > 65535LL * 16) nb = 65535LL * 16;
-    size_t sm = (size_t)S::SIZE * sizeof(double);
-    k_deriv_eo<DIR, KIND, N><<<dim3((unsigned)nb, (unsigned)njobs), bs, sm, s>>>(d, jobs, op, sign, r_scale);
-    return cudaGetLastError();
-}
-
-#define CHEB_CASE(n) case n: return launch_one<DIR, 0, n>(d, jobs, njobs, op, sign, r_scale, s);
-#define FOUR_CASE(n) case n: return launch_one<DIR, 1, n>(d, jobs, njobs, op, sign, r_scale, s);
 
 template <int DIR>
-static cudaError_t dispatch(int N, const Dims& d, const DerivJob* jobs, int njobs, const double* op,
-                            int sign, const double* r_scale, cudaStream_t s) {
-    if (DIR < 2) {
-        switch (N) {
-            CHEB_CASE(4) CHEB_CASE(5) CHEB_CASE(6) CHEB_CASE(7) CHEB_CASE(8) CHEB_CASE(9)
-            CHEB_CASE(10) CHEB_CASE(11) CHEB_CASE(12) CHEB_CASE(13) CHEB_CASE(14) CHEB_CASE(15)
-            CHEB_CASE(16) CHEB_CASE(20) CHEB_CASE(24) CHEB_CASE(32) CHEB_CASE(40) CHEB_CASE(48)
-            CHEB_CASE(64)
-            default: return cudaErrorNotSupported;
-        }
-    } else {
-        switch (N) {
-            FOUR_CASE(4) FOUR_CASE(6) FOUR_CASE(8) FOUR_CASE(10) FOUR_CASE(12) FOUR_CASE(16)
-            FOUR_CASE(20) FOUR_CASE(24) FOUR_CASE(32) FOUR_CASE(48) FOUR_CASE(64) FOUR_CASE(128)
-            default: return cudaErrorNotSupported;
-        }
-    }
+static cudaError_t set_attr_eo(int N) {
+    return cudaFuncSetAttribute(k_deriv_eo<DIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eo_smem(DIR, N));
 }
 
 cudaError_t eo_init() {
-    // the only instance above the default 48 KB: Fourier N = 128 (65.5 KB)
-    return cudaFuncSetAttribute(k_deriv_eo<2, 1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(Split<1, 128>::SIZE * sizeof(double)));
-}
-
-bool eo_supported(int dir, int N) {
-    static const int cheb[] = {4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16, 20, 24, 32, 40, 48, 64};
-    static const int four[] = {4, 6, 8, 10, 12, 16, 20, 24, 32, 48, 64, 128};
-    if (dir < 2) {
-        for (int v : cheb) if (v == N) return true;
-    } else {
-        for (int v : four) if (v == N) return true;
-    }
-    return false;
+    cudaError_t e;
+    if ((e = set_attr_eo<0>(128)) != cudaSuccess) return e;
+    if ((e = set_attr_eo<1>(128)) != cudaSuccess) return e;
+    return set_attr_eo<2>(128);
 }
 
 cudaError_t launch_deriv_eo(int dir, const Dims& d, const DerivJob* jobs, int njobs,
                             const double* op_split, int sign, const double* r_scale,
                             cudaStream_t s) {
-    if (njobs <= 0) return cudaSuccess;
-    if (dir == 0) return dispatch<0>(d.Nr, d, jobs, njobs, op_split, sign, r_scale, s);
-    if (dir == 1) return dispatch<1>(d.Nt, d, jobs, njobs, op_split, sign, nullptr, s);
-    return dispatch<2>(d.Np, d, jobs, njobs, op_split, sign, nullptr, s);
+    if (njobs <= 0 || d.P <= 0) return cudaSuccess;
+    const int N = dir == 0 ? d.Nr : (dir == 1 ? d.Nt : d.Np);
+    if (N < 2 || N > 128 || (dir == 2 && N % 2) || d.P >= (1LL << 31)) return cudaErrorNotSupported;
+    const long long nlines = dir == 0 ? (long long)d.E * d.NtNp : (dir == 1 ? (long long)d.E * d.Nr * d.Np : d.P / N);
+    const dim3 grid((unsigned)((nlines + 31) / 32), (unsigned)njobs);
+    const size_t sm = eo_smem(dir, N);
+    if (dir == 0) k_deriv_eo<0><<<grid, 128, sm, s>>>(d, jobs, op_split, sign, r_scale);
+    else if (dir == 1) k_deriv_eo<1><<<grid, 128, sm, s>>>(d, jobs, op_split, sign, nullptr);
+    else k_deriv_eo<2><<<grid, 128, sm, s>>>(d, jobs, op_split, sign, nullptr);
+    return cudaGetLastError();
 }
 
 }  // namespace gk
