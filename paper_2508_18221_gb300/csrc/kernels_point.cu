@@ -1055,7 +1055,15 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
 // memory: 254 registers without spills, against 904 B of spills per thread).  Measured on
 // 393,216 nodes, per launch: 1.085 -> 0.603 ms.  MODE: 0 the plain right-hand side, 1 the first SSP-RK3 stage Us + dt L, 2 the
 // others a U0 + b (Us + dt L), 3 RK4 stages.  DIVP: parts of divF to add (1, or 3 on small grids).
-template <int MODE>
+//
+// PART: the variables that an instance writes; what only the others need drops out.  One
+// thread per node cannot run faster than ~950 FP64 instructions in turn, 64 clocks each on
+// an SM quarter (30 us), so grids of few nodes, which leave most quarters idle, give a node
+// to two threads: RHS_A Atilde_ij (the Ricci tensor), RHS_B the rest, with the bits of
+// RHS_ALL.  4,608 nodes: 35.9 -> 22.8 us.
+enum { RHS_A = 1, RHS_B = 2, RHS_ALL = 3 };
+
+template <int MODE, int PART>
 struct Emit {
     const double *U0, *Us;
     double *out, *acc;
@@ -1064,6 +1072,7 @@ struct Emit {
     int acc_mode;
     bool frozen;
     __device__ __forceinline__ void operator()(int v, double L) const {
+        if (!((v >= V_AT && v < V_AT + 6 ? RHS_A : RHS_B) & PART)) return;
         const long long ix = v * P + p;
         if (frozen) L = 0.0;
         if (MODE == 0) out[ix] = L;
@@ -1079,24 +1088,22 @@ struct Emit {
     }
 };
 
-template <int MODE, bool HAM, int DIVP>
-__global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const double* __restrict__ U0,
-                                               const double* __restrict__ Us, const double* __restrict__ flux,
-                                               const double* __restrict__ mat, const double* __restrict__ lam,
-                                               const double* __restrict__ met, const double* __restrict__ d1,
-                                               const double* __restrict__ d2, const double* __restrict__ divF,
-                                               const double* __restrict__ divB, const double* __restrict__ r_scale,
-                                               const double* __restrict__ dt_dev, RKCoef co,
-                                               double* __restrict__ out, double* __restrict__ acc,
-                                               double* __restrict__ ham) {
-    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+template <int MODE, bool HAM, int DIVP, int PART>
+__device__ __forceinline__ void rhs64_node(long long p, const Dims& d, const PhysParams& pp,
+                                           const double* __restrict__ U0, const double* __restrict__ Us,
+                                           const double* __restrict__ flux, const double* __restrict__ mat,
+                                           const double* __restrict__ lam, const double* __restrict__ met,
+                                           const double* __restrict__ d1, const double* __restrict__ d2,
+                                           const double* __restrict__ divF, const double* __restrict__ divB,
+                                           const double* __restrict__ r_scale, const double* __restrict__ dt_dev,
+                                           const RKCoef& co, double* __restrict__ out, double* __restrict__ acc,
+                                           double* __restrict__ ham) {
     const long long P = d.P;
-    if (p >= P) return;
     const int e = (int)(p / d.elem);
     const long long ir = (p / d.NtNp) % d.Nr;
     const double dt = MODE == 0 ? 0.0 : dt_dev[d.elem_inst[e]];
     // the outer boundary node of each instance is frozen
-    const Emit<MODE> emit = {U0, Us, out, acc, P, p, co.a, co.b, co.b * dt, co.c * dt, co.w * dt, co.acc_mode,
+    const Emit<MODE, PART> emit = {U0, Us, out, acc, P, p, co.a, co.b, co.b * dt, co.c * dt, co.w * dt, co.acc_mode,
                              ir == d.Nr - 1 && !d.iface_next[e]};
 #define LD(a, k) __ldg((a) + (long long)(k) * P + p)
 #define D1(f, dd) LD(d1, (f) * 3 + (dd))
@@ -1132,7 +1139,8 @@ __global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const doub
 #pragma unroll
         for (int i = 0; i < 3; i++)
             S_u[i] = gti[SI(i, 0)] * S_d[0] + gti[SI(i, 1)] * S_d[1] + gti[SI(i, 2)] * S_d[2];
-        if (pp.evolve_fluid) {
+        if (!(PART & RHS_B)) {
+        } else if (pp.evolve_fluid) {
             double r[8];
 #pragma unroll
             for (int v = 0; v < 8; v++)
@@ -1496,6 +1504,29 @@ __global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const doub
 #undef D2
 }
 
+// SPLIT: blockIdx.y = 0 Atilde, 1 the rest; else all
+template <int MODE, bool HAM, int DIVP, bool SPLIT>
+__global__ void __launch_bounds__(128) k_rhs64(Dims d, PhysParams pp, const double* __restrict__ U0,
+                                               const double* __restrict__ Us, const double* __restrict__ flux,
+                                               const double* __restrict__ mat, const double* __restrict__ lam,
+                                               const double* __restrict__ met, const double* __restrict__ d1,
+                                               const double* __restrict__ d2, const double* __restrict__ divF,
+                                               const double* __restrict__ divB, const double* __restrict__ r_scale,
+                                               const double* __restrict__ dt_dev, RKCoef co,
+                                               double* __restrict__ out, double* __restrict__ acc,
+                                               double* __restrict__ ham) {
+    const long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (p >= d.P) return;
+#define NODE_ARGS p, d, pp, U0, Us, flux, mat, lam, met, d1, d2, divF, divB, r_scale, dt_dev, co, out, acc, ham
+    if constexpr (SPLIT) {
+        if (blockIdx.y == 0) rhs64_node<MODE, HAM, DIVP, RHS_A>(NODE_ARGS);
+        else rhs64_node<MODE, HAM, DIVP, RHS_B>(NODE_ARGS);
+    } else {
+        rhs64_node<MODE, HAM, DIVP, RHS_ALL>(NODE_ARGS);
+    }
+#undef NODE_ARGS
+}
+
 // --------------------------------------------------------------------------- launchers
 cudaError_t launch_prep(const Dims& d, const PhysParams& pp, const double* U, double* prim,
                         double* flux, double* tmn, double* lam, unsigned long long* nfail, double* met,
@@ -1529,18 +1560,30 @@ cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, co
         if (ham) k_rhs<true><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
         else k_rhs<false><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
     } else {
-        const unsigned g = (unsigned)nb;
-        const auto run = [&](auto k) {
-            k<<<g, bs, 0, s>>>(d, pp, U0, Us, flux, tmn, lam, met, (const double*)d1, (const double*)d2,
-                               (const double*)divF, (const double*)divB, r_scale_dev, dt_dev, co, out, acc, ham);
+        // two threads per node while that still leaves every SM quarter at most one warp
+        int dev = 0, nsm = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        const bool split = div_parts == 3 && d.P * 2 <= 32LL * 4 * nsm;
+        if (split) {   // 32 threads a block: a warp per SM quarter
+            bs = 32;
+            nb = (d.P + bs - 1) / bs;
+        }
+        const auto run = [&](auto k, unsigned y) {
+            k<<<dim3((unsigned)nb, y), bs, 0, s>>>(d, pp, U0, Us, flux, tmn, lam, met, (const double*)d1, (const double*)d2,
+                                                   (const double*)divF, (const double*)divB, r_scale_dev, dt_dev, co, out,
+                                                   acc, ham);
         };
         // (a runtime branch on div_parts cost 4 %: the additions were issued either way)
-        const bool p3 = div_parts == 3;
-        if (ham) p3 ? run(k_rhs64<0, true, 3>) : run(k_rhs64<0, true, 1>);
-        else if (co.acc_mode < 0) p3 ? run(k_rhs64<0, false, 3>) : run(k_rhs64<0, false, 1>);
-        else if (co.acc_mode > 0) p3 ? run(k_rhs64<3, false, 3>) : run(k_rhs64<3, false, 1>);
-        else if (co.a == 0.0 && co.b == 1.0) p3 ? run(k_rhs64<1, false, 3>) : run(k_rhs64<1, false, 1>);
-        else p3 ? run(k_rhs64<2, false, 3>) : run(k_rhs64<2, false, 1>);
+#define RHS64_RUN(MODE) \
+        split ? run(k_rhs64<MODE, false, 3, true>, 2) \
+              : (div_parts == 3 ? run(k_rhs64<MODE, false, 3, false>, 1) : run(k_rhs64<MODE, false, 1, false>, 1))
+        if (ham) div_parts == 3 ? run(k_rhs64<0, true, 3, false>, 1) : run(k_rhs64<0, true, 1, false>, 1);
+        else if (co.acc_mode < 0) RHS64_RUN(0);
+        else if (co.acc_mode > 0) RHS64_RUN(3);
+        else if (co.a == 0.0 && co.b == 1.0) RHS64_RUN(1);
+        else RHS64_RUN(2);
+#undef RHS64_RUN
     }
 #undef RHS_ARGS
     return cudaGetLastError();
