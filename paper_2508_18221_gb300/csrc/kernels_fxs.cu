@@ -31,6 +31,11 @@ __host__ __device__ constexpr int fxs_k4(int N) { return (N + 3) / 4; }
 // the row exponents
 __host__ __device__ constexpr int fxs_words(int N) { return N * fxs_k4(N) * 8; }
 
+template <int V>
+struct Int {
+    static constexpr int value = V;
+};
+
 // bytes b of four 64-bit words as one word (b-th byte of z[0] lowest), biased digits made signed
 __device__ __forceinline__ uint32_t pack_byte(const unsigned long long z[4], int b) {
     const uint32_t sel = (uint32_t)((b & 3) | ((4 + (b & 3)) << 4));
@@ -88,22 +93,35 @@ __global__ void __launch_bounds__(NW * 32) k_contract_small(Dims d, FxsOps ops, 
         const int* f = reinterpret_cast<const int*>(img) + words;
         for (int k = threadIdx.x; k < N; k += NW * 32) sF[o * N + k] = f[k];
     }
+    // loads in batches of eight: all of a batch in flight
     if (dir == 2) {
-        // lines are contiguous: coalesced over the tile
-        const int cnt = (int)min((long long)LN, nl - t0) * N;
-        for (int k = threadIdx.x; k < LN * N; k += NW * 32)
-            sV[(k % N) * 33 + k / N] = k < cnt ? jb.src[t0 * N + k] : 0.0;
-    } else {
-        for (int k = warp; k < N; k += NW) {
-            double v = 0.0;
-            if (valid) {
-                v = jb.src[base + k * stride];
-                if (dir == 3) {
-                    const double w = jb.src[base + h + k * stride];
-                    v = lane < 16 ? v + w : v - w;
-                }
+        // lines are contiguous: a warp reads its lines along their length
+        const int cnt = (int)min((long long)LN, nl - t0);
+        for (int k = lane; k < N; k += 32) {
+            double v[LN / NW];
+#pragma unroll
+            for (int q = 0; q < LN / NW; q++) {
+                const int l = warp + q * NW;
+                v[q] = l < cnt ? jb.src[(t0 + l) * N + k] : 0.0;
             }
-            sV[k * 33 + lane] = v;
+#pragma unroll
+            for (int q = 0; q < LN / NW; q++) sV[k * 33 + warp + q * NW] = v[q];
+        }
+    } else {
+        for (int k0 = warp; k0 < N; k0 += 8 * NW) {
+            double v[8], w[8];
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const int k = k0 + q * NW;
+                const bool on = valid && k < N;
+                v[q] = on ? jb.src[base + k * stride] : 0.0;
+                w[q] = on && dir == 3 ? jb.src[base + h + k * stride] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const int k = k0 + q * NW;
+                if (k < N) sV[k * 33 + lane] = dir == 3 ? (lane < 16 ? v[q] + w[q] : v[q] - w[q]) : v[q];
+            }
         }
     }
     __syncthreads();
@@ -123,20 +141,7 @@ __global__ void __launch_bounds__(NW * 32) k_contract_small(Dims d, FxsOps ops, 
     __syncthreads();
     const uint32_t* B = sB + (dir == 3 && lane >= 16 ? words : 0);
     const int* F = sF + (dir == 3 && lane >= 16 ? N : 0);
-    for (int i = warp; i < N; i += NW) {
-        int acc[7] = {0, 0, 0, 0, 0, 0, 0};
-#pragma unroll 2
-        for (int g = 0; g < K4; g++) {
-            const uint4 b0 = *reinterpret_cast<const uint4*>(B + (i * K4 + g) * 8);
-            const uint4 b1 = *reinterpret_cast<const uint4*>(B + (i * K4 + g) * 8 + 4);
-            const uint32_t b[7] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z};
-#pragma unroll
-            for (int q = 0; q < 7; q++) {
-                const int a = (int)sA[(g * 7 + q) * 32 + lane];
-#pragma unroll
-                for (int l = 0; l < 7 - q; l++) acc[q + l] = __dp4a(a, (int)b[l], acc[q + l]);
-            }
-        }
+    const auto finish = [&](const int* acc, int i) {
         // sum_s n_s 2^(8 (7 - s)), the s = 8 term rounded half up: the integer of kernels_fx.cu
         long long R = (long long)acc[0] << 40;
         R += (long long)acc[1] << 32;
@@ -149,6 +154,10 @@ __global__ void __launch_bounds__(NW * 32) k_contract_small(Dims d, FxsOps ops, 
         double v = scale_int_fast(R, X, &ok);
         if (!ok) v = R == 0 ? 0.0 : ldexp_int(R, X);
         if (EL == 0x7FF) v = __longlong_as_double(0x7FF8000000000000ll);
+        if (dir == 2) {
+            sV[i * 33 + lane] = v;     // (the digits are formed: the values are no longer read)
+            return;
+        }
         if (dir == 3) {
             const double o = __shfl_xor_sync(0xffffffffu, v, 16);
             v = lane < 16 ? v + o : o - v;
@@ -157,6 +166,53 @@ __global__ void __launch_bounds__(NW * 32) k_contract_small(Dims d, FxsOps ops, 
             double* q = jb.dst + base + (dir == 3 && lane >= 16 ? h : 0) + i * stride;
             *q = jb.accumulate ? *q + v : v;
         }
+    };
+    // two output rows at a time share the line's digit words, a last odd one goes alone
+    const auto rows = [&](auto nr, int i) {
+        constexpr int NR = decltype(nr)::value;
+        int acc[NR][7];
+#pragma unroll
+        for (int r = 0; r < NR; r++)
+#pragma unroll
+            for (int q = 0; q < 7; q++) acc[r][q] = 0;
+#pragma unroll 2
+        for (int g = 0; g < K4; g++) {
+            uint32_t b[NR][7];
+#pragma unroll
+            for (int r = 0; r < NR; r++) {
+                const uint4* w = reinterpret_cast<const uint4*>(B + ((i + r * NW) * K4 + g) * 8);
+                const uint4 b0 = w[0], b1 = w[1];
+                b[r][0] = b0.x; b[r][1] = b0.y; b[r][2] = b0.z; b[r][3] = b0.w;
+                b[r][4] = b1.x; b[r][5] = b1.y; b[r][6] = b1.z;
+            }
+#pragma unroll
+            for (int q = 0; q < 7; q++) {
+                const int a = (int)sA[(g * 7 + q) * 32 + lane];
+#pragma unroll
+                for (int r = 0; r < NR; r++)
+#pragma unroll
+                    for (int l = 0; l < 7 - q; l++) acc[r][q + l] = __dp4a(a, (int)b[r][l], acc[r][q + l]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < NR; r++) finish(acc[r], i + r * NW);
+    };
+    for (int i = warp; i < N; i += 2 * NW) {
+        if (i + NW < N) rows(Int<2>(), i);
+        else rows(Int<1>(), i);
+    }
+    if (dir == 2) {
+        // along phi the results go out line by line, as the values came in
+        __syncthreads();
+        const int cnt = (int)min((long long)LN, nl - t0);
+        for (int k = lane; k < N; k += 32)
+#pragma unroll
+            for (int q = 0; q < LN / NW; q++) {
+                const int l = warp + q * NW;
+                if (l >= cnt) continue;
+                double* o = jb.dst + (t0 + l) * N + k;
+                *o = jb.accumulate ? *o + sV[k * 33 + l] : sV[k * 33 + l];
+            }
     }
 }
 
