@@ -386,8 +386,7 @@ __device__ __forceinline__ void fluxes64(long long p, long long P, double alpha,
 // or FP32.  Bound by the FP64 pipe (87 % busy): 346 FP64 instructions per node against 707
 // in FP64, so the launch inside the stepping of 393,216 nodes went from 545 to 283 us (ncu),
 // the FP32 form from 340 to 234 us, the recovery of a newly loaded state (grmhd_con2prim,
-// whole call) from 807 to 247 us.  Three blocks per SM (168 registers) hide the serial
-// chains of the root finding better than two of 182 registers do.
+// whole call) from 807 to 247 us.  Three blocks per SM (168 registers).
 enum { PREP_PRIM = 0, PREP_F64 = 1, PREP_F32 = 2 };
 
 template <int WHAT>
@@ -613,10 +612,12 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
 
 // The mixed modes' right-hand side (FP32 algebra; FP64 runs k_rhs64 below).  Bound by memory
 // and latency, not by arithmetic, so it keeps the four-dimensional form of the matter terms.
-// Capped at 170 registers (3 blocks per SM): its spills cost less than the latency its
-// extra warps hide (measured 0.23 -> 0.18 ms on 393k nodes).
-template <bool HAM>
-__global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const double* __restrict__ U0,
+// Each variable is written as soon as it is known, as in k_rhs64 (MODE likewise), and two
+// blocks per SM have the registers to do it without spills: 393,216 nodes 144 -> 101 us (about
+// 5.6 TB/s of its ~1.4 KB per node); three blocks of 168 registers with 500 B of spills a
+// thread take 142 us, four 156 us.
+template <int MODE, bool HAM>
+__global__ void __launch_bounds__(128, 2) k_rhs(Dims d, PhysParams pp, const double* __restrict__ U0,
                                              const double* __restrict__ Us,
                                              const double* __restrict__ prim,
                                              const float* __restrict__ flux,
@@ -637,8 +638,29 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
     if (p >= P) return;
     const R PI = R(3.141592653589793);
     const R third = R(1.0 / 3.0), sixth = R(1.0 / 6.0), two3 = R(2.0 / 3.0);
-    const int nv = NV + pp.glm;
-    R rhs[NV_MAX];
+    const int elem_id = (int)((uint32_t)p / (uint32_t)d.elem);
+    const uint32_t ir = ((uint32_t)p / (uint32_t)d.NtNp) % (uint32_t)d.Nr;
+    // frozen outer boundary node of each instance
+    const bool frozen = ir == (uint32_t)d.Nr - 1 && !d.iface_next[elem_id];
+    const double dt = MODE == 0 ? 0.0 : dt_dev[d.elem_inst[elem_id]];
+    // a variable is written as soon as its right-hand side is known
+    const auto emit = [&](int v, R r) {
+        const long long ix = v * P + p;
+        const double L = frozen ? 0.0 : widen(r);
+        if (MODE == 0) { out[ix] = L; return; }
+        double o;
+        if (MODE == 1) o = Us[ix] + dt * L;
+        else if (MODE == 2) o = co.a * U0[ix] + co.b * (Us[ix] + dt * L);
+        else {
+            // RK4: next stage input U0 + c dt L, accumulator acc (+)= w dt L;
+            // final stage (acc_mode 3): U0 + acc + w dt L
+            const double wl = co.w * dt * L;
+            if (co.acc_mode == 1) { acc[ix] = wl; o = U0[ix] + co.c * dt * L; }
+            else if (co.acc_mode == 2) { acc[ix] += wl; o = U0[ix] + co.c * dt * L; }
+            else { o = U0[ix] + (acc[ix] + wl); }
+        }
+        out[ix] = o;
+    };
 
     // ------------------------------------------------------------ state and metric
     R gt[3][3], At[3][3];
@@ -701,6 +723,7 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
 
     // ------------------------------------------------------------ Valencia
     {
+        R rv[NV_MAX - V_D];
         R T00 = tmn[0 * P + p];
         R T0i[3] = {tmn[1 * P + p], tmn[2 * P + p], tmn[3 * P + p]};
         R Tij[3][3];
@@ -748,7 +771,7 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
             const R tdg = e4r * (sT + f4 * gtw[2]);
             R t0db = T0_d[0] * dbe[jd][0] + T0_d[1] * dbe[jd][1] + T0_d[2] * dbe[jd][2];
             R SS = T00 * (R(0.5) * bbdg - alpha * dal[jd]) + t0dg + t0db + R(0.5) * tdg;
-            rhs[V_S + jd] = -(R)divF[(1 + jd) * P + p] + asg * SS;
+            rv[V_S - V_D + jd] = -(R)divF[(1 + jd) * P + p] + asg * SS;
         }
         R bbK = R(0.0), TK = R(0.0), t0 = R(0.0);
         for (int k = 0; k < 3; k++)
@@ -762,9 +785,9 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
         }
         R bda = beta[0] * dal[0] + beta[1] * dal[1] + beta[2] * dal[2];
         R Stau = T00 * (bbK - bda) + t0 + TK;
-        rhs[V_D] = -(R)divF[0 * P + p];
-        rhs[V_TAU] = -(R)divF[4 * P + p] + asg * Stau;
-        for (int k = 0; k < 3; k++) rhs[V_B + k] = -(R)divF[(5 + k) * P + p];
+        rv[0] = -(R)divF[0 * P + p];
+        rv[V_TAU - V_D] = -(R)divF[4 * P + p] + asg * Stau;
+        for (int k = 0; k < 3; k++) rv[V_B - V_D + k] = -(R)divF[(5 + k) * P + p];
         // GLM cleaning: d_t psi = alpha (-c_h^2 D_i B^i - psi / tau) with the covariant
         // divergence d_i(sqrt(gamma) B^i) / sqrt(gamma); field source -alpha sqrt(gamma)
         // gamma^ij d_j psi (d psi: d1 field N_D1)
@@ -772,17 +795,16 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
             const R psi = narrow<R>(Us[(long long)V_PSI * P + p]);
             R dpsi[3];
             for (int k = 0; k < 3; k++) dpsi[k] = (R)d1[((long long)N_D1 * 3 + k) * P + p];
-            rhs[V_PSI] = alpha * (-narrow<R>(pp.glm_ch2) * (R)divB[p] / sqg - psi * narrow<R>(pp.glm_itau));
+            rv[V_PSI - V_D] = alpha * (-narrow<R>(pp.glm_ch2) * (R)divB[p] / sqg - psi * narrow<R>(pp.glm_itau));
             for (int i = 0; i < 3; i++)
-                rhs[V_B + i] -= asg * (gi[i][0] * dpsi[0] + gi[i][1] * dpsi[1] + gi[i][2] * dpsi[2]);
+                rv[V_B - V_D + i] -= asg * (gi[i][0] * dpsi[0] + gi[i][1] * dpsi[1] + gi[i][2] * dpsi[2]);
         }
 
         // interface penalty (Rusanov flux, strong form) at duplicated element-end nodes
         const long long shell = d.NtNp;
-        const long long ir = (p / shell) % d.Nr;
-        const int e = (int)(p / d.elem);
+        const int e = elem_id;
         int side = 0;
-        if (ir == d.Nr - 1 && d.iface_next[e]) side = +1;
+        if (ir == (uint32_t)d.Nr - 1 && d.iface_next[e]) side = +1;
         if (ir == 0 && e > 0 && d.iface_next[e - 1]) side = -1;
         if (side != 0) {
             long long pl = side > 0 ? p : p - shell;
@@ -796,10 +818,14 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
                 double UL = Us[(V_D + v) * P + pl];
                 double UR = Us[(V_D + v) * P + pr_];
                 double Fs = 0.5 * (FL + FR) - 0.5 * lmax * (UR - UL);
-                if (side > 0) rhs[V_D + v] += narrow<R>((FL - Fs) * fac);
-                else rhs[V_D + v] -= narrow<R>((FR - Fs) * fac);
+                if (side > 0) rv[v] += narrow<R>((FL - Fs) * fac);
+                else rv[v] -= narrow<R>((FR - Fs) * fac);
             }
         }
+
+#pragma unroll
+        for (int v = 0; v < 8; v++) emit(V_D + v, pp.evolve_fluid ? rv[v] : R(0));
+        if (pp.glm) emit(V_PSI, pp.evolve_fluid ? rv[V_PSI - V_D] : R(0));
 
         // matter terms for BSSN: rho = alpha^2 T^00, S_i = alpha T^0_i,
         // S_ij = g_{i mu} g_{j nu} T^{mu nu}
@@ -942,13 +968,13 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
                         la += At[i][k] * dbe[j][k] + At[j][k] * dbe[i][k];
                         AAd += At[i][k] * Aud[k][j];
                     }
-                    rhs[V_GT + sij] = -R(2.0) * alpha * At[i][j] + adv_g + lg - two3 * gt[i][j] * divb;
+                    emit(V_GT + sij, -R(2.0) * alpha * At[i][j] + adv_g + lg - two3 * gt[i][j] * divb);
                     R XTF = X[i][j] - gt[i][j] * trX3;
-                    rhs[V_AT + sij] = e4mr * XTF + alpha * (K * At[i][j] - R(2.0) * AAd) + adv_a + la -
-                                      two3 * At[i][j] * divb;
+                    emit(V_AT + sij, e4mr * XTF + alpha * (K * At[i][j] - R(2.0) * AAd) + adv_a + la -
+                                      two3 * At[i][j] * divb);
                 }
-            rhs[V_PHI] = -alpha * K * sixth + (beta[0] * dphi[0] + beta[1] * dphi[1] + beta[2] * dphi[2]) +
-                         divb * sixth;
+            emit(V_PHI, -alpha * K * sixth + (beta[0] * dphi[0] + beta[1] * dphi[1] + beta[2] * dphi[2]) +
+                         divb * sixth);
             // diagnostics only: the Hamiltonian constraint R + (2/3) K^2 - Atilde.Atilde - 16 pi rho,
             // with R = gamma^ij R_ij = (e^{-4 phi} trX + trDDal) / alpha + 8 pi S (trX, trDDal
             // as above: the same Ricci tensor, no extra derivative)
@@ -956,8 +982,8 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
             if constexpr (HAM)
                 ham[p] = widen((e4mr * trX + trDDal) / alpha + R(8.0) * PI * Str + two3 * K * K - AA -
                                R(16.0) * PI * rho_m);
-            rhs[V_K] = -trDDal + alpha * (AA + K * K3) + R(4.0) * PI * alpha * (rho_m + Str) +
-                       (beta[0] * dK[0] + beta[1] * dK[1] + beta[2] * dK[2]);
+            emit(V_K, -trDDal + alpha * (AA + K * K3) + R(4.0) * PI * alpha * (rho_m + Str) +
+                       (beta[0] * dK[0] + beta[1] * dK[1] + beta[2] * dK[2]));
             // Gammatilde
             R ddb[3][3][3];  // [q pair via j,k][i]
             for (int j = 0; j < 3; j++)
@@ -980,60 +1006,23 @@ __global__ void __launch_bounds__(128, 3) k_rhs(Dims d, PhysParams pp, const dou
                 R Adp = Auu[i][0] * dphi[0] + Auu[i][1] * dphi[1] + Auu[i][2] * dphi[2];
                 R gdK = gti[i][0] * dK[0] + gti[i][1] * dK[1] + gti[i][2] * dK[2];
                 R gS = gti[i][0] * S_i[0] + gti[i][1] * S_i[1] + gti[i][2] * S_i[2];
-                rhs[V_GAM + i] = s + s2 * third + adv - gdb + two3 * Gam[i] * divb - R(2.0) * Ada +
+                const R rg = s + s2 * third + adv - gdb + two3 * Gam[i] * divb - R(2.0) * Ada +
                                  R(2.0) * alpha * (CA + R(6.0) * Adp - two3 * gdK) -
                                  R(16.0) * PI * alpha * gS;
+                emit(V_GAM + i, rg);
+                emit(V_BG + i, pp.gauge == 0 ? rg - narrow<R>(pp.eta) * Bg[i] : R(0.0));
             }
 #undef D2
             if (pp.gauge == 0) {
-                rhs[V_ALPHA] = -R(2.0) * alpha * K + beta[0] * dal[0] + beta[1] * dal[1] + beta[2] * dal[2];
-                for (int i = 0; i < 3; i++) {
-                    rhs[V_BETA + i] = R(0.75) * Bg[i];
-                    rhs[V_BG + i] = rhs[V_GAM + i] - narrow<R>(pp.eta) * Bg[i];
-                }
+                emit(V_ALPHA, -R(2.0) * alpha * K + beta[0] * dal[0] + beta[1] * dal[1] + beta[2] * dal[2]);
+                for (int i = 0; i < 3; i++) emit(V_BETA + i, R(0.75) * Bg[i]);
             } else {
-                rhs[V_ALPHA] = R(0.0);
-                for (int i = 0; i < 3; i++) rhs[V_BETA + i] = rhs[V_BG + i] = R(0.0);
+                emit(V_ALPHA, R(0.0));
+                for (int i = 0; i < 3; i++) emit(V_BETA + i, R(0.0));
             }
         } else {
-            for (int v = 0; v < N_BSSN; v++) rhs[v] = R(0.0);
+            for (int v = 0; v < N_BSSN; v++) emit(v, R(0.0));
         }
-    }
-
-    if (!pp.evolve_fluid)
-        for (int v = V_D; v < nv; v++) rhs[v] = R(0);
-    // frozen outer boundary node of each instance
-    const int elem_id = (int)(p / d.elem);
-    {
-        const long long ir = (p / d.NtNp) % d.Nr;
-        if (ir == d.Nr - 1 && !d.iface_next[elem_id])
-            for (int v = 0; v < nv; v++) rhs[v] = R(0);
-    }
-
-    // ------------------------------------------------------------ output
-    const double dt = dt_dev ? dt_dev[d.elem_inst[elem_id]] : 0.0;
-    if (co.acc_mode < 0) {
-        for (int v = 0; v < nv; v++) out[v * P + p] = widen(rhs[v]);
-        return;
-    }
-    for (int v = 0; v < nv; v++) {
-        long long ix = v * P + p;
-        double L = widen(rhs[v]);
-        double o;
-        if (co.acc_mode == 0) {
-            // SSP-RK3 (Shu-Osher): a U0 + b (Us + dt L); the first stage (a = 0, b = 1) is
-            // Us + dt L alone (a uniform branch: two FP64 operations fewer per output)
-            if (co.a == 0.0 && co.b == 1.0) o = Us[ix] + dt * L;
-            else o = (co.a != 0.0 ? co.a * U0[ix] : 0.0) + co.b * (Us[ix] + dt * L);
-        } else {
-            // RK4: next stage input U0 + c dt L, accumulator acc (+)= w dt L;
-            // final stage (acc_mode 3): U0 + acc + w dt L
-            double wl = co.w * dt * L;
-            if (co.acc_mode == 1) { acc[ix] = wl; o = U0[ix] + co.c * dt * L; }
-            else if (co.acc_mode == 2) { acc[ix] += wl; o = U0[ix] + co.c * dt * L; }
-            else { o = U0[ix] + (acc[ix] + wl); }
-        }
-        out[ix] = o;
     }
 }
 
@@ -1557,8 +1546,12 @@ cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, co
 #define RHS_ARGS d, pp, U0, Us, prim, (const float*)flux, (const float*)tmn, lam, met, (const float*)d1, (const float*)d2, (const float*)divF, \
                     (const float*)divB, r_scale_dev, dt_dev, co, out, acc, ham
     if (deriv_fp32) {
-        if (ham) k_rhs<true><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
-        else k_rhs<false><<<(unsigned)nb, bs, 0, s>>>(RHS_ARGS);
+        const unsigned g = (unsigned)nb;
+        if (ham) k_rhs<0, true><<<g, bs, 0, s>>>(RHS_ARGS);
+        else if (co.acc_mode < 0) k_rhs<0, false><<<g, bs, 0, s>>>(RHS_ARGS);
+        else if (co.acc_mode > 0) k_rhs<3, false><<<g, bs, 0, s>>>(RHS_ARGS);
+        else if (co.a == 0.0 && co.b == 1.0) k_rhs<1, false><<<g, bs, 0, s>>>(RHS_ARGS);
+        else k_rhs<2, false><<<g, bs, 0, s>>>(RHS_ARGS);
     } else {
         // two threads per node while that still leaves every SM quarter at most one warp
         int dev = 0, nsm = 0;
