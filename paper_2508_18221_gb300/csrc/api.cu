@@ -35,11 +35,14 @@ struct NvtxRange {
     ~NvtxRange() { nvtxRangePop(); }
 };
 
-// nodes x (N_r + N_theta + N_phi) up to which a grid's contractions run on the integer units.
-// A time step in us, integer units / tensor cores: 4,608 nodes (2 x 12 x 12 x 16) 224 / 351,
-// 18,432 (8 x 12 x 12 x 16) 318 / 461, 36,864 (2 x 24 x 24 x 32: 2.9e6) 615 / 662, 32,768
-// (1 x 32 x 32 x 32: 3.1e6) 594 / 590, 65,536 (8 x 16 x 16 x 32: 4.2e6) 1,046 / 1,032
-static const long long FXS_MAX_WORK = 3000000;
+// Sizes up to which a grid's contractions run on the integer units: nodes x (N_r + N_theta +
+// N_phi), the products in all, and nodes x N^2 of the longest direction, whose dot products
+// outgrow the tensor cores' padding first.  An SSP-RK3 step in us, integer units / tensor
+// cores: 4,608 nodes (2 x 12 x 12 x 16) 172 / 300; 36,864 (8 x 12 x 12 x 32: 2.1e6, 3.8e7)
+// 581 / 620; 36,864 (2 x 24 x 24 x 32: 2.9e6, 3.8e7) 585 / 601; beyond one bound or the other
+// 65,536 (8 x 16 x 16 x 32: 4.2e6, 6.7e7) 1,022 / 952; 18,432 (2 x 12 x 12 x 64: 1.6e6, 7.5e7)
+// 506 / 421; 30,720 (1 x 20 x 48 x 32: 3.1e6, 7.1e7) 600 / 589
+static const long long FXS_MAX_WORK = 3000000, FXS_MAX_SQUARE = 40000000;
 
 struct grmhd_ctx {
     grmhd_grid grid;
@@ -480,7 +483,8 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
     // small grids take the one-launch contractions: where a launch of the tensor-core kernel,
     // 10-15 us however small, costs more than the products on the integer units.  The bits
     // are the same, so an instance evolves alike alone and in a batch
-    c->small_f = P * (Nr + Nt + Np) <= FXS_MAX_WORK && opts->contraction == 0 && fxs_supported(Nr) && fxs_supported(Nt) &&
+    const long long Nmax = std::max(Nr, std::max(Nt, Np));
+    c->small_f = P * (Nr + Nt + Np) <= FXS_MAX_WORK && P * Nmax * Nmax <= FXS_MAX_SQUARE && opts->contraction == 0 && fxs_supported(Nr) && fxs_supported(Nt) &&
                  fxs_supported(Np) && (!c->ft || (Np / 2) % 2 == 0);
     c->small_d = c->small_f && opts->precision == 0;
     const int ndiv = c->small_d ? 3 : 1;

@@ -9,7 +9,8 @@
 // every direction, with a block of four warps per 32 lines: lane = line, warps share the
 // output rows.  Measured on 4,608 nodes (2 x 12 x
 // 12 x 16): the derivative chain of a right-hand side (six contractions and four interface
-// launches, 92 us) becomes two of 6-13 us and two of 4 us; an SSP-RK3 step 351 -> 224 us.
+// launches, 92 us) becomes two of 6-13 us and two of 4 us; an SSP-RK3 step 351 -> 224 us
+// (172 now).
 //
 // Work of a block: values to shared memory, line exponents, digit bytes packed four along
 // the line (one 32-bit word per digit), then per output row 7 K dot products and the

@@ -21,7 +21,8 @@ SPHERE = dict(theta_min=0.0, theta_max=math.pi, theta_basis=1)
     ((3, 9, 11, 6), {}, dict(integrator=1)),                     # odd node counts, RK4
     ((1, 4, 4, 4), {}, dict(filter=63)),                         # smallest; theta filter on every variable
     ((2, 5, 33, 10), {}, dict(glm=1, filter=0)),                 # GLM, no filter, a line of 33 (nine words)
-    ((1, 7, 64, 34), {}, dict(filter=34, coupling=1)),           # longest theta line; one direction per group
+    ((1, 7, 64, 34), {}, dict(filter=34, coupling=1)),           # one direction per group
+    ((1, 5, 64, 6), {}, dict(filter=34, coupling=1)),            # longest theta line
     ((2, 64, 5, 8), {}, dict(evolve_metric=0)),                  # longest radial line
     ((2, 6, 8, 64), {}, dict(precision=1)),                      # mixed: the filter alone takes this path
     ((2, 7, 9, 8), SPHERE, dict(filter=63)),                     # Fourier theta: fold inside the kernel
