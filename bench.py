@@ -396,32 +396,37 @@ def run_reference(args):
 # (2 x DFMA + DADD + DMUL, smsp__sass_thread_inst_executed_op_d{fma,add,mul}_pred_on.sum)
 # on the 393,216-node workload; the kernels recompute nothing, so this is their algorithmic
 # FP64 work.  The primitive-recovery count is taken inside the time stepping (Newton
-# started from the previous stage's primitives); k_prep<float> (mixed modes) forms the
+# started from the previous stage's primitives); k_prep<PREP_F32> (mixed modes) forms the
 # fluxes and T^{mu nu} in FP32, so only its metric and primitive recovery count.
-FP64_FLOPS_PER_NODE = {"k_rhs<double>": 2501.0, "k_prep<double>": 1050.0, "k_prep<float>": 711.0}
+FP64_FLOPS_PER_NODE = {"k_rhs64": 1656.0, "k_prep<PREP_F64>": 509.0, "k_prep<PREP_F32>": 322.0}
 # Nominal FP64 peak of GB300 from its unit counts and clock: 152 SMs x 2 DFMA/clk x 2 flop
 # x 2.07 GHz (a probe of dependent DFMA chains on all SMs measured 1.198 TFLOP/s).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# bytes per node of the mixed-precision pointwise RHS: state, stage input and T^{mu nu}
-# (FP64), first/second derivatives and flux divergence (FP32) in, stage output out
-RHS32_BYTES_PER_NODE = 8 * (32 + 32 + 10) + 4 * (63 + 66 + 8) + 8 * 32
+# bytes per node of the mixed-precision pointwise RHS: state, stage input and metric (FP64),
+# T^{mu nu}, first/second derivatives and flux divergence (FP32) in, stage output out
+RHS32_BYTES_PER_NODE = 8 * (32 + 32 + 9) + 4 * (10 + 63 + 66 + 8) + 8 * 32
+# a grid's contractions run on the integer units (k_contract_small) up to these bounds on
+# nodes x (N_r + N_theta + N_phi) and nodes x max(N)^2
+SMALL_WORK, SMALL_SQUARE = 3000000, 40000000
 
 
 def _kernel_names(cfg, precision):
     """class of grmhd_kernel_times -> kernel (template instance) that runs it."""
     ns = (cfg.n_r, cfg.n_theta, cfg.n_phi)
-    names = {"prep": "k_prep<double>" if precision == 0 else "k_prep<float>",
+    names = {"prep": "k_prep<PREP_F64>" if precision == 0 else "k_prep<PREP_F32>",
              "iface_d1": "k_iface_avg", "iface_d2": "k_iface_avg",
-             "rhs": "k_rhs<double>" if precision == 0 else "k_rhs<float>"}
+             "rhs": "k_rhs64" if precision == 0 else "k_rhs"}
+    P = cfg.n_elem * cfg.n_r * cfg.n_theta * cfg.n_phi
+    small = P * sum(ns) <= SMALL_WORK and P * max(ns) ** 2 <= SMALL_SQUARE and max(ns) <= 64
+    if getattr(cfg, "theta_basis", 0) == 1 and cfg.n_phi % 4:
+        small = False
     for d, dn in enumerate(("r", "theta", "phi")):
         fx = 2 <= ns[d] <= 128 and (d != 2 or ns[d] % 2 == 0)
         fourier = d == 2 or (d == 1 and getattr(cfg, "theta_basis", 0) == 1)
         # derivatives and the filter: the digit-slice kernel (Chebyshev derivatives above 64
         # nodes: the FP64 units)
         fp64_f = f"k_contract_fx<{d}>" if fx else f"k_deriv_eo<{d}>"
-        fp64_d = f"k_contract_fx<{d}>" if fx else f"k_deriv_eo<{d}>"
-        if fx and not fourier and ns[d] > 64:
-            fp64_d = f"k_deriv<{d}>"
+        fp64_d = f"k_contract_fx<{d}>" if fx and (fourier or ns[d] <= 64) else f"k_deriv_eo<{d}>"
         if d == 1 and getattr(cfg, "theta_basis", 0) == 1:
             # Fourier theta: fold, two half-width contractions, unfold (timed together)
             fx_t = fx and cfg.n_phi % 4 == 0
@@ -430,6 +435,8 @@ def _kernel_names(cfg, precision):
             tc = "theta fold + k_contract_tc<1> x2 + unfold"
         else:
             tc = f"k_contract_tc<{d}>"
+        if small:
+            fp64_f = fp64_d = f"k_contract_small<{d}>"
         for c in ("d1", "d2"):
             names[f"{c}_{dn}"] = fp64_d if precision == 0 else tc
         names[f"filter_{dn}"] = fp64_f
@@ -471,7 +478,7 @@ def roofline(kt_full, P, precision, names):
                          "peak_source": "MEASURED_PEAKS.json hbm_gbs (of measured)",
                          "work": "input read + output written per contracted field"})
     else:
-        by = RHS32_BYTES_PER_NODE if top == "k_rhs<float>" else None
+        by = RHS32_BYTES_PER_NODE if top == "k_rhs" else None
         if by is None:
             roof.update({"bound": None, "achieved": None, "peak": None, "unit": None, "frac": None,
                          "traffic": None})
@@ -492,10 +499,8 @@ def roofline(kt_full, P, precision, names):
 # three stages of a step); absent = not captured since the kernel last changed.  These
 # pointwise kernels move a fixed number of bytes per node, so another workload's launch
 # is scaled by its node count (traffic_note says so).
-# k_rhs<double> moves ~2.8 KB per node, about twice its algorithmic bytes: register spills
-# (it is FP64-bound, the bytes are not).
 TRAFFIC_NODES = 393216
-TRAFFIC = {"k_rhs<double>": 1.10e9, "k_prep<double>": 1.66e8, "k_prep<float>": 1.66e8, "k_rhs<float>": 6.13e8}
+TRAFFIC = {"k_rhs64": 7.75e8, "k_prep<PREP_F64>": 1.92e8, "k_prep<PREP_F32>": 1.17e8, "k_rhs": 5.11e8}
 
 
 def _traffic(kernel, P):
