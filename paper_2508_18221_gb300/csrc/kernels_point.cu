@@ -386,7 +386,9 @@ __device__ __forceinline__ void fluxes64(long long p, long long P, double alpha,
 // or FP32.  Bound by the FP64 pipe (87 % busy): 346 FP64 instructions per node against 707
 // in FP64, so the launch inside the stepping of 393,216 nodes went from 545 to 283 us (ncu),
 // the FP32 form from 340 to 234 us, the recovery of a newly loaded state (grmhd_con2prim,
-// whole call) from 807 to 247 us.  Three blocks per SM (168 registers).
+// whole call) from 807 to 247 us.  Three blocks per SM (168
+// registers): per step of three launches 843 us in FP64 and 575 us in FP32, against 865 and 580
+// with four (128 registers, spills of 120 B) and 972 and 634 with five.
 enum { PREP_PRIM = 0, PREP_F64 = 1, PREP_F32 = 2 };
 
 template <int WHAT>
@@ -613,8 +615,8 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
 // The mixed modes' right-hand side (FP32 algebra; FP64 runs k_rhs64 below).  Bound by memory
 // and latency, not by arithmetic, so it keeps the four-dimensional form of the matter terms.
 // Each variable is written as soon as it is known, as in k_rhs64 (MODE likewise), and two
-// blocks per SM have the registers to do it without spills: 393,216 nodes 144 -> 101 us (about
-// 5.6 TB/s of its ~1.4 KB per node); three blocks of 168 registers with 500 B of spills a
+// blocks per SM have the registers to do it without spills: 393,216 nodes 144 -> 101 us (98 now,
+// about 5.7 TB/s of its ~1.4 KB per node); three blocks of 168 registers with 500 B of spills a
 // thread take 142 us, four 156 us.
 template <int MODE, bool HAM>
 __global__ void __launch_bounds__(128, 2) k_rhs(Dims d, PhysParams pp, const double* __restrict__ U0,

@@ -22,9 +22,9 @@
 // tile's first loads are issued before the epilogue of the current one.  Several CTAs share
 // an SM up to 64 nodes; at 65 .. 128 their operands fill it, so one CTA of 16 warps
 // works alone.  Per launch on 4,194,304 nodes (32 x 64 x 128 per element), before and after:
-// first derivatives r 473 -> 292, theta 996 -> 381, phi 1,099 -> 585 us; second derivatives
-// 458 -> 229, 506 -> 190, 328 -> 196 us (bit-identical results).
-#include <cuda_bf16.h>
+// first derivatives r 473 -> 268, theta 996 -> 356, phi 1,099 -> 572 us; second derivatives
+// 458 -> 219, 506 -> 178, 328 -> 195 us (bit-identical results); of that, slices converted in
+// pairs and the shorter FP64 -> FP32 conversion gave 292 -> 268, 381 -> 356, 585 -> 572.
 #include <stdint.h>
 
 #include "fp_convert.cuh"
@@ -77,8 +77,10 @@ __device__ __forceinline__ void mma_issue(uint32_t tmem, uint64_t da, uint64_t d
                      "l"(da), "l"(db), "r"(id), "r"(acc));
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 a, __nv_bfloat16 b) {
-    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
 }
 
 // eight consecutive values of a line (k >= N and missing lines are zero): 16-byte loads where
@@ -209,17 +211,14 @@ __global__ void __launch_bounds__(128 * W, tc_ctas<TIn>(W))
                 uint32_t w[3][4];
 #pragma unroll
                 for (int u = 0; u < 4; u++) {
-                    __nv_bfloat16 h[3][2];
+                    // two values at a time: one conversion instruction per slice packs both
+                    float f0 = x[2 * u], f1 = x[2 * u + 1];
 #pragma unroll
-                    for (int q = 0; q < 2; q++) {
-                        const float f = x[2 * u + q];
-                        h[0][q] = __float2bfloat16_rn(f);
-                        const float r1 = f - __bfloat162float(h[0][q]);
-                        h[1][q] = __float2bfloat16_rn(r1);
-                        h[2][q] = __float2bfloat16_rn(r1 - __bfloat162float(h[1][q]));
+                    for (int l = 0; l < 3; l++) {
+                        w[l][u] = pack_bf16(f0, f1);
+                        f0 -= __uint_as_float(w[l][u] << 16);
+                        f1 -= __uint_as_float(w[l][u] & 0xFFFF0000u);
                     }
-#pragma unroll
-                    for (int l = 0; l < 3; l++) w[l][u] = pack_bf16(h[l][0], h[l][1]);
                 }
 #pragma unroll
                 for (int l = 0; l < 3; l++)
