@@ -113,7 +113,8 @@ typedef struct {
  * run: 0 (default) on the FP16 tensor cores with exact base-256 digit slices of the
  * FP64 values (Ozaki splitting; up to 128 nodes per direction; each digit-order sum in an
  * exact accumulator of its own, error about 1e-15 of sum_j |D_ij| max_j |u_j|; above 64
- * Chebyshev nodes the FP64 units take the derivatives), 1 on the FP64 units.  coupling: 0 (default) one
+ * Chebyshev nodes the FP64 units take the derivatives; on small grids the same digits are
+ * multiplied on the integer units, same bits), 1 on the FP64 units.  coupling: 0 (default) one
  * unsplit right-hand side over all 32 variables per Runge-Kutta stage; 1 the paper's
  * coupled loop ("Coupled Main Loop"): per step the fluid is advanced by the selected
  * Runge-Kutta scheme on the frozen metric, then BSSN + gauge take one forward-Euler step
