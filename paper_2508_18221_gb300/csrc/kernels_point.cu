@@ -64,27 +64,27 @@ struct C2PScal {
     T v2max;        // r^2 / (1 + r^2), the largest admissible v^2
 };
 
-// g and its slope in FP32, with the derivatives the final correction needs
+// g and its slope in FP32 alone: the search.  The cap on v^2 keeps W finite (at most 4,096: from
+// there on FP32 has no digits of 1 - v^2 left, and eps / W, all that W enters by, has no weight)
 struct Master32 {
-    float g, dg, dx, dv2, dqm;
+    float g, dg;
 };
 __device__ __forceinline__ Master32 master32(float mu, const C2PScal<float>& c) {
     Master32 r;
     const float x = __fdividef(1.f, fmaf(mu, c.bb, 1.f)), mx = mu * x, x2 = x * x;    // d(mu x) = x^2
-    r.dx = -c.bb * x2;
+    const float dx = -c.bb * x2;
     const float rb = c.r2 * x2 + mx * (1.f + x) * c.rb2;
-    const float drb = 2.f * c.r2 * x * r.dx + c.rb2 * (x2 * (1.f + x) + mx * r.dx);
+    const float drb = 2.f * c.r2 * x * dx + c.rb2 * (x2 * (1.f + x) + mx * dx);
     const float m1 = mu * rb, dm1 = fmaf(mu, drb, rb);
     const float qb = c.c0 - c.c1 * mx * mx, dqb = -2.f * c.c1 * mx * x2;
-    r.dqm = dqb - dm1;
-    float v2 = mu * m1;
-    r.dv2 = fmaf(mu, dm1, m1);
-    if (!(v2 <= c.v2max)) { v2 = c.v2max; r.dv2 = 0.f; }
-    const float om = 1.f - v2, W = rsqrtf(om), iW = om * W, diW = -0.5f * r.dv2 * W;
+    float v2 = mu * m1, dv2 = fmaf(mu, dm1, m1);
+    const float cap = fminf(c.v2max, 1.f - 0x1p-24f);
+    if (!(v2 <= cap)) { v2 = cap; dv2 = 0.f; }
+    const float om = 1.f - v2, W = rsqrtf(om), iW = om * W, diW = -0.5f * dv2 * W;
     const float e = fmaf(W, 1.f + (qb - m1), -1.f);
     float z, dz;
     if (e >= c.eps_min) {
-        const float de = 0.5f * r.dv2 * W * W * W * (1.f + (qb - m1)) + W * r.dqm;
+        const float de = 0.5f * dv2 * W * W * W * (1.f + (qb - m1)) + W * (dqb - dm1);
         z = fmaf(c.g1 * e, iW, 1.f + qb);
         dz = dqb + c.g1 * (de * iW + e * diW);
     } else {
@@ -99,7 +99,8 @@ __device__ __forceinline__ Master32 master32(float mu, const C2PScal<float>& c) 
 
 // g in FP64 and the quantities that the primitives are made of
 struct Master64 {
-    double g, x, v2, m1, q2;     // q2 = (mu x)^2
+    double g, x, v2, m1, q2;     // v2 before the clamp to v2max; q2 = (mu x)^2
+    double W, e;                 // of the clamped v2; eps before its floor
 };
 __device__ __forceinline__ Master64 master64(double mu, const C2PScal<double>& c) {
     Master64 r;
@@ -108,23 +109,59 @@ __device__ __forceinline__ Master64 master64(double mu, const C2PScal<double>& c
     r.q2 = mx * mx;
     r.m1 = mu * fma(r.x, c.r2 * r.x, fma(u, r.x, u));
     const double zb = fma(-c.c1, r.q2, 1.0 + c.c0);
-    const double v2 = mu * r.m1;
-    r.v2 = v2 <= c.v2max ? v2 : c.v2max;
-    const double om = 1.0 - r.v2, W = rsqrt64(om), iW = om * W;
-    const double e = fma(W, zb - r.m1, -1.0);
-    const double z = e >= c.eps_min ? fma(c.g1 * e, iW, zb) : fma(fma(1.0 + c.g1, c.eps_min, 1.0), iW, r.m1);
+    r.v2 = mu * r.m1;
+    const double om = 1.0 - (r.v2 <= c.v2max ? r.v2 : c.v2max);
+    r.W = rsqrt64(om);
+    const double iW = om * r.W;
+    r.e = fma(r.W, zb - r.m1, -1.0);
+    const double z = r.e >= c.eps_min ? fma(c.g1 * r.e, iW, zb) : fma(fma(1.0 + c.g1, c.eps_min, 1.0), iW, r.m1);
     r.g = fma(mu, z, -1.0);
+    return r;
+}
+
+// The slope of g where FP64 has evaluated it, and the derivatives that the final correction
+// needs, in FP32.  What FP32 cannot resolve comes from the evaluation: on which side of v2max
+// and of eps_min the point lies (cold gas has v^2 within about eps / W^2 of v2max), W (its
+// relative error is W^2 times that of v^2) and eps (1 + qbar - mu rbar^2 is (1 + eps) / W).
+struct Slope32 {
+    float dg, dx, dv2, dqm, de;  // dv2, de: before the clamp and the floor
+};
+__device__ __forceinline__ Slope32 slope32(float mu, const Master64& f, const C2PScal<double>& c64,
+                                           const C2PScal<float>& c) {
+    Slope32 r;
+    const float x = __fdividef(1.f, fmaf(mu, c.bb, 1.f)), mx = mu * x, x2 = x * x;
+    r.dx = -c.bb * x2;
+    const float rb = c.r2 * x2 + mx * (1.f + x) * c.rb2;
+    const float drb = 2.f * c.r2 * x * r.dx + c.rb2 * (x2 * (1.f + x) + mx * r.dx);
+    const float m1 = mu * rb, dm1 = fmaf(mu, drb, rb);
+    const float qb = c.c0 - c.c1 * mx * mx, dqb = -2.f * c.c1 * mx * x2;
+    r.dqm = dqb - dm1;
+    r.dv2 = fmaf(mu, dm1, m1);
+    const float hdv = f.v2 <= c64.v2max ? 0.5f * r.dv2 : 0.f;
+    const float W = d2f_rn(f.W), iW = __fdividef(1.f, W), diW = -hdv * W;
+    const float e = d2f_rn(f.e);
+    r.de = hdv * (W * W) * (1.f + e) + W * r.dqm;
+    float z, dz;
+    if (f.e >= c64.eps_min) {
+        z = fmaf(c.g1 * e, iW, 1.f + qb);
+        dz = dqb + c.g1 * (r.de * iW + e * diW);
+    } else {
+        const float h = 1.f + (1.f + c.g1) * c.eps_min;
+        z = fmaf(h, iW, m1);
+        dz = fmaf(h, diW, dm1);
+    }
+    r.dg = fmaf(mu, dz, z);
     return r;
 }
 
 // Primitive recovery at one point: the root of g in the bracket [0, 1] (h >= 1).  FP32 finds
 // it to FP32's accuracy from the guess (its pipe is idle: 64 FP32 instructions issue in the
 // time of one FP64 instruction); then Newton steps with the residual in FP64 and the slope in
-// FP32, so that each step leaves about 1e-6 of the last one's error: two FP64 evaluations
-// of 27 instructions in place of three or four of ~110 with the derivative carried in
-// FP64.  Safeguarded by bisection throughout.  Returns 1 on success without floor, 0 if
-// eps was floored or the iteration did not converge; *mu_o, *x_o, *W_o, *iW_o, *eps_o
-// (floored) at the root.
+// FP32 to about 1e-6, so that a step leaves that much of the last one's error unless a kink of g
+// lies between: two FP64 evaluations of 27 instructions in place of three or four of ~110
+// with the derivative carried in FP64.  Safeguarded by bisection throughout.  Returns 1 on
+// success without floor, 0 if eps was floored or the iteration did not converge; *mu_o, *x_o,
+// *W_o, *iW_o, *eps_o (floored) at the root.
 __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit, double tol, float guess,
                                              double* mu_o, double* x_o, double* W_o, double* iW_o, double* eps_o) {
     const C2PScal<float> cf = {d2f_rn(c.r2), d2f_rn(c.bb), d2f_rn(c.rb2),     d2f_rn(c.c0),
@@ -150,16 +187,17 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
     float dprev = 0.f;
     int conv = 0;
     Master64 f;
-    Master32 s;
+    Slope32 s;
     const float tolf = (float)tol;
     // f(0+) < 0 and f(1) >= 0 for every admissible state (h >= 1); a state without a root
     // never converges and is flagged below.  Stop when the Newton step is below tol, or when
     // two consecutive steps d_{k-1} > d_k predict the next one, d_k (d_k / d_{k-1}) for linear
-    // convergence, below tol / 100, or when a step of rounding size leaves the bracket.  The
+    // convergence, below tol / 100 and the step crosses no kink of g (the slope changes there:
+    // for cold gas by a factor of two), or when a step of rounding size leaves the bracket.  The
     // limit counts the FP64 evaluations after the first two.
     for (int it = 0;; it++) {
         f = master64(mu, c);
-        s = master32(d2f_rn(mu), cf);
+        s = slope32(d2f_rn(mu), f, c, cf);
         delta = 0.0;
         if (f.g == 0.0) { conv = 1; break; }
         if (it >= maxit + 1) break;
@@ -173,7 +211,8 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
         delta = mn - mu;
         const float dk = fabsf(d2f_rn(delta)), mf = d2f_rn(mn);
         if (dk <= tolf * mf) { conv = 1; break; }
-        if (newton && dprev > dk && dk <= 1e-3f * mf && __fdividef(dk, dprev) * dk <= 0.01f * tolf * mf) {
+        if (newton && dprev > dk && dk <= 1e-3f * mf && __fdividef(dk, dprev) * dk <= 0.01f * tolf * mf &&
+            fabsf(s.dv2) * dk < fabsf(d2f_rn(f.v2 - c.v2max)) && fabsf(s.de) * dk < fabsf(d2f_rn(f.e - c.eps_min))) {
             conv = 1;
             break;
         }
@@ -191,7 +230,7 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
         // the last step is not evaluated any more: to first order, or, where tol let it be
         // large, after all
         mu += delta;
-        if (fabs(delta) > 1e-9 * mu) {
+        if (fabs(delta) > 1e-10 * mu) {
             f = master64(mu, c);
             qm = fma(-c.c1, f.q2, c.c0) - f.m1;
         } else {
@@ -200,9 +239,10 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
             qm = fma(f2d(s.dqm), delta, qm);
         }
     }
-    const double om = 1.0 - f.v2, W = rsqrt64(om);
+    const double v2 = f.v2 <= c.v2max ? f.v2 : c.v2max;
+    const double om = 1.0 - v2, W = rsqrt64(om);
     // eps without the cancellation of W (1 + qm) - 1: W - 1 = W^2 v^2 / (1 + W)
-    const double e = fma(W, qm, f.v2 * W * W * rcp64(1.0 + W));
+    const double e = fma(W, qm, v2 * W * W * rcp64(1.0 + W));
     *mu_o = mu;
     *x_o = f.x;
     *W_o = W;
@@ -449,7 +489,7 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
             c.c1 = 0.5 * (c.bb * c.r2 - c.rb2);
             c.g1 = pp.gam - 1.0;
             c.eps_min = pp.eps_atm;
-            c.v2max = c.r2 * rcp64(1.0 + c.r2);
+            c.v2max = fmin(c.r2 * rcp64(1.0 + c.r2), 1.0 - 0x1p-53);   // W stays finite without a root too
             // guess mu = 1/(h W) from the stored primitives
             const float guess = __fdividef(1.f, (1.f + (float)pp.gam * d2f_rn(prim[4 * P + p])) * d2f_rn(prim[6 * P + p]));
             double mu, x;
