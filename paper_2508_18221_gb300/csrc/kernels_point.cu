@@ -194,13 +194,13 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
     // two consecutive steps d_{k-1} > d_k predict the next one, d_k (d_k / d_{k-1}) for linear
     // convergence, below tol / 100 and the step crosses no kink of g (the slope changes there:
     // for cold gas by a factor of two), or when a step of rounding size leaves the bracket.  The
-    // limit counts the FP64 evaluations after the first two.
+    // limit counts the FP64 evaluations that a step follows.
     for (int it = 0;; it++) {
         f = master64(mu, c);
         s = slope32(d2f_rn(mu), f, c, cf);
         delta = 0.0;
+        if (it >= maxit) break;
         if (f.g == 0.0) { conv = 1; break; }
-        if (it >= maxit + 1) break;
         if (f.g < 0.0) lo = mu; else hi = mu;
         double mn = fma(-f.g, f2d(__fdividef(1.f, s.dg)), mu);
         const bool newton = mn > lo && mn < hi;

@@ -67,3 +67,16 @@ def test_recovery_returns_the_primitives(w, eps, sigma):
         assert float((np.abs(got[4] - e) / (h * W ** 2)).max()) <= unit, start
         assert float(np.abs(got[1:4] - v).max()) <= unit, start
     ctx.close()
+
+
+def test_iteration_limit():
+    """c2p_maxit = 1: one FP64 step does not bring the search's FP32 root to c2p_tol, so every
+    node counts as failed; the default solves all of them."""
+    cfg, U, *_ = _state(5.0, 1e-3, 0.0, 4.0 / 3.0)
+    state = torch.from_numpy(U.reshape(-1).copy()).cuda()
+    for maxit in (1, None):
+        ctx = pkg.Context(*pkg.make_structs(cfg, **({} if maxit is None else {"c2p_maxit": maxit})))
+        ctx.set_state(state, True)
+        out = torch.empty(pkg.NPRIM * ctx.n_points, dtype=torch.float64, device="cuda")
+        assert ctx.con2prim(out, True) == (0 if maxit is None else ctx.n_points)
+        ctx.close()
