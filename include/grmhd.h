@@ -104,7 +104,8 @@ typedef struct {
  * runs the paper's damped iteration instead ("The Primitive Variable Recovery"): from the
  * stored primitives (or, after grmhd_set_state, the dust estimates v^i = gamma^ij
  * S_j / (tau + D), eps = (tau + D)/(D W) - 1), the update v^i += lam gamma^ij dS_j /
- * (rho h W^2), eps += lam dtau / (rho W^2), rho = D / W with lam = c2p_lambda at first and halved while the residual grows, until ||dS|| + |dtau| <
+ * (rho h W^2), eps += lam dtau / (rho W^2), rho = D / W with lam = c2p_lambda at first and
+ * halved while the residual grows, until ||dS|| + |dtau| <
  * c2p_tol D or c2p_maxit updates (the paper: 30-40), then one Newton update of eps.  It
  * converges linearly: after 40 iterations from a cold start eps is within about 1e-9 of
  * the exact root on the 2-element workload (2e-11 in the torus), so the default stays

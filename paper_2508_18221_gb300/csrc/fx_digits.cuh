@@ -12,9 +12,11 @@ constexpr unsigned long long DIG_BIAS = 0x80808080808080ull;  // 128 in each dig
 // signed fixed-point integer relative to the line exponent EL (|X| <= 2^54; the value is
 // X 2^(EL - 1076)); byte b of Z minus 128 is the balanced digit of weight 256^b.  Branch-
 // free (the values of a thread overlap): with y = +-(4 m >> sh), sh = EL - e in 0 .. 63
-// (4 m < 2^56, so every sh >= 56 gives 0; zero for e = 0), X + bias is (y + 1 + 2 bias) >> 1:
-// sign, rounding (half up) and bias in one 64-bit addition.  The integer pipes bound the
-// conversion, so the shift by two is left to the multiply-add pipe (four).
+// (4 m < 2^56, so every sh >= 56 gives 0; zero for e = 0), X + bias is (y + 1 + 2 bias) >> 1
+// for y >= 0 and (y + 2 bias) >> 1 = (~|y| + 1 + 2 bias) >> 1 below: sign, rounding (to the
+// nearest, halves away from zero) and bias in one 64-bit addition to the magnitude or its
+// complement.  The integer pipes bound the conversion, so the shift by two is left to the
+// multiply-add pipe (four).
 __device__ __forceinline__ unsigned long long digit_word(double u, int EL, uint32_t four) {
     const uint32_t hi = (uint32_t)__double2hiint(u), lo = (uint32_t)__double2loint(u);
     const int e = (int)((hi >> 20) & 0x7FFu);
@@ -24,7 +26,7 @@ __device__ __forceinline__ unsigned long long digit_word(double u, int EL, uint3
     const unsigned long long y = m4 >> sh;
     const uint32_t s = (uint32_t)((int)hi >> 31);
     const unsigned long long ys = y ^ (((unsigned long long)s << 32) | s);
-    return (ys + (2 * DIG_BIAS + 1) + (s & 1u)) >> 1;
+    return (ys + (2 * DIG_BIAS + 1)) >> 1;
 }
 
 // R * 2^X: one correctly rounded integer-to-double conversion, then the power of two is
