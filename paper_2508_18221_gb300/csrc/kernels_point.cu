@@ -120,9 +120,11 @@ __device__ __forceinline__ Master64 master64(double mu, const C2PScal<double>& c
 }
 
 // The slope of g where FP64 has evaluated it, and the derivatives that the final correction
-// needs, in FP32.  What FP32 cannot resolve comes from the evaluation: on which side of v2max
-// and of eps_min the point lies (cold gas has v^2 within about eps / W^2 of v2max), W (its
-// relative error is W^2 times that of v^2) and eps (1 + qbar - mu rbar^2 is (1 + eps) / W).
+// needs, in FP32.  With d(1/W) = -W dv^2 / 2 and eps = W (1 + qbar - mu rbar^2) - 1,
+// d(eps / W) = W dv^2 / 2 + d(qbar - mu rbar^2): what FP32 cannot resolve is W (its relative error
+// is W^2 times that of v^2) and on which side of v2max and of eps_min the point lies (cold gas
+// has v^2 within about eps / W^2 of v2max).  Both come from the evaluation; the rest does not
+// wait for it (eps and W of FP32 enter g + 1 = mu z by eps / W alone).
 struct Slope32 {
     float dg, dx, dv2, dqm, de;  // dv2, de: before the clamp and the floor
 };
@@ -137,19 +139,15 @@ __device__ __forceinline__ Slope32 slope32(float mu, const Master64& f, const C2
     const float qb = c.c0 - c.c1 * mx * mx, dqb = -2.f * c.c1 * mx * x2;
     r.dqm = dqb - dm1;
     r.dv2 = fmaf(mu, dm1, m1);
-    const float hdv = f.v2 <= c64.v2max ? 0.5f * r.dv2 : 0.f;
-    const float W = d2f_rn(f.W), iW = __fdividef(1.f, W), diW = -hdv * W;
-    const float e = d2f_rn(f.e);
-    r.de = hdv * (W * W) * (1.f + e) + W * r.dqm;
-    float z, dz;
-    if (f.e >= c64.eps_min) {
-        z = fmaf(c.g1 * e, iW, 1.f + qb);
-        dz = dqb + c.g1 * (r.de * iW + e * diW);
-    } else {
-        const float h = 1.f + (1.f + c.g1) * c.eps_min;
-        z = fmaf(h, iW, m1);
-        dz = fmaf(h, diW, dm1);
-    }
+    const float om = 1.f - fminf(mu * m1, fminf(c.v2max, 1.f - 0x1p-24f)), W1 = rsqrtf(om), iW1 = om * W1;
+    const float e1 = W1 * (1.f + (qb - m1)), h = 1.f + (1.f + c.g1) * c.eps_min;        // 1 + eps
+    // W of the evaluation (1 <= W < 2^27), cut to FP32
+    const float W = __uint_as_float(__funnelshift_l((uint32_t)__double2loint(f.W), (uint32_t)__double2hiint(f.W) - 0x38000000u, 3));
+    const float hdvW = f.v2 <= c64.v2max ? 0.5f * r.dv2 * W : 0.f;
+    r.de = W * fmaf(hdvW, e1, r.dqm);
+    const bool gas = f.e >= c64.eps_min;
+    const float z = gas ? fmaf(c.g1 * (e1 - 1.f), iW1, 1.f + qb) : fmaf(h, iW1, m1);
+    const float dz = gas ? fmaf(c.g1, hdvW + r.dqm, dqb) : fmaf(-h, hdvW, dm1);
     r.dg = fmaf(mu, dz, z);
     return r;
 }
@@ -212,7 +210,7 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
         const float dk = fabsf(d2f_rn(delta)), mf = d2f_rn(mn);
         if (dk <= tolf * mf) { conv = 1; break; }
         if (newton && dprev > dk && dk <= 1e-3f * mf && __fdividef(dk, dprev) * dk <= 0.01f * tolf * mf &&
-            fabsf(s.dv2) * dk < fabsf(d2f_rn(f.v2 - c.v2max)) && fabsf(s.de) * dk < fabsf(d2f_rn(f.e - c.eps_min))) {
+            fabsf(s.dv2) * dk <= fabsf(d2f_rn(f.v2 - c.v2max)) && fabsf(s.de) * dk <= fabsf(d2f_rn(f.e - c.eps_min))) {
             conv = 1;
             break;
         }
