@@ -61,15 +61,15 @@ struct grmhd_ctx {
     double* acc;             // RK4 accumulator (allocated for integrator = 1)
     double* prim;
     double* flux;
-    double* tmn;
+    double* tmn;             // matter terms, from k_prep to k_rhs of a stage: in scratch, idle meanwhile
     double* lam;
     double* d1;
     double* d2;
     double* divF;
-    double* scratch;         // nv * P
+    double* scratch;         // nv * P: between the links of a filter; diagnostics; tmn
     double* divB;            // d_i (sqrt(gamma) B^i) (GLM only)
     double* ham;             // Hamiltonian constraint per node (diagnostics)
-    double* met;             // N_MET * P: the metric of the last k_prep
+    double* met;             // N_MET * P (mixed modes one less): the metric of the last k_prep
     double* ham_out;         // non-null while a diagnostic stage is enqueued: k_rhs writes H there
     int nv;                  // evolved variables: GRMHD_NV, + 1 (psi) with GLM
     double* Ds[3];           // reflection-split derivative operators r / theta / phi
@@ -259,7 +259,7 @@ static int validate(const grmhd_grid* g, const grmhd_physics* ph, const grmhd_op
 static void free_ctx(grmhd_ctx* c) {
     if (!c) return;
     if (c->gexec) cudaGraphExecDestroy(c->gexec);
-    double** bufs[] = {&c->U[0], &c->U[1], &c->U[2], &c->acc, &c->prim, &c->flux, &c->tmn, &c->lam,
+    double** bufs[] = {&c->U[0], &c->U[1], &c->U[2], &c->acc, &c->prim, &c->flux, &c->lam,
                        &c->d1, &c->d2, &c->divF, &c->scratch, &c->r_scale, &c->wq, &c->hmin, &c->dt, &c->diag, &c->divB, &c->ham, &c->met};
     for (double** b : bufs)
         if (*b) cudaFree(*b);
@@ -496,15 +496,15 @@ static int ctx_create(int ninst, const grmhd_grid* grids, const grmhd_physics* p
     if (opts->integrator == 1) AL(c->acc, nv * P);
     AL(c->prim, N_PRIM * P);
     AL(c->flux, N_FLUX * P);
-    AL(c->tmn, N_TMN * P);
     AL(c->lam, P);
     AL(c->d1, (N_D1 + glm) * 3 * P);
     if (glm) AL(c->divB, P);
     AL(c->d2, N_D2 * 6 * P);
     AL(c->divF, ndiv * 8 * P);
     AL(c->ham, P);
-    AL(c->met, N_MET * P);
+    AL(c->met, (opts->precision > 0 ? N_MET - 1 : N_MET) * P);
     AL(c->scratch, nv * P);
+    c->tmn = c->scratch;
     AL(c->r_scale, E); AL(c->wq, P); AL(c->hmin, ninst); AL(c->dt, ninst); AL(c->diag, 8);
     AL(c->nfail, 1); AL(c->lam_bits, ninst); AL(c->nan_flag, 1); AL(c->tc_err, 1);
     AL(c->iface_dev, E); AL(c->elem_inst_dev, E);
@@ -1434,11 +1434,11 @@ extern "C" int grmhd_rhs(grmhd_ctx* c, double* out, int on_device) {
     c->launches_tmp = 0;
     CK(cudaMemsetAsync(c->nfail, 0, sizeof(unsigned long long), c->stream));
     RKCoef co = {0, 0, 0, 0, -1};
-    double* dst = on_device ? out : c->scratch;
+    double* dst = on_device ? out : c->U[1];
     int st = enqueue_stage(c, 0, co, dst, c->pp);
     if (st) return st;
     c->launches_per_call = c->launches_tmp;
-    if (!on_device) return copy_out(c, out, c->scratch, (size_t)c->nv * c->d.P, 0);
+    if (!on_device) return copy_out(c, out, c->U[1], (size_t)c->nv * c->d.P, 0);
     return GRMHD_OK;
 }
 
@@ -1529,7 +1529,7 @@ extern "C" int grmhd_diag(grmhd_ctx* c, double out[GRMHD_NDIAG]) {
     NvtxRange nvtx_range("grmhd_diag");
     if (!c || !out) return GRMHD_EINVAL;
     // Hamiltonian constraint: one right-hand-side evaluation of the current state with the
-    // metric part always on (its result, written to scratch, is discarded); k_rhs writes H
+    // metric part always on (its result, written to U[1], is discarded); k_rhs writes H
     // per node from the Ricci tensor it forms anyway
     {
         PhysParams ph = c->pp;
@@ -1538,7 +1538,7 @@ extern "C" int grmhd_diag(grmhd_ctx* c, double out[GRMHD_NDIAG]) {
         const RKCoef co = {0, 0, 0, 0, -1};
         c->ham_out = c->ham;
         const long long keep = c->launches_tmp;
-        const int st = enqueue_stage(c, 0, co, c->scratch, ph);
+        const int st = enqueue_stage(c, 0, co, c->U[1], ph);
         c->ham_out = nullptr;
         c->launches_tmp = keep;
         if (st) return st;
@@ -1617,14 +1617,14 @@ extern "C" int grmhd_kernel_times(grmhd_ctx* c, int reps, double* ms_out, double
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
-    // keep the state: U[1] <- U[0], work on U[1], U[2] holds the saved copy
+    // keep the state: U[1] <- U[0], work on U[1], results to U[0], U[2] holds the saved copy
     CK(cudaMemcpyAsync(c->U[2], c->U[0], sizeof(double) * c->nv * P, cudaMemcpyDeviceToDevice, c->stream));
     CK(cudaMemcpyAsync(c->U[1], c->U[0], sizeof(double) * c->nv * P, cudaMemcpyDeviceToDevice, c->stream));
     RKCoef co = {0, 0, 0, 0, -1};
     int st = GRMHD_OK;
     for (int k = 0; k < GRMHD_NKT && st == GRMHD_OK; k++) {
         // bring the buffers the kernel reads up to date (untimed)
-        if (k >= 1) { c->launches_tmp = 0; st = enqueue_stage(c, 1, co, c->scratch, c->pp); if (st) break; }
+        if (k >= 1) { c->launches_tmp = 0; st = enqueue_stage(c, 1, co, c->U[0], c->pp); if (st) break; }
         CK(cudaEventRecord(e0, c->stream));
         for (int r = 0; r < reps; r++) {
             cudaError_t e = cudaSuccess;
@@ -1682,7 +1682,7 @@ extern "C" int grmhd_kernel_times(grmhd_ctx* c, int reps, double* ms_out, double
                           : launch_iface_avg(c->d, c->d2, P, 3 * N_D2, c->stream, 3, 6 * P);
             }
             else if (k == 9) e = launch_rhs(c->d, c->pp, c->U[0], c->U[1], c->prim, c->flux, c->tmn, c->lam, c->met, c->d1, c->d2,
-                                            c->divF, c->divB, c->opts.precision > 0, c->r_scale, c->dt, co, c->scratch,
+                                            c->divF, c->divB, c->opts.precision > 0, c->r_scale, c->dt, co, c->U[0],
                                             c->acc, c->stream, nullptr, c->small_d ? 3 : 1);
             else {
                 int dir = k - 10;
