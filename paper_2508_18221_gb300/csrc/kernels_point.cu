@@ -185,7 +185,7 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
         const float dk = fabsf(d2f_rn(delta)), mf = d2f_rn(mn);
         if (dk <= tolf * mf) { conv = 1; break; }
         if (newton && dprev > dk && dk <= 1e-3f * mf && __fdividef(dk, dprev) * dk <= 0.01f * tolf * mf &&
-            fabsf(s.dv2) * dk <= fabsf(d2f_rn(f.v2 - c.v2max)) && fabsf(s.de) * dk <= fabsf(d2f_rn(f.e - c.eps_min))) {
+            fabsf(s.dv2) * dk <= fabsf(d2f_rn(f.v2 - c.v2max)) && fabsf(s.de) * dk <= fabsf(d2f_rn(f.e) - cf.eps_min)) {
             conv = 1;
             break;
         }
@@ -213,7 +213,9 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
         }
     }
     const double v2 = f.v2 <= c.v2max ? f.v2 : c.v2max;
-    const double om = 1.0 - v2, W = rsqrt64(om);
+    double om = 1.0 - v2;
+    if (__double2hiint(om) == 0) om = 0x1p-53;    // no root at r above 1e8: W stays finite
+    const double W = rsqrt64(om);
     // eps without the cancellation of W (1 + qm) - 1: W - 1 = W^2 v^2 / (1 + W)
     const double e = fma(W, qm, v2 * W * W * rcp64(1.0 + W));
     *mu_o = mu;
@@ -462,7 +464,7 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
             c.c1 = 0.5 * (c.bb * c.r2 - c.rb2);
             c.g1 = pp.gam - 1.0;
             c.eps_min = pp.eps_atm;
-            c.v2max = fmin(c.r2 * rcp64(1.0 + c.r2), 1.0 - 0x1p-53);   // W stays finite without a root too
+            c.v2max = c.r2 * rcp64(1.0 + c.r2);
             // guess mu = 1/(h W) from the stored primitives
             const float guess = __fdividef(1.f, (1.f + (float)pp.gam * d2f_rn(prim[4 * P + p])) * d2f_rn(prim[6 * P + p]));
             double mu, x;
