@@ -661,9 +661,10 @@ __global__ void __launch_bounds__(fx_threads(WC, WE), WC == 4 ? 2 : 1) k_contrac
             const int* meta = reinterpret_cast<const int*>(fp.img + (DIR == 0 ? tl.e * fp.img_estride : 0) +
                                                            (size_t)op_bytes) + Np;
             const bool wide = __ldg(meta) != 0;
-            // R has 63 bits at most, so every result of the line is a normal number or zero
-            const bool safe = EL + __ldg(meta + 1) >= 1096 && EL + __ldg(meta + 2) <= 2996;
+            // R has 63 bits at most, so every result of the line is a normal number or zero (a line
+            // with an Inf or a NaN is not, however small the operator's entries)
             const bool line_bad = EL == 0x7FF;
+            const bool safe = !line_bad && EL + __ldg(meta + 1) >= 1096 && EL + __ldg(meta + 2) <= 2996;
             // column blocks holding output rows of this pass (the padding blocks beyond N are
             // computed by the MMAs but not read)
             const int ncol = min(Npp, N - pass * Npp);
