@@ -1138,7 +1138,7 @@ static int enqueue_stage(grmhd_ctx* c, int b, RKCoef co, double* out, const Phys
     st = enqueue_first_derivs(c, b, 1);
     if (st) return st;
     CK(cudaStreamWaitEvent(c->stream, c->ev_join, 0));
-    CK(launch_rhs(c->d, pp, c->U[0], c->U[b], c->prim, c->flux, c->tmn, c->lam, c->met, c->d1, c->d2,
+    CK(launch_rhs(c->d, pp, c->U[0], c->U[b], c->flux, c->tmn, c->lam, c->met, c->d1, c->d2,
                   c->divF, c->divB, c->opts.precision > 0, c->r_scale, c->dt, co, out, c->acc, c->stream,
                   c->ham_out, c->small_d ? 3 : 1));
     c->launches_tmp++;
@@ -1681,7 +1681,7 @@ extern "C" int grmhd_kernel_times(grmhd_ctx* c, int reps, double* ms_out, double
                 e = mixed ? launch_iface_avg_f(c->d, reinterpret_cast<float*>(c->d2), P, 3 * N_D2, c->stream, 3, 6 * P)
                           : launch_iface_avg(c->d, c->d2, P, 3 * N_D2, c->stream, 3, 6 * P);
             }
-            else if (k == 9) e = launch_rhs(c->d, c->pp, c->U[0], c->U[1], c->prim, c->flux, c->tmn, c->lam, c->met, c->d1, c->d2,
+            else if (k == 9) e = launch_rhs(c->d, c->pp, c->U[0], c->U[1], c->flux, c->tmn, c->lam, c->met, c->d1, c->d2,
                                             c->divF, c->divB, c->opts.precision > 0, c->r_scale, c->dt, co, c->U[0],
                                             c->acc, c->stream, nullptr, c->small_d ? 3 : 1);
             else {

@@ -40,13 +40,9 @@ __device__ __forceinline__ double f2d(float f) {
     return __hiloint2double((int)(ef == 0u ? s : (s | eh | (m >> 3))), (int)(ef == 0u ? 0u : (m << 29)));
 }
 
-// FP64 -> the algebra type R (identity for FP64)
+// FP64 -> the mixed modes' algebra type, and back
 template <class R> __device__ __forceinline__ R narrow(double x);
-template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
 template <> __device__ __forceinline__ float narrow<float>(double x) { return d2f_rn(x); }
-
-// the algebra type -> FP64 (identity for FP64)
-__device__ __forceinline__ double widen(double x) { return x; }
 __device__ __forceinline__ double widen(float x) { return f2d(x); }
 
 // Reciprocal and reciprocal square root: the hardware's 20-bit seeds (rcp / rsqrt.approx.f64)

@@ -102,10 +102,9 @@ struct RKCoef { double a, b, c, w; int acc_mode; };  // out = a U0 + b Us + c dt
 // also writes the Hamiltonian constraint per node (diagnostics); div_parts: 1, or 3 when divF
 // holds the three directions' terms one after the other (small grids, FP64)
 cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, const double* Us,
-                       const double* prim, const double* flux, const double* tmn,
-                       const double* lam, const double* met, const void* d1, const void* d2,
-                       const void* divF, const void* divB, int deriv_fp32, const double* r_scale_dev,
-                       const double* dt_dev, RKCoef co, double* out, double* acc, cudaStream_t s,
+                       const double* flux, const double* tmn, const double* lam, const double* met,
+                       const void* d1, const void* d2, const void* divF, const void* divB, int deriv_fp32,
+                       const double* r_scale_dev, const double* dt_dev, RKCoef co, double* out, double* acc, cudaStream_t s,
                        double* ham = nullptr, int div_parts = 1);
 // tensor-core contraction (kernels_tc.cu); op_img in the kernel's shared-memory layout
 cudaError_t launch_contract_tc(int dir, int in_fp32, const Dims& d, const TcJob* jobs, int njobs,

@@ -524,98 +524,98 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
         prim[6 * P + p] = W;
 
         if constexpr (WHAT != PREP_PRIM) {
-        met[0 * P + p] = e4;
-        met[1 * P + p] = e4m;
-        met[2 * P + p] = sqg;
-        for (int q = 0; q < 6; q++) met[(3 + q) * P + p] = gti[q];
-        const double alpha = U[V_ALPHA * P + p];
-        const double beta[3] = {U[V_BETA * P + p], U[(V_BETA + 1) * P + p], U[(V_BETA + 2) * P + p]};
-        // the light-cone speed is read at the element ends (interface penalty) only
-        const uint32_t ir = ((uint32_t)p / (uint32_t)d.NtNp) % (uint32_t)d.Nr;
-        if (ir == 0 || ir == (uint32_t)d.Nr - 1) lam[p] = fabs(beta[0]) + alpha * sqrt(e4m * gti[0]);
-        if constexpr (WHAT == PREP_F64) {
-            met[9 * P + p] = isq;
-            fluxes64(p, P, alpha, beta, gti, e4m, sqg, rho, v, v_d, eps, pr, W, iW, B_u, B_d, B2, Bs, flux, tmn);
-        } else {
-        using R = float;
-        double g[3][3], gi[3][3];
-        for (int i = 0; i < 3; i++)
-            for (int j = 0; j < 3; j++) {
-                g[i][j] = e4 * gt[SI(i, j)];
-                gi[i][j] = e4m * gti[SI(i, j)];
+            met[0 * P + p] = e4;
+            met[1 * P + p] = e4m;
+            met[2 * P + p] = sqg;
+            for (int q = 0; q < 6; q++) met[(3 + q) * P + p] = gti[q];
+            const double alpha = U[V_ALPHA * P + p];
+            const double beta[3] = {U[V_BETA * P + p], U[(V_BETA + 1) * P + p], U[(V_BETA + 2) * P + p]};
+            // the light-cone speed is read at the element ends (interface penalty) only
+            const uint32_t ir = ((uint32_t)p / (uint32_t)d.NtNp) % (uint32_t)d.Nr;
+            if (ir == 0 || ir == (uint32_t)d.Nr - 1) lam[p] = fabs(beta[0]) + alpha * sqrt(e4m * gti[0]);
+            if constexpr (WHAT == PREP_F64) {
+                met[9 * P + p] = isq;
+                fluxes64(p, P, alpha, beta, gti, e4m, sqg, rho, v, v_d, eps, pr, W, iW, B_u, B_d, B2, Bs, flux, tmn);
+            } else {
+                using R = float;
+                double g[3][3], gi[3][3];
+                for (int i = 0; i < 3; i++)
+                    for (int j = 0; j < 3; j++) {
+                        g[i][j] = e4 * gt[SI(i, j)];
+                        gi[i][j] = e4m * gti[SI(i, j)];
+                    }
+                // ---- four-vectors, fluxes and T^{mu nu} of the mixed modes in FP32 (their consumers,
+                // the tensor-core contractions and the FP32 right-hand side, keep about 24 bits); the
+                // primitive recovery above stays FP64
+                const R alphaR = narrow<R>(alpha), sqgR = narrow<R>(sqg), WR = narrow<R>(W);
+                R gR[3][3], betaR[3], vR[3], BR[3];
+                for (int i = 0; i < 3; i++) {
+                    betaR[i] = narrow<R>(beta[i]);
+                    vR[i] = narrow<R>(v[i]);
+                    BR[i] = narrow<R>(B_u[i]);
+                    for (int j = 0; j < 3; j++) gR[i][j] = narrow<R>(g[i][j]);
+                }
+                R vR_d[3];
+                for (int i = 0; i < 3; i++) vR_d[i] = gR[i][0] * vR[0] + gR[i][1] * vR[1] + gR[i][2] * vR[2];
+                R ia = R(1.0) / alphaR;
+                R u0 = WR * ia;
+                R uu[3];
+                for (int i = 0; i < 3; i++) uu[i] = WR * (vR[i] - betaR[i] * ia);
+                R b0 = WR * (vR_d[0] * BR[0] + vR_d[1] * BR[1] + vR_d[2] * BR[2]) * ia;
+                R iWR = R(1.0) / WR;
+                R bu[3];
+                for (int i = 0; i < 3; i++) bu[i] = (BR[i] + alphaR * b0 * uu[i]) * iWR;
+                R beta_d[3];
+                for (int i = 0; i < 3; i++)
+                    beta_d[i] = gR[i][0] * betaR[0] + gR[i][1] * betaR[1] + gR[i][2] * betaR[2];
+                R bb_ = beta_d[0] * betaR[0] + beta_d[1] * betaR[1] + beta_d[2] * betaR[2];
+                R g00 = -alphaR * alphaR + bb_;
+                R bd0 = g00 * b0 + beta_d[0] * bu[0] + beta_d[1] * bu[1] + beta_d[2] * bu[2];
+                R bd[3];
+                for (int i = 0; i < 3; i++)
+                    bd[i] = beta_d[i] * b0 + gR[i][0] * bu[0] + gR[i][1] * bu[1] + gR[i][2] * bu[2];
+                R b2 = b0 * bd0 + bu[0] * bd[0] + bu[1] * bd[1] + bu[2] * bd[2];
+                const R rhoR = narrow<R>(rho), epsR = narrow<R>(eps), prR = narrow<R>(pr);
+                R pstar = prR + R(0.5) * b2;
+                R rhohs = rhoR * (R(1.0) + epsR) + prR + b2;   // rho h*
+                // conserved variables from the primitives (undensitized)
+                R Dp = rhoR * WR;
+                R Sp[3];
+                for (int j = 0; j < 3; j++) Sp[j] = rhohs * WR * WR * vR_d[j] - alphaR * b0 * bd[j];
+                // tau = rho h* W^2 - p* - alpha^2 b0^2 - D without its cancellation: with
+                // W^2 - 1 = W^2 v^2 and W - 1 = W^2 v^2 / (W + 1),
+                // tau = rho W (eps W + W^2 v^2 / (W + 1)) + p W^2 v^2 + b^2 (W^2 - 1/2) - alpha^2 b0^2
+                // (tau ~ 1e-3 D for a cold gas: the direct form loses 3 digits, all of FP32's margin)
+                const R Wv2 = WR * WR * (vR_d[0] * vR[0] + vR_d[1] * vR[1] + vR_d[2] * vR[2]);
+                const R taup = rhoR * WR * (epsR * WR + Wv2 / (WR + R(1.0))) + prR * Wv2 + b2 * (WR * WR - R(0.5)) -
+                               alphaR * alphaR * b0 * b0;
+                // ---- densitized fluxes [dir][var]
+                R vt[3];
+                for (int i = 0; i < 3; i++) vt[i] = alphaR * vR[i] - betaR[i];
+                for (int i = 0; i < 3; i++) {
+                    // kept in FP32, as is T^{mu nu}: half the bytes, no conversion here and in the readers
+                    R* F = reinterpret_cast<R*>(flux) + (long long)(i * 8) * P + p;
+                    F[0 * P] = sqgR * (Dp * vt[i]);
+                    for (int j = 0; j < 3; j++)
+                        F[(1 + j) * P] = sqgR * (Sp[j] * vt[i] + (i == j ? alphaR * pstar : R(0.0)) -
+                                                 alphaR * bd[j] * BR[i] * iWR);
+                    F[4 * P] = sqgR * (taup * vt[i] + alphaR * pstar * vR[i] - alphaR * alphaR * b0 * BR[i] * iWR);
+                    for (int k = 0; k < 3; k++) F[(5 + k) * P] = sqgR * (vt[i] * BR[k] - vt[k] * BR[i]);
+                }
+                // ---- T^{mu nu}
+                R ia2 = ia * ia;
+                R gu[4][4];
+                gu[0][0] = -ia2;
+                for (int i = 0; i < 3; i++) gu[0][i + 1] = gu[i + 1][0] = betaR[i] * ia2;
+                for (int i = 0; i < 3; i++)
+                    for (int j = 0; j < 3; j++) gu[i + 1][j + 1] = narrow<R>(gi[i][j]) - betaR[i] * betaR[j] * ia2;
+                R u4[4] = {u0, uu[0], uu[1], uu[2]};
+                R b4[4] = {b0, bu[0], bu[1], bu[2]};
+                int n = 0;
+                for (int m = 0; m < 4; m++)
+                    for (int k = m; k < 4; k++, n++)
+                        reinterpret_cast<R*>(tmn)[n * P + p] = rhohs * u4[m] * u4[k] + pstar * gu[m][k] - b4[m] * b4[k];
             }
-        // ---- four-vectors, fluxes and T^{mu nu} of the mixed modes in FP32 (their consumers,
-        // the tensor-core contractions and the FP32 right-hand side, keep about 24 bits); the
-        // primitive recovery above stays FP64
-        const R alphaR = narrow<R>(alpha), sqgR = narrow<R>(sqg), WR = narrow<R>(W);
-        R gR[3][3], betaR[3], vR[3], BR[3];
-        for (int i = 0; i < 3; i++) {
-            betaR[i] = narrow<R>(beta[i]);
-            vR[i] = narrow<R>(v[i]);
-            BR[i] = narrow<R>(B_u[i]);
-            for (int j = 0; j < 3; j++) gR[i][j] = narrow<R>(g[i][j]);
-        }
-        R vR_d[3];
-        for (int i = 0; i < 3; i++) vR_d[i] = gR[i][0] * vR[0] + gR[i][1] * vR[1] + gR[i][2] * vR[2];
-        R ia = R(1.0) / alphaR;
-        R u0 = WR * ia;
-        R uu[3];
-        for (int i = 0; i < 3; i++) uu[i] = WR * (vR[i] - betaR[i] * ia);
-        R b0 = WR * (vR_d[0] * BR[0] + vR_d[1] * BR[1] + vR_d[2] * BR[2]) * ia;
-        R iW = R(1.0) / WR;
-        R bu[3];
-        for (int i = 0; i < 3; i++) bu[i] = (BR[i] + alphaR * b0 * uu[i]) * iW;
-        R beta_d[3];
-        for (int i = 0; i < 3; i++)
-            beta_d[i] = gR[i][0] * betaR[0] + gR[i][1] * betaR[1] + gR[i][2] * betaR[2];
-        R bb_ = beta_d[0] * betaR[0] + beta_d[1] * betaR[1] + beta_d[2] * betaR[2];
-        R g00 = -alphaR * alphaR + bb_;
-        R bd0 = g00 * b0 + beta_d[0] * bu[0] + beta_d[1] * bu[1] + beta_d[2] * bu[2];
-        R bd[3];
-        for (int i = 0; i < 3; i++)
-            bd[i] = beta_d[i] * b0 + gR[i][0] * bu[0] + gR[i][1] * bu[1] + gR[i][2] * bu[2];
-        R b2 = b0 * bd0 + bu[0] * bd[0] + bu[1] * bd[1] + bu[2] * bd[2];
-        const R rhoR = narrow<R>(rho), epsR = narrow<R>(eps), prR = narrow<R>(pr);
-        R pstar = prR + R(0.5) * b2;
-        R rhohs = rhoR * (R(1.0) + epsR) + prR + b2;   // rho h*
-        // conserved variables from the primitives (undensitized)
-        R Dp = rhoR * WR;
-        R Sp[3];
-        for (int j = 0; j < 3; j++) Sp[j] = rhohs * WR * WR * vR_d[j] - alphaR * b0 * bd[j];
-        // tau = rho h* W^2 - p* - alpha^2 b0^2 - D without its cancellation: with
-        // W^2 - 1 = W^2 v^2 and W - 1 = W^2 v^2 / (W + 1),
-        // tau = rho W (eps W + W^2 v^2 / (W + 1)) + p W^2 v^2 + b^2 (W^2 - 1/2) - alpha^2 b0^2
-        // (tau ~ 1e-3 D for a cold gas: the direct form loses 3 digits, all of FP32's margin)
-        const R Wv2 = WR * WR * (vR_d[0] * vR[0] + vR_d[1] * vR[1] + vR_d[2] * vR[2]);
-        const R taup = rhoR * WR * (epsR * WR + Wv2 / (WR + R(1.0))) + prR * Wv2 + b2 * (WR * WR - R(0.5)) -
-                       alphaR * alphaR * b0 * b0;
-        // ---- densitized fluxes [dir][var]
-        R vt[3];
-        for (int i = 0; i < 3; i++) vt[i] = alphaR * vR[i] - betaR[i];
-        for (int i = 0; i < 3; i++) {
-            // kept in FP32, as is T^{mu nu}: half the bytes, no conversion here and in the readers
-            R* F = reinterpret_cast<R*>(flux) + (long long)(i * 8) * P + p;
-            F[0 * P] = sqgR * (Dp * vt[i]);
-            for (int j = 0; j < 3; j++)
-                F[(1 + j) * P] = sqgR * (Sp[j] * vt[i] + (i == j ? alphaR * pstar : R(0.0)) -
-                                         alphaR * bd[j] * BR[i] * iW);
-            F[4 * P] = sqgR * (taup * vt[i] + alphaR * pstar * vR[i] - alphaR * alphaR * b0 * BR[i] * iW);
-            for (int k = 0; k < 3; k++) F[(5 + k) * P] = sqgR * (vt[i] * BR[k] - vt[k] * BR[i]);
-        }
-        // ---- T^{mu nu}
-        R ia2 = ia * ia;
-        R gu[4][4];
-        gu[0][0] = -ia2;
-        for (int i = 0; i < 3; i++) gu[0][i + 1] = gu[i + 1][0] = betaR[i] * ia2;
-        for (int i = 0; i < 3; i++)
-            for (int j = 0; j < 3; j++) gu[i + 1][j + 1] = narrow<R>(gi[i][j]) - betaR[i] * betaR[j] * ia2;
-        R u4[4] = {u0, uu[0], uu[1], uu[2]};
-        R b4[4] = {b0, bu[0], bu[1], bu[2]};
-        int n = 0;
-        for (int m = 0; m < 4; m++)
-            for (int k = m; k < 4; k++, n++)
-                reinterpret_cast<R*>(tmn)[n * P + p] = rhohs * u4[m] * u4[k] + pstar * gu[m][k] - b4[m] * b4[k];
-        }
         }
     }
     // warp-aggregated failure count
@@ -636,7 +636,6 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
 template <int MODE, bool HAM>
 __global__ void __launch_bounds__(128, 2) k_rhs(Dims d, PhysParams pp, const double* __restrict__ U0,
                                              const double* __restrict__ Us,
-                                             const double* __restrict__ prim,
                                              const float* __restrict__ flux,
                                              const float* __restrict__ tmn,
                                              const double* __restrict__ lam,
@@ -1553,14 +1552,13 @@ cudaError_t launch_con2prim(const Dims& d, const PhysParams& pp, const double* U
 }
 
 cudaError_t launch_rhs(const Dims& d, const PhysParams& pp, const double* U0, const double* Us,
-                       const double* prim, const double* flux, const double* tmn,
-                       const double* lam, const double* met, const void* d1, const void* d2,
-                       const void* divF, const void* divB, int deriv_fp32, const double* r_scale_dev,
-                       const double* dt_dev, RKCoef co, double* out, double* acc, cudaStream_t s,
+                       const double* flux, const double* tmn, const double* lam, const double* met,
+                       const void* d1, const void* d2, const void* divF, const void* divB, int deriv_fp32,
+                       const double* r_scale_dev, const double* dt_dev, RKCoef co, double* out, double* acc, cudaStream_t s,
                        double* ham, int div_parts) {
     int bs = 128;
     long long nb = (d.P + bs - 1) / bs;
-#define RHS_ARGS d, pp, U0, Us, prim, (const float*)flux, (const float*)tmn, lam, met, (const float*)d1, (const float*)d2, (const float*)divF, \
+#define RHS_ARGS d, pp, U0, Us, (const float*)flux, (const float*)tmn, lam, met, (const float*)d1, (const float*)d2, (const float*)divF, \
                     (const float*)divB, r_scale_dev, dt_dev, co, out, acc, ham
     if (deriv_fp32) {
         const unsigned g = (unsigned)nb;

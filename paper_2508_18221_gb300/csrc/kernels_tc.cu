@@ -365,7 +365,10 @@ static cudaError_t launch_w(const Dims& d, const TcJob* jobs, int njobs, const u
     // jobs walked by a CTA: about eight rounds of CTAs in all.  Fewer rounds leave a longer last
     // one, one job per CTA repeats the set-up (4.2M nodes, phi first derivatives: 620 us at two
     // rounds, 618 at four, 585 at eight, 658 at one job each)
-    const long long want = tc_ctas<TIn>(W) * 152LL * 8;
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const long long want = tc_ctas<TIn>(W) * (long long)nsm * 8;
     long long gy = (want + nb - 1) / nb;
     if (gy > njobs) gy = njobs;
     if (gy < 1) gy = 1;
