@@ -39,6 +39,17 @@ struct C2PScal {
     T v2max;        // r^2 / (1 + r^2), the largest admissible v^2
 };
 
+// With x = 1/(1 + mu bb), t = r^2 x^3 + mu x (S.B)^2/D^3 (1 + x + x^2) (r_par^2 + r_perp^2 x^3, split
+// along and across the field), the derivatives by mu are those of sums of positive terms,
+//   dv^2 = 2 mu t,  d(qbar - mu rbar^2) = -t,
+//   dg = h/W + mu t (1 + (Gamma - 1) (mu W - 1)),  below the floor h/W + mu t (2 - h mu W),
+// without the mu W where v^2 is clamped: FP32 keeps its accuracy of the slope however strong the
+// field (differentiated term by term, x^3 is the difference of terms larger by 1/x: with fields
+// of B^2 = 1e4 rho h and more the steps came out wrong, and W with them).
+__device__ __forceinline__ float slope_t(float x, float w, float u) {    // w = r^2 x, u = mu x rb2
+    return fmaf(w * x, x, u * fmaf(x, x, 1.f + x));
+}
+
 // g and its slope in FP32 alone: the search.  The cap on v^2 keeps W finite (at most 4,096: from
 // there on FP32 has no digits of 1 - v^2 left, and eps / W, all that W enters by, has no weight)
 struct Master32 {
@@ -46,43 +57,38 @@ struct Master32 {
 };
 __device__ __forceinline__ Master32 master32(float mu, const C2PScal<float>& c) {
     Master32 r;
-    const float x = __fdividef(1.f, fmaf(mu, c.bb, 1.f)), mx = mu * x, x2 = x * x;    // d(mu x) = x^2
-    const float dx = -c.bb * x2;
-    const float rb = c.r2 * x2 + mx * (1.f + x) * c.rb2;
-    const float drb = 2.f * c.r2 * x * dx + c.rb2 * (x2 * (1.f + x) + mx * dx);
-    const float m1 = mu * rb, dm1 = fmaf(mu, drb, rb);
-    const float qb = c.c0 - c.c1 * mx * mx, dqb = -2.f * c.c1 * mx * x2;
-    float v2 = mu * m1, dv2 = fmaf(mu, dm1, m1);
+    const float x = __fdividef(1.f, fmaf(mu, c.bb, 1.f)), mx = mu * x, w = c.r2 * x, u = mx * c.rb2;
+    const float m1 = mu * fmaf(w, x, fmaf(u, x, u)), mt = mu * slope_t(x, w, u);
+    const float qb = c.c0 - c.c1 * mx * mx;
+    float v2 = mu * m1;
     const float cap = fminf(c.v2max, 1.f - 0x1p-24f);
-    if (!(v2 <= cap)) { v2 = cap; dv2 = 0.f; }
-    const float om = 1.f - v2, W = rsqrtf(om), iW = om * W, diW = -0.5f * dv2 * W;
+    const bool clamped = !(v2 <= cap);
+    if (clamped) v2 = cap;
+    const float om = 1.f - v2, W = rsqrtf(om), iW = om * W, muW = clamped ? 0.f : mu * W;
     const float e = fmaf(W, 1.f + (qb - m1), -1.f);
-    float z, dz;
-    if (e >= c.eps_min) {
-        const float de = 0.5f * dv2 * W * W * W * (1.f + (qb - m1)) + W * (dqb - dm1);
-        z = fmaf(c.g1 * e, iW, 1.f + qb);
-        dz = dqb + c.g1 * (de * iW + e * diW);
-    } else {
-        const float h = 1.f + (1.f + c.g1) * c.eps_min;
-        z = fmaf(h, iW, m1);
-        dz = fmaf(h, diW, dm1);
-    }
+    const bool gas = e >= c.eps_min;
+    const float h = fmaf(1.f + c.g1, gas ? e : c.eps_min, 1.f);
+    const float z = gas ? fmaf(c.g1 * e, iW, 1.f + qb) : fmaf(h, iW, m1);
     r.g = fmaf(mu, z, -1.f);
-    r.dg = fmaf(mu, dz, z);
+    r.dg = fmaf(mt, gas ? fmaf(c.g1, muW - 1.f, 1.f) : fmaf(-h, muW, 2.f), h * iW);
     return r;
 }
 
 // g in FP64 and the quantities that the primitives are made of
 struct Master64 {
     double g, x, v2, m1, q2;     // v2 before the clamp to v2max; q2 = (mu x)^2
+    float w, u;                  // r^2 x, mu x rb2
     double W, e;                 // of the clamped v2; eps before its floor
 };
 __device__ __forceinline__ Master64 master64(double mu, const C2PScal<double>& c) {
     Master64 r;
     r.x = rcp64(fma(mu, c.bb, 1.0));
-    const double mx = mu * r.x, u = mx * c.rb2;
+    const double mx = mu * r.x;
+    const double w = c.r2 * r.x, u = mx * c.rb2;
+    r.w = d2f_rn(w);
+    r.u = d2f_rn(u);
     r.q2 = mx * mx;
-    r.m1 = mu * fma(r.x, c.r2 * r.x, fma(u, r.x, u));
+    r.m1 = mu * fma(r.x, w, fma(u, r.x, u));
     const double zb = fma(-c.c1, r.q2, 1.0 + c.c0);
     r.v2 = mu * r.m1;
     const double om = 1.0 - (r.v2 <= c.v2max ? r.v2 : c.v2max);
@@ -94,36 +100,25 @@ __device__ __forceinline__ Master64 master64(double mu, const C2PScal<double>& c
     return r;
 }
 
-// The slope of g where FP64 has evaluated it, and the derivatives that the final correction
-// needs, in FP32.  With d(1/W) = -W dv^2 / 2 and eps = W (1 + qbar - mu rbar^2) - 1,
-// d(eps / W) = W dv^2 / 2 + d(qbar - mu rbar^2): what FP32 cannot resolve is W (its relative error
-// is W^2 times that of v^2) and on which side of v2max and of eps_min the point lies (cold gas
-// has v^2 within about eps / W^2 of v2max).  Both come from the evaluation; the rest does not
-// wait for it (eps and W of FP32 enter g + 1 = mu z by eps / W alone).
+// The slope of g where FP64 has evaluated it, in FP32, from the evaluation's own quantities: W (what
+// FP32 cannot resolve of 1 - v^2, W enters with W^2 times its relative error), eps, and on which
+// side of v2max and of eps_min the point lies (cold gas has v^2 within about eps / W^2 of v2max).
 struct Slope32 {
-    float dg, dx, dv2, dqm, de;  // dv2, de: before the clamp and the floor
+    float dg, t, dv2, de;        // dv2, de: before the clamp and the floor
 };
 __device__ __forceinline__ Slope32 slope32(float mu, const Master64& f, const C2PScal<double>& c64,
                                            const C2PScal<float>& c) {
     Slope32 r;
-    const float x = __fdividef(1.f, fmaf(mu, c.bb, 1.f)), mx = mu * x, x2 = x * x;
-    r.dx = -c.bb * x2;
-    const float rb = c.r2 * x2 + mx * (1.f + x) * c.rb2;
-    const float drb = 2.f * c.r2 * x * r.dx + c.rb2 * (x2 * (1.f + x) + mx * r.dx);
-    const float m1 = mu * rb, dm1 = fmaf(mu, drb, rb);
-    const float qb = c.c0 - c.c1 * mx * mx, dqb = -2.f * c.c1 * mx * x2;
-    r.dqm = dqb - dm1;
-    r.dv2 = fmaf(mu, dm1, m1);
-    const float om = 1.f - fminf(mu * m1, fminf(c.v2max, 1.f - 0x1p-24f)), W1 = rsqrtf(om), iW1 = om * W1;
-    const float e1 = W1 * (1.f + (qb - m1)), h = 1.f + (1.f + c.g1) * c.eps_min;        // 1 + eps
+    r.t = slope_t(d2f_rn(f.x), f.w, f.u);
+    const float mt = mu * r.t;
+    r.dv2 = 2.f * mt;
     // W of the evaluation (1 <= W < 2^27), cut to FP32
     const float W = __uint_as_float(__funnelshift_l((uint32_t)__double2loint(f.W), (uint32_t)__double2hiint(f.W) - 0x38000000u, 3));
-    const float hdvW = f.v2 <= c64.v2max ? 0.5f * r.dv2 * W : 0.f;
-    r.de = W * fmaf(hdvW, e1, r.dqm);
+    const float muW = f.v2 <= c64.v2max ? mu * W : 0.f, e = d2f_rn(f.e);
+    r.de = W * r.t * fmaf(muW, 1.f + e, -1.f);
     const bool gas = f.e >= c64.eps_min;
-    const float z = gas ? fmaf(c.g1 * (e1 - 1.f), iW1, 1.f + qb) : fmaf(h, iW1, m1);
-    const float dz = gas ? fmaf(c.g1, hdvW + r.dqm, dqb) : fmaf(-h, hdvW, dm1);
-    r.dg = fmaf(mu, dz, z);
+    const float h = fmaf(1.f + c.g1, gas ? e : c.eps_min, 1.f);
+    r.dg = fmaf(mt, gas ? fmaf(c.g1, muW - 1.f, 1.f) : fmaf(-h, muW, 2.f), __fdividef(h, W));
     return r;
 }
 
@@ -176,7 +171,9 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
         if (f.g == 0.0) { conv = 1; break; }
         if (f.g < 0.0) lo = mu; else hi = mu;
         double mn = fma(-f.g, f2d(__fdividef(1.f, s.dg)), mu);
-        const bool newton = mn > lo && mn < hi;
+        // (late steps that do not shrink are rounding noise of g, which a strong field makes large:
+        // the bracket is halved instead)
+        const bool newton = mn > lo && mn < hi && !(it >= 24 && dprev > 0.f && fabsf(d2f_rn(mn - mu)) > 0.5f * dprev);
         if (!newton) {
             if (fabsf(d2f_rn(mn - mu)) <= 4e-15f * d2f_rn(mu)) { conv = 1; break; }
             mn = 0.5 * (lo + hi);
@@ -207,15 +204,14 @@ __device__ __forceinline__ int con2prim_root(const C2PScal<double>& c, int maxit
             f = master64(mu, c);
             qm = fma(-c.c1, f.q2, c.c0) - f.m1;
         } else {
-            f.x = fma(f2d(s.dx), delta, f.x);
+            const float x = d2f_rn(f.x);
+            f.x = fma(f2d(__fdividef(x * x - x, d2f_rn(mu))), delta, f.x);    // dx = -bb x^2
             f.v2 = fma(f2d(s.dv2), delta, f.v2);
-            qm = fma(f2d(s.dqm), delta, qm);
+            qm = fma(f2d(-s.t), delta, qm);
         }
     }
     const double v2 = f.v2 <= c.v2max ? f.v2 : c.v2max;
-    double om = 1.0 - v2;
-    if (__double2hiint(om) == 0) om = 0x1p-53;    // no root at r above 1e8: W stays finite
-    const double W = rsqrt64(om);
+    const double om = 1.0 - v2, W = rsqrt64(om);
     // eps without the cancellation of W (1 + qm) - 1: W - 1 = W^2 v^2 / (1 + W)
     const double e = fma(W, qm, v2 * W * W * rcp64(1.0 + W));
     *mu_o = mu;
@@ -465,6 +461,7 @@ __global__ void __launch_bounds__(128, 3) k_prep(Dims d, PhysParams pp, const do
             c.g1 = pp.gam - 1.0;
             c.eps_min = pp.eps_atm;
             c.v2max = c.r2 * rcp64(1.0 + c.r2);
+            if (__double2hiint(c.v2max) >= 0x3FF00000) c.v2max = 1.0 - 0x1p-53;    // r above 1e8: W stays finite
             // guess mu = 1/(h W) from the stored primitives
             const float guess = __fdividef(1.f, (1.f + (float)pp.gam * d2f_rn(prim[4 * P + p])) * d2f_rn(prim[6 * P + p]));
             double mu, x;
