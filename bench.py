@@ -398,7 +398,7 @@ def run_reference(args):
 # FP64 work.  The primitive-recovery count is taken inside the time stepping (Newton
 # started from the previous stage's primitives); k_prep<PREP_F32> (mixed modes) forms the
 # fluxes and T^{mu nu} in FP32, so only its metric and primitive recovery count.
-FP64_FLOPS_PER_NODE = {"k_rhs64": 1656.0, "k_prep<PREP_F64>": 509.0, "k_prep<PREP_F32>": 322.0}
+FP64_FLOPS_PER_NODE = {"k_rhs64": 1656.0, "k_prep<PREP_F64>": 508.0, "k_prep<PREP_F32>": 322.0}
 # Nominal FP64 peak of GB300 from its unit counts and clock: 152 SMs x 2 DFMA/clk x 2 flop
 # x 2.07 GHz (a probe of dependent DFMA chains on all SMs measured 1.198 TFLOP/s).
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
@@ -406,7 +406,8 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # T^{mu nu}, first/second derivatives and flux divergence (FP32) in, stage output out
 RHS32_BYTES_PER_NODE = 8 * (32 + 32 + 9) + 4 * (10 + 63 + 66 + 8) + 8 * 32
 # a grid's contractions run on the integer units (k_contract_small) up to these bounds on
-# nodes x (N_r + N_theta + N_phi) and nodes x max(N)^2
+# nodes x (N_r + N_theta + N_phi) and nodes x max(N)^2: FXS_MAX_WORK and FXS_MAX_SQUARE of
+# csrc/api.cu, here for the kernels' names only
 SMALL_WORK, SMALL_SQUARE = 3000000, 40000000
 
 

@@ -395,11 +395,12 @@ __device__ __forceinline__ void fluxes64(long long p, long long P, double alpha,
 
 // What a launch computes: the primitives alone, or also the fluxes and matter terms in FP64
 // or FP32.  Bound by the FP64 pipe (87 % busy): 346 FP64 instructions per node against 707
-// in FP64, so the launch inside the stepping of 393,216 nodes went from 545 to 283 us (ncu),
-// the FP32 form from 340 to 234 us, the recovery of a newly loaded state (grmhd_con2prim,
-// whole call) from 807 to 247 us.  Three blocks per SM (168
-// registers): per step of three launches 843 us in FP64 and 575 us in FP32, against 865 and 580
-// with four (128 registers, spills of 120 B) and 972 and 634 with five.
+// in FP64, so the launch inside the stepping of 393,216 nodes went from 545 to 281 us (ncu),
+// the FP32 form from 384 to 198 us, the recovery of a newly loaded state (grmhd_con2prim,
+// whole call) from 807 to 247 us.  Three blocks per SM (168 registers): per step of three
+// launches 843 us in FP64 and 586 us in FP32.  Measured when that was chosen, with a slope of a
+// few instructions less: 843 and 575 with three, 865 and 580 with four (128 registers, spills of
+// 120 B), 972 and 634 with five.
 enum { PREP_PRIM = 0, PREP_F64 = 1, PREP_F32 = 2 };
 
 template <int WHAT>
